@@ -408,6 +408,14 @@ static void mass_enqueue(const fe_hierarchy* h, const Level& L, const double* x,
     launch_mass_df(L, x, y, s);
 }
 
+// Whether operator applications of this precision on level l run in flux form
+// (fe_flux.cu): FP32, and FP64 in the default mode, on levels that have it.
+static bool use_flux(const fe_hierarchy* h, int l, int dtype) {
+  const Level& L = h->L[l];
+  if (L.flux == FLUX_NONE) return false;
+  return dtype == FE_F32 || (dtype == FE_F64 && h->f64_mode == FE_F64_DOUBLE_FLOAT);
+}
+
 // Whether the FP64 operator on level l is the per-tet float-pair kernel that can
 // gather pre-split dofs (P1 in FE_F64_DOUBLE_FLOAT_TET mode, P2 in the default
 // mode), so that the vector kernels producing its inputs write float pairs too.
@@ -415,7 +423,7 @@ static void mass_enqueue(const fe_hierarchy* h, const Level& L, const double* x,
 // comparison); the fused and patch smoothers update x without pairs.
 static bool presplit(const fe_hierarchy* h, int l) {
   const Level& L = h->L[l];
-  return h->f64_mode == FE_F64_DOUBLE_FLOAT && L.deg == 2 && L.xs64.p && !h->fuse_smoother &&
+  return h->f64_mode == FE_F64_DOUBLE_FLOAT && L.deg == 2 && L.xs64.p && !h->fuse_smoother && !use_flux(h, l, FE_F64) &&
          !(h->smoother == FE_SMOOTHER_PATCH && h->deg >= 2 && l >= 1 && L.pdof.p);
 }
 
@@ -433,6 +441,13 @@ void apply_enqueue(const fe_hierarchy* h, int level, const void* x, void* y, int
       apply_bf16_enqueue(L, (const float*)x, (float*)y, s);
     else
       FE_FAIL(FE_ERR_ARG, "unknown dtype");
+    return;
+  }
+  if (use_flux(h, level, dtype)) {
+    if (dtype == FE_F64)
+      launch_flux_apply<double>(L, (const double*)x, (double*)y, s);
+    else
+      launch_flux_apply<float>(L, (const float*)x, (float*)y, s);
     return;
   }
   // measured on GB300 (P*64^3): P1 per cube 0.025 ms vs per tet 0.041 ms; P2 per tet 0.139 ms vs per cube
@@ -511,6 +526,38 @@ static void smooth_enqueue(fe_hierarchy* h, int l, const T* b, T* x, T* y, T* d,
         launch_cheb_pc<T>(L.n, z, x, d, rn * rho, 2.0 * rn / delta, false, !last, s);
         rho = rn;
       }
+    }
+    return;
+  }
+  if (use_flux(h, l, dtype) && !(h->fuse_smoother && L.cnt_tet.p)) {
+    // one launch per step, from one vector to another: x and y in turn, ending in x
+    int k = 0;
+    double c1 = 0.0, c2 = 1.0 / theta;
+    auto next = [&] {
+      const double rn = 1.0 / (2.0 * sigma - rho);
+      c1 = rn * rho;
+      c2 = 2.0 * rn / delta;
+      rho = rn;
+      ++k;
+    };
+    T* cur = x;
+    const T* din = d;
+    if (x_zero) {  // the first direction is the iterate itself
+      if ((steps - 1) & 1) cur = y;
+      launch_cheb_step<T>(L.n, b, nullptr, lv_dinv<T>(L), cur, d, c1, c2, true, s, false);
+      din = cur;
+      next();
+    } else if (steps & 1) {  // an odd number of steps from x to x: the first in place
+      apply_enqueue(h, l, x, y, dtype, s);
+      launch_cheb_step<T>(L.n, b, y, lv_dinv<T>(L), x, d, c1, c2, false, s, steps > 1);
+      next();
+    }
+    while (k < steps) {
+      T* to = cur == x ? y : x;
+      launch_flux_cheb<T>(L, b, cur, to, din, k + 1 < steps ? d : nullptr, c1, c2, s);
+      cur = to;
+      din = d;
+      next();
     }
     return;
   }
@@ -968,7 +1015,7 @@ static PcgResult pcg_low(fe_hierarchy* h, int dtype, const fe_solver_opts& o, cu
   while (res.it < o.inner_max_it) {
     {
       PhaseScope ps(FE_PHASE_APPLY, top, s);
-      launch_apply32(F, p, q, s);
+      apply_enqueue(h, top, p, q, FE_F32, s);
     }
     ++res.applies;
     {
@@ -1082,8 +1129,8 @@ static void set_coefficient_impl(fe_hierarchy* h, const double* kappa, cudaStrea
   for (int l = 0; l < h->nlev; ++l) {
     launch_geometry(h->L[l], s);
     launch_split_geometry(h->L[l], s);
-    launch_uniform_geometry(h->L[l], h->cs.flag, s);
-    if (h->geometry_form == FE_GEOMETRY_PER_CELL) h->L[l].uniform = 0;
+    launch_uniform_geometry(h->L[l], h->geometry_form == FE_GEOMETRY_PER_CELL, h->cs.flag, s);
+    launch_flux_setup(h->L[l], s);
     launch_diag(h->L[l], h->tmp, s);
   }
   if (h->smoother == FE_SMOOTHER_PATCH && h->deg >= 2)
@@ -1447,8 +1494,8 @@ int fe_set_geometry_form(fe_hierarchy* h, int form) {
   CUDA_CHECK(cudaDeviceSynchronize());
   h->geometry_form = form;
   for (int l = 0; l < h->nlev; ++l) {
-    launch_uniform_geometry(h->L[l], h->cs.flag, nullptr);
-    if (form == FE_GEOMETRY_PER_CELL) h->L[l].uniform = 0;
+    launch_uniform_geometry(h->L[l], form == FE_GEOMETRY_PER_CELL, h->cs.flag, nullptr);
+    launch_flux_setup(h->L[l], nullptr);
   }
   invalidate_graphs(h);
   API_END

@@ -1,0 +1,761 @@
+// Operator kernels on Kuhn meshes that form each row of A x in one thread, from
+// the lattice neighbours of its dof: no scatter, no dof maps, no zero-fill, and
+// the Chebyshev update of the row in the same launch.
+//
+// Every Kuhn tet is a path of three axis-parallel edges and its geometric factor
+// is c M (one c = kappa h / w per tet, see Level), which is diagonal in the
+// directions of that path: the bilinear form of Section 2, Eq. 4 on a tet is c
+// times the integral of (du/dx)^2 + (du/dy)^2 + (du/dz)^2, each axis taken along
+// the tet's own edge of that axis.
+//
+// P1 (any coefficient): du/da is the difference along that edge, so A is the
+// graph Laplacian of the axis edges with the weight of an edge the sum of c over
+// its (up to six) tets: seven entries per row.
+//
+// P2 with one coefficient on the level: the rows are eight constant stencils of
+// small integers times 8 c, one per parity class of the dof lattice.
+//
+// x is read as 0 on and outside the boundary.  An interior row only couples to
+// points of tets that exist, so edges of the domain need no special case.
+#include <algorithm>
+#include <cmath>
+#include <type_traits>
+#include <utility>
+
+#include "fe_internal.cuh"
+#include "fe_kuhn.h"
+
+namespace {
+
+inline int ceil_div(long long a, int b) { return (int)((a + b - 1) / b); }
+
+// What a kernel does with its row y_i of A x.
+enum Epilogue { EPI_APPLY = 0, EPI_CHEB = 1 };
+
+template <typename T>
+struct Rows {
+  const T* x;     // the operator's input (also the iterate that a Chebyshev step updates)
+  T* out;         // APPLY: y; CHEB: the new iterate (another vector than x)
+  const T* b;     // CHEB: right-hand side
+  const T* din;   // CHEB, c1 != 0: the previous direction
+  T* dout;        // CHEB: the new direction (null: not stored)
+  const T* dinv;  // CHEB on P1 with a coefficient per cell: inverse diagonal
+  T c1, c2;
+  T wd[8];        // CHEB with one coefficient: c2 / diagonal per parity code (P1: wd[0])
+};
+
+// The vectors that a row needs besides y, loaded before the row is formed.
+template <int EPI, typename T>
+struct RowIn {
+  T b = T(0), d = T(0), x = T(0);
+  __device__ __forceinline__ RowIn(const Rows<T>& R, int i) {
+    if constexpr (EPI == EPI_CHEB) {
+      b = __ldg(R.b + i);
+      if (R.c1 != T(0)) d = R.din[i];
+      x = __ldg(R.x + i);
+    }
+  }
+};
+
+__device__ __forceinline__ double fma_t(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float fma_t(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+
+// Row y_i = s v; Chebyshev: d = c1 d + w (b - y), x += d with w = c2 / A_ii.
+// FP64 operations are scarce (2 per clock and SM), so the scaling of y and the
+// diagonal are folded: 4 of them per row with a previous direction.
+template <int EPI, typename T>
+__device__ __forceinline__ void finish_row(const Rows<T>& R, const RowIn<EPI, T>& in, int i, T v, T s, T w) {
+  if constexpr (EPI == EPI_APPLY) {
+    R.out[i] = v * s;
+  } else {
+    const T r = fma_t(-v, s, in.b);
+    const T dn = R.c1 != T(0) ? fma_t(w, r, R.c1 * in.d) : w * r;
+    if (R.dout) R.dout[i] = dn;
+    R.out[i] = in.x + dn;
+  }
+}
+// A Dirichlet row: y = x.
+template <int EPI, typename T>
+__device__ __forceinline__ void identity_row(const Rows<T>& R, int i) {
+  const RowIn<EPI, T> in(R, i);
+  finish_row<EPI>(R, in, i, R.x[i], T(1), R.c2);
+}
+
+// ------------------------------------------------------------------- P1 ---
+// One thread per vertex: y = D x - sum over the six axis edges of w x, with D
+// the diagonal and w the weight of the edge (stored at its lower end; CONST:
+// one coefficient, w = 6 c and D = 36 c).  FP64 issues 2 operations per clock
+// and SM, so the row is kept at 7 of them (differences would take 12): bound by
+// the FP64 pipe with a coefficient per edge, else by memory.
+constexpr int kP1Block = 256;
+
+template <typename T, bool CONST, int EPI>
+__global__ void __launch_bounds__(kP1Block) k_flux1(int N, int n, const T* __restrict__ w, T c, Rows<T> R) {
+  const int i = blockIdx.x * kP1Block + threadIdx.x;
+  if (i >= n) return;
+  const int n1 = N + 1, sz = n1 * n1;
+  const int X = i % n1, q = i / n1, Y = q % n1, Z = q / n1;
+  if (X == 0 || Y == 0 || Z == 0 || X == N || Y == N || Z == N) {
+    identity_row<EPI>(R, i);
+    return;
+  }
+  const RowIn<EPI, T> in(R, i);
+  const T* __restrict__ x = R.x;
+  const T xi = x[i];
+  // a neighbour on the boundary counts as 0
+  const T xl = X > 1 ? x[i - 1] : T(0), xr = X < N - 1 ? x[i + 1] : T(0);
+  const T yl = Y > 1 ? x[i - n1] : T(0), yr = Y < N - 1 ? x[i + n1] : T(0);
+  const T zl = Z > 1 ? x[i - sz] : T(0), zr = Z < N - 1 ? x[i + sz] : T(0);
+  if constexpr (CONST) {
+    finish_row<EPI>(R, in, i, fma_t(T(6), xi, -(((xl + xr) + (yl + yr)) + (zl + zr))), c, R.wd[0]);
+  } else {
+    const T* wx = w;
+    const T* wy = w + n;
+    const T* wz = w + 2 * (size_t)n;
+    T y = w[3 * (size_t)n + i] * xi;
+    y = fma_t(-wx[i - 1], xl, y);
+    y = fma_t(-wx[i], xr, y);
+    y = fma_t(-wy[i - n1], yl, y);
+    y = fma_t(-wy[i], yr, y);
+    y = fma_t(-wz[i - sz], zl, y);
+    y = fma_t(-wz[i], zr, y);
+    finish_row<EPI>(R, in, i, y, T(1), EPI == EPI_CHEB ? R.c2 * R.dinv[i] : T(0));
+  }
+}
+
+// Edge weights from the coefficients c of the cells: the edge of axis a that
+// starts at vertex v belongs to a ring of six tets; ring tet f is Kuhn type
+// ring_type of the cube at v + ring_b(f) e_b + ring_c(f) e_c (b < c the other axes).
+__host__ __device__ constexpr int ring_type(int axis, int f) {
+  constexpr int t[3][6] = {{0, 1, 2, 5, 3, 4}, {2, 3, 0, 4, 1, 5}, {4, 5, 1, 2, 0, 3}};
+  return t[axis][f];
+}
+__host__ __device__ constexpr int ring_b(int f) { return f >= 2 && f <= 4 ? -1 : 0; }  // offset along b
+__host__ __device__ constexpr int ring_c(int f) { return f >= 3 ? -1 : 0; }            // offset along c
+
+__global__ void k_edge_weights(int N, int n, const double* __restrict__ geo22, double* __restrict__ w64,
+                               float* __restrict__ w32) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int n1 = N + 1;
+  const int p[3] = {i % n1, (i / n1) % n1, i / (n1 * n1)};
+  // weight of the edge of `axis` starting at vertex v
+  auto weight = [&](int axis, int vx, int vy, int vz) {
+    const int v[3] = {vx, vy, vz};
+    if (v[axis] < 0 || v[axis] >= N) return 0.0;
+    const int b = axis == 0 ? 1 : 0, c = axis == 2 ? 1 : 2;
+    double s = 0.0;
+#pragma unroll
+    for (int f = 0; f < 6; ++f) {
+      int q[3];
+      q[axis] = v[axis];
+      q[b] = v[b] + ring_b(f);
+      q[c] = v[c] + ring_c(f);
+      if (q[b] < 0 || q[b] >= N || q[c] < 0 || q[c] >= N) continue;
+      s += geo22[6 * (q[0] + (size_t)N * (q[1] + (size_t)N * q[2])) + ring_type(axis, f)];
+    }
+    return s;
+  };
+  const double wx = weight(0, p[0], p[1], p[2]), wy = weight(1, p[0], p[1], p[2]), wz = weight(2, p[0], p[1], p[2]);
+  const double dg = wx + wy + wz + weight(0, p[0] - 1, p[1], p[2]) + weight(1, p[0], p[1] - 1, p[2]) +
+                    weight(2, p[0], p[1], p[2] - 1);
+  const size_t m = n;
+  w64[i] = wx;
+  w64[m + i] = wy;
+  w64[2 * m + i] = wz;
+  w64[3 * m + i] = dg;
+  w32[i] = (float)wx;
+  w32[m + i] = (float)wy;
+  w32[2 * m + i] = (float)wz;
+  w32[3 * m + i] = (float)dg;
+}
+
+// FP64 values as 64-bit integers of a common scale: with E the largest biased
+// exponent of a tile, |x| is cut into windows of TB + 1 bits below 2^(E - 1022);
+// window `pass` of x is returned with x's sign.  Sums of such integers wrap
+// modulo 2^64 and are exact as long as the final row fits.
+template <int TB>
+__device__ __forceinline__ long long fixed_window(unsigned int hi, unsigned int lo, int E, int pass) {
+  const int e = (int)((hi >> 20) & 0x7FFu);
+  if (e == 0 || e == 0x7FF) return 0;  // zero, subnormal (flushed), or not finite (handled by the caller)
+  const unsigned long long m = ((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
+  const unsigned long long M = m << (TB - 52);
+  const int r = (E - e) - pass * (TB + 1);
+  unsigned long long w;
+  if (r >= 0)
+    w = r < 64 ? M >> r : 0ull;
+  else
+    w = r > -64 ? (M << -r) & ((1ull << (TB + 1)) - 1) : 0ull;
+  return (hi >> 31) ? -(long long)w : (long long)w;
+}
+
+constexpr int kTop = 59;    // top bit of a staged value: |x| < 2^60 units
+constexpr int kRange = 15;  // bits by which a cell may lie below its tile's largest value in one pass
+
+__device__ __forceinline__ double pow2(int e) {  // 2^e, -1022 <= e <= 1023
+  return __hiloint2double((e + 1023) << 20, 0);
+}
+
+// ------------------------------------------- P2, one coefficient: stencils ---
+// With one c on the level the rows of A are eight constant stencils of 19 to 51
+// small integers times 8 c, one per parity
+// class of the dof lattice; 23 entries per row on average, all in 58 lattice
+// values around a vertex cell.  A block stages the values of TX x TY x KZ
+// vertex cells and one layer around them in shared memory (asynchronous copies,
+// all in flight at once) and each thread forms the eight rows of a cell.
+//
+// FP64: the staged values become two 30-bit integers hi 2^30 + lo of the tile's
+// common scale (its largest exponent), a value and its mirror image (every
+// stencil is symmetric) are added in 32 bits, the coefficient times that sum in
+// 64 bits: every sum is exact (rows of |K| / 8 sum to at most 216 < 2^8), and a
+// row is rounded once, by one int64 -> FP64 conversion and one multiplication.
+// The FP64 pipe (2 operations per clock and SM) would need 23 operations per row,
+// the element-by-element form on the FP32 pipes 453 instructions per dof, this
+// form 180.  What the integers cut off is below 2^-59 of the tile's largest
+// value; the cells that lie more than kRange bits below it are formed again from
+// the windows of the next lower bits, and the parts are added in FP64.
+struct Pair32 {  // hi 2^30 + lo
+  int hi, lo;
+};
+__device__ __forceinline__ Pair32 operator+(Pair32 a, Pair32 b) { return {a.hi + b.hi, a.lo + b.lo}; }
+
+template <typename V>
+struct RowSum;
+template <>
+struct RowSum<float> {
+  float s = 0.0f;
+  template <typename... A>
+  __device__ __forceinline__ void add(int k, A... v) {
+    s = __fmaf_rn((float)k, (v + ...), s);
+  }
+};
+template <>
+struct RowSum<double> {
+  double s = 0.0;
+  template <typename... A>
+  __device__ __forceinline__ void add(int k, A... v) {
+    s = __fma_rn((double)k, (v + ...), s);
+  }
+};
+template <>
+struct RowSum<Pair32> {
+  long long hi = 0, lo = 0;
+  template <typename... A>
+  __device__ __forceinline__ void add(int k, A... v) {  // sums of at most two staged values
+    ((hi += (long long)k * v.hi, lo += (long long)k * v.lo), ...);
+  }
+};
+
+// The row of the lattice point of parity code CODE in units of 8 c; at(x, y, z):
+// the value at that offset from the vertex of its cell, components in [-2, 2].
+template <int CODE, typename V, typename At>
+__device__ __forceinline__ RowSum<V> stencil_row(At at) {
+  constexpr int X = CODE & 1, Y = (CODE >> 1) & 1, Z = CODE >> 2;
+  RowSum<V> r;
+  auto p = [&](int x, int y, int z) -> V { return at(X + x, Y + y, Z + z); };
+  auto s = [&](int x, int y, int z) -> V { return p(x, y, z) + p(-x, -y, -z); };
+  if constexpr (CODE == 0) {  // a vertex
+    r.add(54, p(0, 0, 0));
+    r.add(-14, s(1, 0, 0), s(0, 1, 0), s(0, 0, 1));
+    r.add(3, s(2, 0, 0), s(0, 2, 0), s(0, 0, 2));
+    r.add(-3, s(1, 1, 1), s(1, 1, 0), s(1, 0, 1), s(0, 1, 1));
+    r.add(2, s(1, -1, 0), s(1, 0, -1), s(0, 1, -1));
+    r.add(1, s(2, 1, 1), s(1, 2, 1), s(1, 1, 2), s(2, 1, 0), s(2, 0, 1), s(1, 2, 0), s(0, 2, 1), s(1, 0, 2),
+          s(0, 1, 2), s(1, 1, -1), s(1, -1, 1), s(-1, 1, 1));
+  } else if constexpr (CODE == 7) {  // on the cube's main diagonal
+    r.add(48, p(0, 0, 0));
+    r.add(-4, s(1, 0, 0), s(0, 1, 0), s(0, 0, 1), s(1, -1, 0), s(1, 0, -1), s(0, 1, -1));
+    r.add(-3, s(1, 1, 1));
+    r.add(1, s(1, 1, -1), s(1, -1, 1), s(-1, 1, 1));
+  } else if constexpr (X + Y + Z == 1) {  // on an axis edge a
+    auto t = [&](int a, int b, int c) -> V {
+      if constexpr (CODE == 1) return s(a, b, c);
+      if constexpr (CODE == 2) return s(b, a, c);
+      if constexpr (CODE == 4) return s(b, c, a);
+    };
+    r.add(56, p(0, 0, 0));
+    r.add(-14, t(1, 0, 0));
+    r.add(-6, t(0, 1, 0), t(0, 0, 1));
+    r.add(-4, t(0, 1, -1));
+    r.add(4, t(1, 1, 1));
+    r.add(-2, t(1, 1, 2), t(1, 2, 1));
+    r.add(1, t(1, 0, 2), t(1, 2, 0));
+  } else {  // on a face diagonal, n normal to the face
+    auto t = [&](int a, int b, int n) -> V {
+      if constexpr (CODE == 3) return s(a, b, n);
+      if constexpr (CODE == 5) return s(a, n, b);
+      if constexpr (CODE == 6) return s(n, a, b);
+    };
+    r.add(48, p(0, 0, 0));
+    r.add(-6, t(1, 0, 0), t(0, 1, 0), t(1, 0, 1), t(0, 1, 1));
+    r.add(-4, t(0, 0, 1));
+    r.add(4, t(1, 1, 1));
+    r.add(-3, t(1, 1, 0));
+    r.add(2, t(1, -1, 0));
+    r.add(1, t(1, 1, 2));
+  }
+  return r;
+}
+
+// The coefficient (in units of 8 c) of the lattice point at offset (ox, oy, oz)
+// from the vertex of a cell in the row of the cell's point of parity code CODE:
+// the integer element matrices of the tets that hold both, summed.
+__host__ __device__ constexpr int stencil_coef(int code, int ox, int oy, int oz) {
+  const int p[3] = {code & 1, (code >> 1) & 1, code >> 2}, o[3] = {ox, oy, oz};
+  int sum = 0;
+  for (int cube = 0; cube < 8; ++cube) {
+    int a[3] = {0, 0, 0}, b[3] = {0, 0, 0};  // both points in the cube's lattice [0, 2]^3
+    bool in = true;
+    for (int d = 0; d < 3; ++d) {
+      const int c = (cube >> d & 1) ? -2 : 0;
+      a[d] = p[d] - c;
+      b[d] = o[d] - c;
+      in = in && a[d] <= 2 && b[d] >= 0 && b[d] <= 2;
+    }
+    if (!in) continue;
+    const int la = a[0] + 3 * a[1] + 9 * a[2], lb = b[0] + 3 * b[1] + 9 * b[2];
+    for (int t = 0; t < 6; ++t) {
+      int i = -1, j = -1;
+      for (int n = 0; n < 10; ++n) {
+        if (cube_local(2, t, n) == la) i = n;
+        if (cube_local(2, t, n) == lb) j = n;
+      }
+      if (i >= 0 && j >= 0) sum += fe_kuhn::kuhn_p2_k(i, j);
+    }
+  }
+  return sum / 2;
+}
+// the eight coefficients of one offset, packed for a compile-time test that any is not zero
+__host__ __device__ constexpr bool stencil_uses(int ox, int oy, int oz) {
+  for (int code = 0; code < 8; ++code)
+    if (stencil_coef(code, ox, oy, oz) != 0) return true;
+  return false;
+}
+static_assert(stencil_coef(0, 0, 0, 0) == 54 && stencil_coef(3, 1, 1, 0) == 48 && stencil_coef(1, 1, 0, 0) == 56 && stencil_coef(7, 1, 1, 1) == 48 &&
+                  stencil_coef(0, 2, 1, 1) == 1 && stencil_coef(3, 0, 0, -1) == 4,
+              "P2 Kuhn stencils");
+
+// All eight rows of a cell, one lattice value at a time: each is loaded once and
+// goes into every row that couples to it.
+template <int I, typename V, typename At>
+__device__ __forceinline__ void stencil_point(RowSum<V> (&r)[8], At& at) {
+  constexpr int x = I % 5 - 2, y = I / 5 % 5 - 2, z = I / 25 - 2;
+  if constexpr (stencil_uses(x, y, z)) {
+    const V v = at(x, y, z);
+    auto one = [&](auto code_) {
+      constexpr int code = decltype(code_)::value;
+      constexpr int k = stencil_coef(code, x, y, z);
+      if constexpr (k != 0) r[code].add(k, v);
+    };
+    one(std::integral_constant<int, 0>{});
+    one(std::integral_constant<int, 1>{});
+    one(std::integral_constant<int, 2>{});
+    one(std::integral_constant<int, 3>{});
+    one(std::integral_constant<int, 4>{});
+    one(std::integral_constant<int, 5>{});
+    one(std::integral_constant<int, 6>{});
+    one(std::integral_constant<int, 7>{});
+  }
+}
+// The cell's own points, whose coefficients (the diagonals among them) are the
+// largest, come last, so that few sums are rounded at their size.
+template <typename V, typename At, int... I>
+__device__ __forceinline__ void stencil_rows(RowSum<V> (&r)[8], At at, std::integer_sequence<int, I...>) {
+  constexpr auto own = [](int i) { return i % 5 - 2 >> 1 == 0 && (i / 5 % 5 - 2) >> 1 == 0 && (i / 25 - 2) >> 1 == 0; };
+  auto point = [&](auto i, auto want) {
+    if constexpr (own(decltype(i)::value) == decltype(want)::value) stencil_point<decltype(i)::value>(r, at);
+  };
+  (point(std::integral_constant<int, I>{}, std::false_type{}), ...);
+  (point(std::integral_constant<int, I>{}, std::true_type{}), ...);
+}
+
+// x as hi 2^30 + lo of the scale E, both with the sign of x (the first window of
+// fixed_window in 30-bit halves).  A shift beyond 63 (zeros, far smaller values
+// and, with e > E, values that are not finite) gives 0; needs E >= 64.
+__device__ __forceinline__ Pair32 fixed_pair(double x, int E) {
+  const unsigned int xh = (unsigned int)__double2hiint(x), xl = (unsigned int)__double2loint(x);
+  const unsigned int r = min((unsigned int)(E - (int)((xh >> 20) & 0x7FFu)), 63u);
+  const unsigned long long m = ((unsigned long long)((xh & 0xFFFFFu) | 0x100000u) << 32) | xl;
+  const unsigned long long w = (m << (kTop - 52)) >> r;
+  const int sg = 1 | ((int)xh >> 31);
+  return {sg * (int)(w >> 30), sg * (int)((unsigned int)w & 0x3FFFFFFFu)};
+}
+// any window, any E
+__device__ __noinline__ Pair32 fixed_pair_window(double x, int E, int pass) {
+  const unsigned int xh = (unsigned int)__double2hiint(x), xl = (unsigned int)__double2loint(x);
+  const long long w = fixed_window<kTop>(xh & 0x7FFFFFFFu, xl, E, pass);
+  const int sg = 1 | ((int)xh >> 31);
+  return {sg * (int)(w >> 30), sg * (int)(w & 0x3FFFFFFF)};
+}
+
+template <int BYTES>
+__device__ __forceinline__ void cp_async_or_zero(void* smem, const void* gmem, bool valid) {
+  const unsigned int sa = (unsigned int)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(sa), "l"(gmem), "n"(BYTES),
+               "r"(valid ? BYTES : 0)
+               : "memory");
+}
+
+template <int TX_, int TY_, int KZ_, int THREADS_, int BLOCKS_>
+struct TileShape {  // BLOCKS: resident blocks per SM that the registers are limited for
+  static constexpr int blocks = BLOCKS_;
+  static constexpr int TX = TX_, TY = TY_, KZ = KZ_, threads = THREADS_;
+  static constexpr int W = TX + 2, H = TY + 2, D = KZ + 2, cells = W * H * D, own = TX * TY * KZ;
+  template <typename T>
+  static constexpr size_t smem() {
+    return (size_t)cells * (8 * sizeof(T) + (sizeof(T) == 8 ? 2 : 0));
+  }
+};
+
+struct Lattice2 {  // the P2 numbering per parity code px + 2 py + 4 pz: first dof and strides of its class
+  int N, off[8], sy[8], sz[8];
+};
+
+template <typename T, int EPI, typename S>
+__global__ void __launch_bounds__(S::threads, S::blocks)
+    k_stencil2(Lattice2 G, double scale, Rows<T> R, int nb, const int* __restrict__ bnd) {
+  constexpr bool FIX = sizeof(T) == 8;
+  using V = typename std::conditional<FIX, Pair32, float>::type;
+  static_assert(sizeof(V) == sizeof(T), "staged in place");
+  extern __shared__ __align__(16) unsigned char smem[];
+  T* raw = reinterpret_cast<T*>(smem);  // [8][cells]
+  V* xs = reinterpret_cast<V*>(smem);
+  unsigned short* se = reinterpret_cast<unsigned short*>(smem + (size_t)S::cells * 8 * sizeof(T));  // exponents
+  __shared__ int s_max, s_min, s_bad;
+  const int tid = threadIdx.x, N = G.N;
+  const int ntx = (N + S::TX - 1) / S::TX, nty = (N + S::TY - 1) / S::TY;
+  const int i0 = (blockIdx.x % ntx) * S::TX, j0 = (blockIdx.x / ntx) % nty * S::TY, k0 = blockIdx.x / (ntx * nty) * S::KZ;
+  if constexpr (FIX)
+    if (tid == 0) {
+      s_max = 1;
+      s_min = 0x7FF;
+      s_bad = 0;
+    }
+  // the values of staged cell s: f(code, dof, whether it is interior)
+  auto for_points = [&](int s, auto&& f) {
+    const int ci = i0 - 1 + s % S::W, cj = j0 - 1 + (s / S::W) % S::H, ck = k0 - 1 + s / (S::W * S::H);
+    // even coordinates are interior for 0 < c < N, odd ones for 0 <= c < N
+    const bool below = ci < N && cj < N && ck < N;
+    const bool xe = ci > 0, xo = ci >= 0, ye = cj > 0 && below, yo = cj >= 0 && below, ze = ck > 0, zo = ck >= 0;
+#pragma unroll
+    for (int code = 0; code < 8; ++code)
+      f(code, G.off[code] + ci + G.sy[code] * cj + G.sz[code] * ck,
+        (code & 1 ? xo : xe) && (code & 2 ? yo : ye) && (code & 4 ? zo : ze));
+  };
+  for (int s = tid; s < S::cells; s += S::threads)
+    for_points(s, [&](int code, int i, bool in) {
+      cp_async_or_zero<sizeof(T)>(raw + code * S::cells + s, R.x + (in ? i : 0), in);
+    });
+  cp_async_commit();
+  for (int i = blockIdx.x * S::threads + tid; i < nb; i += gridDim.x * S::threads) {  // Dirichlet rows: identity
+    identity_row<EPI>(R, bnd[i]);
+  }
+  cp_async_wait_all();
+  __syncthreads();
+  int E = 0, passes = 1;
+  bool bad = false;
+  auto exponent = [&](int c) {  // of own cell c (the rows of a cell all couple to most of its eight points)
+    return (int)se[c % S::TX + 1 + S::W * ((c / S::TX) % S::TY + 1 + S::H * (c / (S::TX * S::TY) + 1))];
+  };
+  // windows that a cell of exponent e takes until what is left is below 2^(kRange - kTop) of its values
+  auto windows = [&](int e) { return E - e > kRange ? 1 + (E - e - kRange + kTop) / (kTop + 1) : 1; };
+  if constexpr (FIX) {
+    int emax = 0, nf = 0;
+    for (int s = tid; s < S::cells; s += S::threads) {
+      int e = 0;
+#pragma unroll
+      for (int code = 0; code < 8; ++code)
+        e = max(e, (int)(((unsigned int)__double2hiint(raw[code * S::cells + s]) >> 20) & 0x7FFu));
+      nf |= e == 0x7FF;
+      se[s] = (unsigned short)e;
+      emax = max(emax, e == 0x7FF ? 0 : e);
+    }
+    emax = __reduce_max_sync(0xffffffffu, emax);
+    nf = __any_sync(0xffffffffu, nf);
+    if ((tid & 31) == 0) {
+      if (emax > 0) atomicMax(&s_max, emax);
+      if (nf) atomicOr(&s_bad, 1);
+    }
+    __syncthreads();
+    E = s_max;
+    bad = s_bad != 0;
+    for (int s = tid; s < S::cells; s += S::threads)
+#pragma unroll
+      for (int code = 0; code < 8; ++code) {
+        const double v = raw[code * S::cells + s];
+        xs[code * S::cells + s] = E >= 64 ? fixed_pair(v, E) : fixed_pair_window(v, E, 0);
+      }
+    int emin = 0x7FF;
+    for (int c = tid; c < S::own; c += S::threads) {
+      const int e = exponent(c);
+      if (e > 0) emin = min(emin, e);
+    }
+    emin = __reduce_min_sync(0xffffffffu, emin);
+    if ((tid & 31) == 0) atomicMin(&s_min, emin);
+    __syncthreads();
+    emin = s_min;
+    if (emin < 0x7FF) passes = windows(emin);
+  }
+  for (int pass = 0; pass < passes; ++pass) {
+    double s1 = scale, s2 = 1.0, s64 = scale;
+    if constexpr (FIX) {
+      if (pass > 0) {  // the window of the next lower bits
+        __syncthreads();
+        for (int s = tid; s < S::cells; s += S::threads)
+          for_points(s, [&](int code, int i, bool in) {
+            xs[code * S::cells + s] = fixed_pair_window(in ? R.x[i] : 0.0, E, pass);
+          });
+        __syncthreads();
+      }
+      // rows are in units of scale 2^ex; applied in two factors where one would leave the FP64 range
+      const int ex = E - 1023 - kTop - pass * (kTop + 1);
+      const int ea = max(-900, min(900, ex));
+      s1 = scale * pow2(ea);
+      s64 = 64.0 * s1;
+      s2 = pow2(max(-1022, ex - ea));
+    }
+    const bool plain = passes == 1 && s2 == 1.0;
+    for (int c = tid; c < S::own; c += S::threads) {
+      const int a = c % S::TX, b = (c / S::TX) % S::TY, e = c / (S::TX * S::TY);
+      const int vi = i0 + a, vj = j0 + b, vk = k0 + e;
+      if (vi >= N || vj >= N || vk >= N) continue;
+      int last = 0;  // the cell's last pass
+      if constexpr (FIX)
+        if (passes > 1) {
+          const int e = exponent(c);
+          last = e > 0 ? windows(e) - 1 : 0;
+          if (pass > last) continue;
+        }
+      const V* base = xs + (a + 1 + S::W * (b + 1 + S::H * (e + 1)));
+      auto at = [&](int x, int y, int z) -> V {
+        return base[((x & 1) | ((y & 1) << 1) | ((z & 1) << 2)) * S::cells + (x >> 1) +
+                    S::W * ((y >> 1) + S::H * (z >> 1))];
+      };
+      RowSum<V> rs[8];
+      if constexpr (!FIX) stencil_rows(rs, at, std::make_integer_sequence<int, 125>{});
+      auto row = [&](auto code_) {
+        constexpr int code = decltype(code_)::value;
+        if (!((code & 1) || vi > 0) || !((code & 2) || vj > 0) || !((code & 4) || vk > 0)) return;
+        const int i = G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk;
+        if constexpr (FIX) {
+          const RowIn<EPI, T> in(R, i);
+          const RowSum<V> r = stencil_row<code, V>(at);
+          // |hi|, |lo| < 216 * 2^30: as one int64 directly, or in units of 64 where hi is large
+          const bool small = (unsigned long long)(r.hi + (1ll << 32)) < (1ull << 33);
+          const long long v = small ? (long long)((unsigned long long)r.hi << 30) + r.lo
+                                    : (long long)((unsigned long long)r.hi << 24) + (r.lo >> 6);
+          const double sv = small ? s1 : s64;
+          if (plain) {
+            finish_row<EPI>(R, in, i, (double)v, sv, R.wd[code]);
+          } else {
+            const double y = (double)v * sv * s2 + (pass > 0 ? R.out[i] : 0.0);
+            if (pass < last)
+              R.out[i] = y;
+            else
+              finish_row<EPI>(R, in, i, y, 1.0, R.wd[code]);
+          }
+        } else {
+          const RowIn<EPI, T> in(R, i);
+          finish_row<EPI>(R, in, i, rs[code].s, (float)scale, R.wd[code]);
+        }
+      };
+      row(std::integral_constant<int, 0>{});
+      row(std::integral_constant<int, 1>{});
+      row(std::integral_constant<int, 2>{});
+      row(std::integral_constant<int, 3>{});
+      row(std::integral_constant<int, 4>{});
+      row(std::integral_constant<int, 5>{});
+      row(std::integral_constant<int, 6>{});
+      row(std::integral_constant<int, 7>{});
+    }
+  }
+  if constexpr (FIX) {
+    if (bad) {  // rows that couple to a value that is not finite (staged as 0) are NaN
+      __syncthreads();
+      for (int c = tid; c < S::own; c += S::threads) {
+        const int a = c % S::TX, b = (c / S::TX) % S::TY, e = c / (S::TX * S::TY);
+        const int vi = i0 + a, vj = j0 + b, vk = k0 + e;
+        if (vi >= N || vj >= N || vk >= N) continue;
+        bool hit = false;
+        for (int z = -1; z <= 1; ++z)
+          for (int y = -1; y <= 1; ++y)
+            for (int x = -1; x <= 1; ++x)
+              hit = hit || se[a + 1 + x + S::W * (b + 1 + y + S::H * (e + 1 + z))] == 0x7FF;
+        if (!hit) continue;
+        for (int code = 0; code < 8; ++code)
+          if (((code & 1) || vi > 0) && ((code & 2) || vj > 0) && ((code & 4) || vk > 0))
+            R.out[G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk] = __longlong_as_double(0x7ff8000000000000ll);
+      }
+    }
+  }
+}
+
+// Small levels: one thread per dof (a block row per parity class, so that its
+// threads share one stencil) reads its 19 to 51 values from the caches and sums
+// them in the vectors' own arithmetic.  A level of a few thousand cells is bound by
+// the latency of its one launch, and this form has no staging, no scale and no
+// barrier: P2 16^3 in FP64 is 36 k rows of 23 operations, 1.3 us of the FP64 pipe.
+constexpr int kDirectBlock = 128;
+
+template <typename T, int EPI>
+__global__ void __launch_bounds__(kDirectBlock)
+    k_stencil2_direct(Lattice2 G, double scale, Rows<T> R, int nb, const int* __restrict__ bnd) {
+  const int N = G.N, tid = blockIdx.x * kDirectBlock + threadIdx.x;
+  const int stride = gridDim.x * gridDim.y * kDirectBlock;
+  for (int i = tid + blockIdx.y * gridDim.x * kDirectBlock; i < nb; i += stride) {  // Dirichlet rows: identity
+    identity_row<EPI>(R, bnd[i]);
+  }
+  const int vi = tid % N, vj = (tid / N) % N, vk = tid / (N * N);
+  if (vk >= N) return;
+  auto row = [&](auto code_) {
+    constexpr int code = decltype(code_)::value;
+    if (!((code & 1) || vi > 0) || !((code & 2) || vj > 0) || !((code & 4) || vk > 0)) return;
+    auto at = [&](int x, int y, int z) -> T {
+      // coarse coordinate v + floor(o / 2) of the point's class; interior for 0 < 2 v + o < 2 N
+      const int px = 2 * vi + x, py = 2 * vj + y, pz = 2 * vk + z;
+      const bool in = px > 0 && px < 2 * N && py > 0 && py < 2 * N && pz > 0 && pz < 2 * N;
+      const int c = (x & 1) | ((y & 1) << 1) | ((z & 1) << 2);
+      return in ? __ldg(R.x + G.off[c] + (px >> 1) + G.sy[c] * (py >> 1) + G.sz[c] * (pz >> 1)) : T(0);
+    };
+    const int i = G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk;
+    const RowIn<EPI, T> in(R, i);
+    const RowSum<T> r = stencil_row<code, T>(at);
+    finish_row<EPI>(R, in, i, r.s, (T)scale, R.wd[code]);
+  };
+  switch (blockIdx.y) {
+    case 0: row(std::integral_constant<int, 0>{}); break;
+    case 1: row(std::integral_constant<int, 1>{}); break;
+    case 2: row(std::integral_constant<int, 2>{}); break;
+    case 3: row(std::integral_constant<int, 3>{}); break;
+    case 4: row(std::integral_constant<int, 4>{}); break;
+    case 5: row(std::integral_constant<int, 5>{}); break;
+    case 6: row(std::integral_constant<int, 6>{}); break;
+    default: row(std::integral_constant<int, 7>{}); break;
+  }
+}
+
+// FP64 tiles: 71 KB, three blocks per SM; FP32 tiles have rows of 32 cells, so
+// that a warp's shared-memory accesses fall into distinct banks.
+#ifndef TL
+#define TL 16, 8, 4, 256, 3
+#endif
+#ifndef TF
+#define TF 32, 4, 8, 256, 3
+#endif
+#ifndef DIRECT
+#define DIRECT 16
+#endif
+using Tile64 = TileShape<TL>;
+using Tile32 = TileShape<TF>;
+constexpr int kDirectMax = DIRECT;
+
+Lattice2 lattice_of(const Level& L) {
+  Lattice2 G{};
+  G.N = L.N;
+  for (int code = 0; code < 8; ++code) {
+    const int c = code == 3 ? 4 : code == 4 ? 3 : code;
+    G.off[code] = L.num.off[c];
+    G.sy[code] = L.num.sx[c];
+    G.sz[code] = L.num.sx[c] * L.num.sy[c];
+  }
+  return G;
+}
+
+template <typename T>
+using Tile = typename std::conditional<sizeof(T) == 8, Tile64, Tile32>::type;
+
+template <int EPI, typename T>
+void launch_stencil(const Level& L, const Rows<T>& R, cudaStream_t s) {
+  using S = Tile<T>;
+  const double scale = 8.0 * (L.kappa0 / (120.0 * L.N));
+  if (L.N <= kDirectMax) {
+    k_stencil2_direct<T, EPI><<<dim3(ceil_div((long long)L.Q, kDirectBlock), 8), kDirectBlock, 0, s>>>(
+        lattice_of(L), scale, R, L.nb, L.bnd);
+  } else {
+    const int grid = ceil_div(L.N, S::TX) * ceil_div(L.N, S::TY) * ceil_div(L.N, S::KZ);
+    k_stencil2<T, EPI, S><<<grid, S::threads, S::template smem<T>(), s>>>(lattice_of(L), scale, R, L.nb, L.bnd);
+  }
+  LAUNCH_CHECK();
+}
+
+// The shared-memory limit of a kernel is a property of the device's context and
+// has one value per kernel, so setting it again for another hierarchy is harmless.
+template <typename T, int EPI>
+void set_smem() {
+  CUDA_CHECK(cudaFuncSetAttribute((const void*)k_stencil2<T, EPI, Tile<T>>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)Tile<T>::template smem<T>()));
+}
+
+template <int EPI, typename T>
+void launch(const Level& L, const Rows<T>& R, cudaStream_t s) {
+  constexpr bool F64 = sizeof(T) == 8;
+  if (L.deg == 1) {
+    const int grid = ceil_div(L.n, kP1Block);
+    const T* w = nullptr;
+    if constexpr (F64)
+      w = L.fw64;
+    else
+      w = L.fw32;
+    if (L.flux == FLUX_CONST)
+      k_flux1<T, true, EPI><<<grid, kP1Block, 0, s>>>(L.N, L.n, nullptr, (T)(L.kappa0 / L.N), R);
+    else
+      k_flux1<T, false, EPI><<<grid, kP1Block, 0, s>>>(L.N, L.n, w, T(0), R);
+    LAUNCH_CHECK();
+    return;
+  }
+  launch_stencil<EPI, T>(L, R, s);
+}
+
+}  // namespace
+
+// Data of the flux form of a level whose L.flux launch_uniform_geometry has set.
+void launch_flux_setup(Level& L, cudaStream_t s) {
+  if (L.flux == FLUX_NONE) return;
+  if (L.deg == 2) {
+    set_smem<double, EPI_APPLY>();
+    set_smem<double, EPI_CHEB>();
+    set_smem<float, EPI_APPLY>();
+    set_smem<float, EPI_CHEB>();
+  } else if (L.flux == FLUX_VAR) {
+    L.fw64.alloc((size_t)4 * L.n);
+    L.fw32.alloc((size_t)4 * L.n);
+    k_edge_weights<<<ceil_div(L.n, 128), 128, 0, s>>>(L.N, L.n, L.geo64.p + (size_t)5 * L.Cs, L.fw64, L.fw32);
+    LAUNCH_CHECK();
+  }
+}
+
+template <typename T>
+void launch_flux_apply(const Level& L, const T* x, T* y, cudaStream_t s) {
+  Rows<T> R{};
+  R.x = x;
+  R.out = y;
+  launch<EPI_APPLY>(L, R, s);
+}
+template void launch_flux_apply<double>(const Level&, const double*, double*, cudaStream_t);
+template void launch_flux_apply<float>(const Level&, const float*, float*, cudaStream_t);
+
+template <typename T>
+void launch_flux_cheb(const Level& L, const T* b, const T* x, T* xout, const T* din, T* dout, double c1, double c2,
+                      cudaStream_t s) {
+  Rows<T> R{};
+  R.x = x;
+  R.out = xout;
+  R.b = b;
+  R.din = din;
+  R.dout = dout;
+  if constexpr (sizeof(T) == 8)
+    R.dinv = L.dinv64;
+  else
+    R.dinv = L.dinv32;
+  R.c1 = (T)c1;
+  R.c2 = (T)c2;
+  const double k = L.kappa0 / L.N;
+  const int diag[8] = {54, 56, 56, 48, 56, 48, 48, 48};
+  for (int code = 0; code < 8; ++code)
+    R.wd[code] = (T)(L.deg == 1 ? c2 / (6.0 * k) : c2 * (120.0 / 8.0) / (diag[code] * k));
+  launch<EPI_CHEB>(L, R, s);
+}
+template void launch_flux_cheb<double>(const Level&, const double*, const double*, double*, const double*, double*,
+                                       double, double, cudaStream_t);
+template void launch_flux_cheb<float>(const Level&, const float*, const float*, float*, const float*, float*, double,
+                                      double, cudaStream_t);

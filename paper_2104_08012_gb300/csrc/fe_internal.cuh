@@ -225,6 +225,9 @@ inline int resident_grid(K kernel, int block, int work_items) {
 }
 
 // ---------------------------------------------------------- level data ---
+// Operator in flux form (fe_flux.cu): not available, a coefficient per tet, one coefficient.
+enum FluxForm { FLUX_NONE = 0, FLUX_VAR = 1, FLUX_CONST = 2 };
+
 struct Level {
   int N = 0, deg = 0, nd = 0;
   int n = 0, C = 0, V = 0, nb = 0;
@@ -248,6 +251,11 @@ struct Level {
   int pair_uniform = 0;
   DBuf<float> c32;        // [C] c in FP32
   DBuf<float2> cdf;       // [C] c as a float pair
+  // Flux form of the operator (fe_flux.cu): P1 with `uniform`, P2 also with one coefficient on the level
+  int flux = FLUX_NONE;
+  double kappa0 = 1.0;  // the coefficient of cell 0 (the one coefficient with FLUX_CONST)
+  DBuf<double> fw64;    // P1: [4][n] weights of the x, y, z edges starting at a vertex, diagonal
+  DBuf<float> fw32;
   DBuf<float2> massdf;    // |det J| / 120 (P1) or / 2520 (P2) per cell as a float pair (double-float mass)
   DBuf<double> dinv64;    // 1/diag(A)
   DBuf<float> dinv32;
@@ -439,6 +447,14 @@ void launch_apply_cheb64_df(const Level& L, const double* b, double* x, double* 
                             bool store_d, cudaStream_t s);
 void launch_apply_cheb64_cube_df(const Level& L, const double* b, double* x, double* y, double* d, double c1,
                                  double c2, bool store_d, cudaStream_t s);
+// Flux form (fe_flux.cu): set-up, y = A x, and a Chebyshev step xout = x + d with d = c1 din + c2 D^-1 (b - A x)
+// (xout another vector than x; d also to dout unless null; din is not read with c1 = 0).
+void launch_flux_setup(Level& L, cudaStream_t s);
+template <typename T>
+void launch_flux_apply(const Level& L, const T* x, T* y, cudaStream_t s);
+template <typename T>
+void launch_flux_cheb(const Level& L, const T* b, const T* x, T* xout, const T* din, T* dout, double c1, double c2,
+                      cudaStream_t s);
 void launch_build_valence(Level& L, cudaStream_t s);
 // band < 0: dense nci x nci (both triangles); band >= 0: band storage [nci][band + 1], lower triangle only
 void launch_coarse_assemble_p3(const Level& L0, const int* dof2int, int nci, double* A, int band, cudaStream_t s);
@@ -451,8 +467,9 @@ template <typename T>
 void launch_cheb_pc(int n, const T* z, T* x, T* d, double c1, double c2, bool first_from_zero, bool store_d,
                     cudaStream_t s);
 void launch_split_geometry(Level& L, cudaStream_t s);
-// Checks geo64 = c M cell by cell, fills c32 and cdf and sets L.uniform and L.pair_uniform (synchronises s).
-void launch_uniform_geometry(Level& L, int* dflag, cudaStream_t s);
+// Checks geo64 = c M cell by cell, fills c32 and cdf and sets L.uniform, L.pair_uniform, L.flux and L.kappa0
+// (synchronises s).  per_cell: treat every level as if the check had failed.
+void launch_uniform_geometry(Level& L, bool per_cell, int* dflag, cudaStream_t s);
 // b -= A g on interior rows and b = g on the boundary (inhomogeneous Dirichlet data, symmetric elimination)
 void launch_bc_lift(const Level& L, const double* g, double* b, cudaStream_t s);
 void launch_mass(const Level& L, const double* x, double* y, cudaStream_t s);

@@ -191,8 +191,10 @@ __global__ void k_geometry(int C, int Cs, const int* __restrict__ map, const dou
 // order 00, 01, 02, 11, 12, 22), c = geo64[22]; a cell whose G differs from
 // c M by more than 1e-12 |c| sets bit 0 of the flag, an odd cell whose c
 // differs from that of the cell before it (the other tet of its pair) bit 1.
-__global__ void k_uniform_geometry(int C, int Cs, const double* __restrict__ geo64, float* __restrict__ c32,
-                                   float2* __restrict__ cdf, int* __restrict__ flag) {
+// flag bits: 1 some G is not c M, 2 the tets of some pair differ in c, 4 kappa is
+// not one value (one atomic per warp that finds something new).
+__global__ void k_uniform_geometry(int C, int Cs, const double* __restrict__ geo64, const double* __restrict__ kappa,
+                                   float* __restrict__ c32, float2* __restrict__ cdf, int* flag) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= C) return;
   const double c = geo64[(size_t)5 * Cs + t];
@@ -200,8 +202,10 @@ __global__ void k_uniform_geometry(int C, int Cs, const double* __restrict__ geo
   bool ok = c >= 0x1p-100 && c <= 0x1p100;  // the float-pair kernels normalise c.hi by its exponent field
 #pragma unroll
   for (int a = 0; a < 5; ++a) ok = ok && fabs(geo64[(size_t)a * Cs + t] - m[a] * c) <= 1e-12 * c;
-  if (!ok) atomicOr(flag, 1);
-  if ((t & 1) && c != geo64[(size_t)5 * Cs + t - 1]) atomicOr(flag, 2);
+  const unsigned int mine = (ok ? 0u : 1u) | ((t & 1) && c != geo64[(size_t)5 * Cs + t - 1] ? 2u : 0u) |
+                            (kappa[t] != kappa[0] ? 4u : 0u);
+  const unsigned int found = __reduce_or_sync(__activemask(), mine);
+  if (found & ~(unsigned int)*(volatile int*)flag) atomicOr(flag, (int)found);
   c32[t] = (float)c;
   const float hi = (float)c;
   cdf[t] = make_float2(hi, (float)(c - (double)hi));
@@ -1215,19 +1219,21 @@ void launch_build_level(Level& L, cudaStream_t s) {
   LAUNCH_CHECK();
 }
 
-void launch_uniform_geometry(Level& L, int* dflag, cudaStream_t s) {
+void launch_uniform_geometry(Level& L, bool per_cell, int* dflag, cudaStream_t s) {
   if (!L.c32.p) {  // rows of Cs (a multiple of 128 cells): the tensor-core operator stages c32 by TMA tiles
     L.c32.alloc(L.Cs);
     L.cdf.alloc(L.Cs);
   }
   CUDA_CHECK(cudaMemsetAsync(dflag, 0, sizeof(int), s));
-  k_uniform_geometry<<<ceil_div(L.C, kBlock), kBlock, 0, s>>>(L.C, L.Cs, L.geo64, L.c32, L.cdf, dflag);
+  k_uniform_geometry<<<ceil_div(L.C, kBlock), kBlock, 0, s>>>(L.C, L.Cs, L.geo64, L.kappa, L.c32, L.cdf, dflag);
   LAUNCH_CHECK();
   int hflag = 1;
   CUDA_CHECK(cudaMemcpyAsync(&hflag, dflag, sizeof(int), cudaMemcpyDeviceToHost, s));
+  CUDA_CHECK(cudaMemcpyAsync(&L.kappa0, L.kappa, sizeof(double), cudaMemcpyDeviceToHost, s));
   CUDA_CHECK(cudaStreamSynchronize(s));
-  L.uniform = (hflag & 1) == 0 ? 1 : 0;
-  L.pair_uniform = hflag == 0 ? 1 : 0;
+  L.uniform = (hflag & 1) == 0 && !per_cell ? 1 : 0;
+  L.pair_uniform = (hflag & 3) == 0 ? 1 : 0;
+  L.flux = !L.uniform || L.deg > 2 ? FLUX_NONE : (hflag & 4) == 0 ? FLUX_CONST : L.deg == 1 ? FLUX_VAR : FLUX_NONE;
 }
 
 void launch_geometry(Level& L, cudaStream_t s) {
