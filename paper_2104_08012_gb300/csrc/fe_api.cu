@@ -293,14 +293,23 @@ static bool use_patch(const fe_hierarchy* h, int l) {
   return h->smoother == FE_SMOOTHER_PATCH && h->deg >= 2 && l >= 1 && h->L[l].pdof.p;
 }
 
-// lambda_max(M^-1 A) from the Lanczos tridiagonal of `steps` PCG iterations
-// (M = D, or the patch preconditioner on patch-smoothed levels).
-static double estimate_lmax(fe_hierarchy* h, int l, int steps, cudaStream_t s) {
+// lambda_max(M^-1 A) from the Lanczos tridiagonal of kLmaxSteps PCG iterations
+// (M = D, or the patch preconditioner on patch-smoothed levels), on every level.
+// The iterations of all levels are enqueued with the CG scalars of each copied to
+// a pinned history, and the host waits once (a wait per iteration cost more than
+// the small levels' iterations); iterations after a level's last valid one are
+// not used.
+constexpr int kLmaxSteps = 20;
+
+static void enqueue_lmax(fe_hierarchy* h, int l, double* hist, cudaStream_t s) {
   Level& L = h->L[l];
   const int n = L.n;
   ReduceCtx& R = h->red;
   double *b = h->b, *x = h->x, *r = h->r, *z = h->z, *p = h->p, *q = h->q;
   const bool patch = use_patch(h, l);
+  auto record = [&](int it) {
+    CUDA_CHECK(cudaMemcpyAsync(hist + (size_t)it * S_COUNT, R.scal, sizeof(double) * S_COUNT, cudaMemcpyDeviceToHost, s));
+  };
   launch_random(n, 0x2104080120210416ull + (uint64_t)l, b, s);
   launch_zero_boundary64(L, b, s);
   CUDA_CHECK(cudaMemsetAsync(x, 0, sizeof(double) * n, s));
@@ -312,11 +321,8 @@ static double estimate_lmax(fe_hierarchy* h, int l, int steps, cudaStream_t s) {
     launch_cheb_step<double>(n, r, nullptr, L.dinv64, p, z, 0.0, 1.0, true, s);  // z = p = D^-1 r
   }
   launch_dot<double>(R, n, r, z, S_RZ, s);
-  CUDA_CHECK(cudaMemcpyAsync(R.h_scal, R.scal, sizeof(double) * S_COUNT, cudaMemcpyDeviceToHost, s));
-  CUDA_CHECK(cudaStreamSynchronize(s));
-  if (!(R.h_scal[S_RZ] > 0.0)) return 1.0;  // no interior dofs: D^-1 A is the identity
-  std::vector<double> al, be;
-  for (int it = 0; it < steps; ++it) {
+  record(0);
+  for (int it = 0; it < kLmaxSteps; ++it) {
     apply_enqueue(h, l, p, q, FE_F64, s);
     launch_cg_alpha<double>(R, n, p, q, s);
     if (patch) {
@@ -327,13 +333,20 @@ static double estimate_lmax(fe_hierarchy* h, int l, int steps, cudaStream_t s) {
       launch_cg_update<double>(R, n, x, r, p, q, L.dinv64, z, s);
     }
     launch_cg_update_p<double>(R, n, p, z, s);
-    CUDA_CHECK(cudaMemcpyAsync(R.h_scal, R.scal, sizeof(double) * S_COUNT, cudaMemcpyDeviceToHost, s));
-    CUDA_CHECK(cudaStreamSynchronize(s));
-    const double alpha = R.h_scal[S_ALPHA], beta = R.h_scal[S_BETA];
+    record(it + 1);
+  }
+}
+
+static double lmax_of(const double* hist) {
+  if (!(hist[S_RZ] > 0.0)) return 1.0;  // no interior dofs: D^-1 A is the identity
+  std::vector<double> al, be;
+  for (int it = 0; it < kLmaxSteps; ++it) {
+    const double* sc = hist + (size_t)(it + 1) * S_COUNT;
+    const double alpha = sc[S_ALPHA], beta = sc[S_BETA];
     if (!(std::isfinite(alpha) && std::isfinite(beta)) || alpha <= 0) break;
     al.push_back(alpha);
     be.push_back(beta);
-    if (R.h_scal[S_RR] <= 0.0) break;
+    if (sc[S_RR] <= 0.0) break;
   }
   FE_REQUIRE(!al.empty(), FE_ERR_NAN, "eigenvalue estimate failed");
   const int k = (int)al.size();
@@ -343,6 +356,14 @@ static double estimate_lmax(fe_hierarchy* h, int l, int steps, cudaStream_t s) {
     if (i + 1 < k) off[i] = std::sqrt(be[i]) / al[i];
   }
   return tridiag_max_eig(a, off);
+}
+
+static void estimate_lmax(fe_hierarchy* h, cudaStream_t s) {
+  constexpr size_t per = (size_t)(kLmaxSteps + 1) * S_COUNT;
+  if (!h->lmax_hist) CUDA_CHECK(cudaMallocHost(&h->lmax_hist, sizeof(double) * per * FE_MAX_LEVELS));
+  for (int l = 0; l < h->nlev; ++l) enqueue_lmax(h, l, h->lmax_hist + per * l, s);
+  CUDA_CHECK(cudaStreamSynchronize(s));
+  for (int l = 0; l < h->nlev; ++l) h->L[l].lmax = lmax_of(h->lmax_hist + per * l);
 }
 
 // -------------------------------------------------------- V-cycle
@@ -1127,15 +1148,20 @@ static void set_coefficient_impl(fe_hierarchy* h, const double* kappa, cudaStrea
   }
   for (int l = h->nlev - 1; l >= 1; --l) launch_coarsen_kappa(h->L[l - 1], h->L[l], h->children, s);
   for (int l = 0; l < h->nlev; ++l) {
-    launch_geometry(h->L[l], s);
-    launch_split_geometry(h->L[l], s);
-    launch_uniform_geometry(h->L[l], h->geometry_form == FE_GEOMETRY_PER_CELL, h->cs.flag, s);
+    const bool per_cell = h->geometry_form == FE_GEOMETRY_PER_CELL;
+    if (h->L[l].kuhn) {
+      launch_scale_geometry(h->L[l], per_cell, h->cs.flag, s);
+    } else {
+      launch_geometry(h->L[l], s);
+      launch_split_geometry(h->L[l], s);
+      launch_uniform_geometry(h->L[l], per_cell, h->cs.flag, s);
+    }
     launch_flux_setup(h->L[l], s);
     launch_diag(h->L[l], h->tmp, s);
   }
   if (h->smoother == FE_SMOOTHER_PATCH && h->deg >= 2)
     for (int l = 1; l < h->nlev; ++l) launch_patch_setup(h->L[l], s);
-  for (int l = 0; l < h->nlev; ++l) h->L[l].lmax = estimate_lmax(h, l, 20, s);
+  estimate_lmax(h, s);
   if (h->nlev > 1) coarse_setup(h, s);
   invalidate_graphs(h);
   CUDA_CHECK(cudaStreamSynchronize(s));
@@ -1351,6 +1377,7 @@ void fe_hierarchy_destroy(fe_hierarchy* h) {
     if (g.stream) cudaStreamDestroy(g.stream);
   for (auto& L : h->L) bf16_forget_level(&L);
   red_free(h->red);
+  if (h->lmax_hist) cudaFreeHost(h->lmax_hist);
   delete h;
 }
 
@@ -1480,7 +1507,7 @@ int fe_set_smoother(fe_hierarchy* h, int smoother) {
           L.z32.alloc(L.n);
         }
       }
-    for (int l = 0; l < h->nlev; ++l) h->L[l].lmax = estimate_lmax(h, l, 20, s);
+    estimate_lmax(h, s);
     invalidate_graphs(h);
     CUDA_CHECK(cudaStreamSynchronize(s));
   }

@@ -4,8 +4,8 @@
 // Setup (once per coefficient): the interior block of the coarse operator is
 // assembled densely in the lexicographic lattice order of the interior dofs,
 // which makes it banded with half-bandwidth w = k (1 + e + e^2) (e interior
-// points per axis); a right-looking band Cholesky A = L L^T runs one launch
-// per column, and the inverse factor L^-1 is formed column by column (one
+// points per axis); a right-looking band Cholesky A = L L^T runs two launches
+// per panel of 32 columns, and the inverse factor L^-1 is formed column by column (one
 // warp per column, forward substitution over the band).
 // Solve (every V-cycle): x = L^-T (L^-1 b) as two dense triangular
 // matrix-vector products, which are fully parallel instead of 2 n
@@ -208,65 +208,199 @@ __global__ void __launch_bounds__(kBlkThreads) k_blkmv(int B, const double* __re
   }
 }
 
-// Right-looking step j: A[i][k] -= A[i][j] A[k][j] / A[j][j] for j < k <= i <= j + w.
-__global__ void k_chol_update(int n, int w, int j, double* __restrict__ A) {
-  const int b = blockIdx.x * blockDim.x + threadIdx.x + 1;  // k - j
-  const int a = blockIdx.y * blockDim.y + threadIdx.y + 1;  // i - j
-  const int wl = min(w, n - 1 - j);
-  if (a > wl || b > a) return;
-  const int i = j + a, k = j + b;
-  const double piv = A[(size_t)j * n + j];
-  A[(size_t)i * n + k] -= A[(size_t)i * n + j] * A[(size_t)k * n + j] / piv;
-}
+// ---- dense form: right-looking band Cholesky in panels of kPanel columns ----
+// One launch per column (the first form) spent the factorisation on launches:
+// P1 12^3 (1331 unknowns, half-bandwidth 133) took 4.7 ms for 12 M FMAs.  A panel
+// is two launches: the panel's columns of L (every block factors the diagonal
+// block itself, 32 serial steps, and solves for 8 rows), then the rank-32 update
+// of the trailing 16 x 16 tiles inside the band.  L goes to its own array, so
+// that blocks never read what another block of the same launch writes.
+constexpr int kPanel = 32, kPanelRows = 8, kUpdTile = 16;
 
-// L[i][j] = A[i][j] / sqrt(A[j][j]) inside the band, 0 elsewhere; flags a non-positive pivot.
-__global__ void k_chol_scale(int n, int w, double* __restrict__ A, double* __restrict__ dinv, int* __restrict__ flag) {
-  const size_t t = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= (size_t)n * n) return;
-  const int i = (int)(t / n), j = (int)(t - (size_t)i * n);
-  const double piv = A[(size_t)j * n + j];
-  if (i == j && !(piv > 0.0)) atomicOr(flag, 1);
-  if (i < j || i - j > w) {
-    A[t] = 0.0;
+// Columns [j0, j0 + nb) of L for the rows [j0, j0 + nb + w): block 0 also writes
+// the diagonal block; then block x the rows j0 + nb + 8 x .. + 7.
+__global__ void __launch_bounds__(kPanelRows * 32)
+    k_chol_panel(int n, int ld, int w, int j0, double* A, double* __restrict__ L, double* __restrict__ dinv,
+                 int* __restrict__ flag) {
+  __shared__ double D[kPanel][kPanel + 1], inv[kPanel];
+  __shared__ int bad;
+  if (threadIdx.x == 0) bad = 0;
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nb = min(kPanel, n - j0);
+  for (int r = wib; r < nb; r += kPanelRows)
+    D[r][lane] = lane <= r ? A[(size_t)(j0 + r) * n + j0 + lane] : 0.0;
+  __syncthreads();
+  for (int c = 0; c < nb; ++c) {
+    if (wib == 0) {  // one warp: FP64 square roots of every warp would queue on the FP64 pipe
+      const double piv = D[c][c], rs = rsqrt(piv);
+      __syncwarp();
+      if (lane > c && lane < nb) D[lane][c] *= rs;
+      if (lane == c) {
+        D[c][c] = piv * rs;
+        inv[c] = rs;
+        if (!(piv > 0.0)) bad = 1;
+      }
+    }
+    __syncthreads();
+    for (int r = c + 1 + wib; r < nb; r += kPanelRows)
+      if (lane > c && lane <= r) D[r][lane] -= D[r][c] * D[lane][c];
+    __syncthreads();
+  }
+  if (bad) {
+    if (threadIdx.x == 0) atomicOr(flag, 1);
     return;
   }
-  // every thread of column j reads the untouched pivot before it is overwritten:
-  // the diagonal is rescaled in a separate pass below
-  if (i != j) A[t] = A[t] / sqrt(piv);
+  if (blockIdx.x == 0) {
+    for (int r = wib; r < nb; r += kPanelRows) {
+      if (lane <= r) L[(size_t)(j0 + r) * ld + j0 + lane] = D[r][lane];
+      if (lane < r) A[(size_t)(j0 + lane) * n + j0 + r] = D[r][lane];
+    }
+    if (threadIdx.x < nb) dinv[j0 + threadIdx.x] = inv[threadIdx.x];
+  }
+  // one warp per row, lane = column: x_c = p_c / L_cc, then the later columns lose x_c L[., c]
+  const int i = j0 + nb + blockIdx.x * kPanelRows + wib;
+  if (i >= n || i >= j0 + nb + w) return;
+  double p = lane < nb ? A[(size_t)i * n + j0 + lane] : 0.0;
+  for (int c = 0; c < nb; ++c) {
+    const double x = __shfl_sync(0xffffffffu, p, c) * inv[c];
+    if (lane == c) p = x;
+    if (lane > c && lane < nb) p -= x * D[lane][c];
+  }
+  if (lane < nb) {
+    L[(size_t)i * ld + j0 + lane] = p;
+    A[(size_t)(j0 + lane) * n + i] = p;
+  }
 }
 
-__global__ void k_chol_diag(int n, double* __restrict__ A, double* __restrict__ dinv) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  const double l = sqrt(A[(size_t)j * n + j]);
-  A[(size_t)j * n + j] = l;
-  dinv[j] = 1.0 / l;
-}
-
-// X = L^-1, one warp per column j: X[i][j] = (delta_ij - sum_{k} L[i][k] X[k][j]) / L[i][i]
-// for k in [max(j, i-w), i-1]; the last w+1 values of the column live in a
-// shared-memory ring.
-__global__ void k_tri_inverse(int n, int w, const double* __restrict__ L, const double* __restrict__ dinv,
-                              double* __restrict__ Linv, double* __restrict__ LinvT) {
-  extern __shared__ double ring_all[];
-  const int warps = blockDim.x >> 5;
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int j = blockIdx.x * warps + wib;
-  if (j >= n) return;
-  const int R = w + 1;
-  double* ring = ring_all + (size_t)wib * R;
-  for (int i = j; i < n; ++i) {
-    const int kmin = max(j, i - w);
-    double s = 0.0;
-    for (int k = kmin + lane; k < i; k += 32) s += L[(size_t)i * n + k] * ring[k % R];
+// A[i][k] -= sum over the panel's columns of L[i][.] L[k][.] for j1 <= k <= i < j1 + w (j1: the first column after the
+// panel), one 16 x 16 tile per block.
+__global__ void __launch_bounds__(kUpdTile* kUpdTile)
+    k_chol_update(int n, int ld, int w, int j0, double* __restrict__ A, const double* __restrict__ L) {
+  if (blockIdx.x > blockIdx.y) return;
+  __shared__ double Li[kUpdTile][kPanel + 1], Lk[kUpdTile][kPanel + 1];
+  const int j1 = j0 + kPanel, end = min(n, j1 + w);
+  const int i0 = j1 + blockIdx.y * kUpdTile, k0 = j1 + blockIdx.x * kUpdTile;
+  for (int t = threadIdx.x; t < kUpdTile * kPanel; t += kUpdTile * kUpdTile) {
+    const int r = t / kPanel, c = t % kPanel;
+    Li[r][c] = i0 + r < end ? L[(size_t)(i0 + r) * ld + j0 + c] : 0.0;
+    Lk[r][c] = k0 + r < end ? L[(size_t)(k0 + r) * ld + j0 + c] : 0.0;
+  }
+  __syncthreads();
+  const int r = threadIdx.x / kUpdTile, c = threadIdx.x % kUpdTile, i = i0 + r, k = k0 + c;
+  if (i >= end || k > i) return;
+  double s0 = 0.0, s1 = 0.0;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) {
-      const double xi = ((i == j) ? 1.0 : 0.0) - s;
-      const double v = xi * dinv[i];
+  for (int m = 0; m < kPanel; m += 2) {
+    s0 = fma(Li[r][m], Lk[c][m], s0);
+    s1 = fma(Li[r][m + 1], Lk[c][m + 1], s1);
+  }
+  A[(size_t)i * n + k] -= s0 + s1;
+}
+
+// One column j of L^-1 (forward) or of A^-1 = L^-T L^-1 (backward) per warp, 32
+// rows at a time with lane = row: the rows already known, at most w + 31 of them,
+// lie in the warp's ring in shared memory; each lane sums over them, with one
+// coalesced load of 32 entries of L^T (forward) or L (backward) per known row, and
+// the 32 new rows follow by substitution in the diagonal block, one shuffle each.
+// Both need n^2 w / 2 FMAs in all (A^-1 is symmetric, so its column starts at
+// row j), bound by the FP64 pipe.  A row at a time with a reduction over the warp
+// (the first form of L^-1) was bound by its latency, 1.5 ms for P1 12^3 and
+// 14 ms for P2 8^3, and A^-1 as a product of dense triangles needs n^3 / 6 FMAs,
+// 1.0 and 11.3 ms.
+constexpr int kInvCols = 8;    // columns (warps) per block
+constexpr int kInvLoads = 16;  // loads in flight per lane
+
+// U: L^T in the upper triangle, rows of n; dinv: 1 / diagonal of L.
+__global__ void __launch_bounds__(kInvCols * 32)
+    k_tri_forward(int n, int w, const double* __restrict__ U, const double* __restrict__ dinv,
+                  double* __restrict__ Linv, double* __restrict__ LinvT) {
+  extern __shared__ double ring_all[];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, j = blockIdx.x * kInvCols + wib;
+  if (j >= n) return;
+  const int R = (w + 63) & ~31;  // ring of whole 32-row groups, the current one included
+  double* ring = ring_all + (size_t)wib * R;
+  for (int i0 = j & ~31; i0 < n; i0 += 32) {
+    const int i = i0 + lane, ic = min(i, n - 1);
+    double s0 = i == j ? 1.0 : 0.0, s1 = 0.0;
+    int k = max(j, i0 - w);
+    const int base = k / R * R;
+    auto known = [&](int q) { return ring[q - base >= R ? q - base - R : q - base]; };
+    for (; k + kInvLoads <= i0; k += kInvLoads) {
+      double a[kInvLoads];
+#pragma unroll
+      for (int q = 0; q < kInvLoads; ++q) a[q] = U[(size_t)(k + q) * n + ic];
+#pragma unroll
+      for (int q = 0; q < kInvLoads; q += 2) {
+        s0 = fma(-a[q], known(k + q), s0);
+        s1 = fma(-a[q + 1], known(k + q + 1), s1);
+      }
+    }
+    for (; k < i0; ++k) s0 = fma(-U[(size_t)k * n + ic], known(k), s0);
+    double s = s0 + s1, u[32];
+    const double di = dinv[ic];
+#pragma unroll
+    for (int c = 0; c < 32; ++c) u[c] = i0 + c < n && lane > c ? U[(size_t)(i0 + c) * n + ic] : 0.0;
+#pragma unroll
+    for (int c = 0; c < 32; ++c) {  // rows before j and beyond n hold 0 and change nothing
+      const double x = __shfl_sync(0xffffffffu, s * di, c);
+      s = lane == c ? x : fma(-u[c], x, s);
+    }
+    __syncwarp();
+    if (i < n) {
+      const double v = i >= j ? s : 0.0;
       ring[i % R] = v;
-      Linv[(size_t)i * n + j] = v;
-      LinvT[(size_t)j * n + i] = v;
+      if (i >= j) {
+        Linv[(size_t)i * n + j] = v;
+        LinvT[(size_t)j * n + i] = v;
+      }
+    }
+    __syncwarp();
+  }
+}
+
+// L: rows of ld.  Writes rows j .. n - 1 of column j of A^-1 and their mirror images.
+__global__ void __launch_bounds__(kInvCols * 32)
+    k_tri_backward(int n, int ld, int w, const double* __restrict__ L, const double* __restrict__ dinv,
+                   const double* __restrict__ LinvT, double* __restrict__ Ainv) {
+  extern __shared__ double ring_all[];
+  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, j = blockIdx.x * kInvCols + wib;
+  if (j >= n) return;
+  const int R = (w + 63) & ~31;
+  double* ring = ring_all + (size_t)wib * R;
+  for (int i0 = (n - 1) & ~31; i0 + 31 >= j; i0 -= 32) {
+    const int i = i0 + lane, ic = min(i, n - 1);
+    double s0 = i >= j && i < n ? LinvT[(size_t)j * n + i] : 0.0, s1 = 0.0;
+    const int end = min(n, i0 + 32 + w);
+    int k = i0 + 32;
+    const int base = k / R * R;
+    auto known = [&](int q) { return ring[q - base >= R ? q - base - R : q - base]; };
+    // entries of L beyond the band of row k are not stored
+    for (; k + kInvLoads <= end; k += kInvLoads) {
+      double a[kInvLoads];
+#pragma unroll
+      for (int q = 0; q < kInvLoads; ++q) a[q] = k + q - i <= w ? L[(size_t)(k + q) * ld + ic] : 0.0;
+#pragma unroll
+      for (int q = 0; q < kInvLoads; q += 2) {
+        s0 = fma(-a[q], known(k + q), s0);
+        s1 = fma(-a[q + 1], known(k + q + 1), s1);
+      }
+    }
+    for (; k < end; ++k) s0 = fma(k - i <= w ? -L[(size_t)k * ld + ic] : 0.0, known(k), s0);
+    double s = s0 + s1, u[32];
+    const double di = dinv[ic];
+#pragma unroll
+    for (int c = 0; c < 32; ++c) u[c] = i0 + c < n && lane < c ? L[(size_t)(i0 + c) * ld + ic] : 0.0;
+#pragma unroll
+    for (int c = 31; c >= 0; --c) {  // rows beyond n hold 0; rows before j are not written
+      const double x = __shfl_sync(0xffffffffu, s * di, c);
+      s = lane == c ? x : fma(-u[c], x, s);
+    }
+    __syncwarp();
+    if (i < n) {
+      ring[i % R] = s;
+      if (i >= j) {
+        Ainv[(size_t)i * n + j] = s;
+        Ainv[(size_t)j * n + i] = s;
+      }
     }
     __syncwarp();
   }
@@ -311,46 +445,6 @@ __global__ void __launch_bounds__(kRowThreads) k_trimv(int n, const double* __re
 #pragma unroll
     for (int w = 0; w < kRowThreads / 32; ++w) t += sh[w];
     out[row] = t;
-  }
-}
-
-// The coarse inverse A^-1 = L^-T L^-1 from the inverse factor (row-major,
-// lower triangular): entry (i, j) is the sum over k >= max(i, j) of
-// Linv[k][i] Linv[k][j], in FP64 (n x n, row-major).  One 32 x 32 tile per
-// block, tiles above the diagonal only, each mirrored.
-constexpr int kGramTile = 32;
-__global__ void __launch_bounds__(kGramTile * 8) k_inv_gram(int n, const double* __restrict__ Linv,
-                                                            double* __restrict__ Ainv) {
-  const int I = blockIdx.y, J = blockIdx.x;
-  if (I > J) return;
-  __shared__ double si[kGramTile][kGramTile + 1], sj[kGramTile][kGramTile + 1];
-  const int tx = threadIdx.x, ty = threadIdx.y;  // 32 x 8
-  const int i0 = I * kGramTile, j0 = J * kGramTile;
-  double acc[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int k0 = j0; k0 < n; k0 += kGramTile) {  // Linv[k][i] = 0 for k < i: k starts at the tile's larger index
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const int k = k0 + ty + 8 * r;
-      si[ty + 8 * r][tx] = k < n && i0 + tx < n ? Linv[(size_t)k * n + i0 + tx] : 0.0;
-      sj[ty + 8 * r][tx] = k < n && j0 + tx < n ? Linv[(size_t)k * n + j0 + tx] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int kk = 0; kk < kGramTile; ++kk) {
-      const double b = sj[kk][tx];
-#pragma unroll
-      for (int r = 0; r < 4; ++r) acc[r] = fma(si[kk][ty + 8 * r], b, acc[r]);
-    }
-    __syncthreads();
-  }
-  const int j = j0 + tx;
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    const int i = i0 + ty + 8 * r;
-    if (i < n && j < n) {
-      Ainv[(size_t)i * n + j] = acc[r];
-      Ainv[(size_t)j * n + i] = acc[r];
-    }
   }
 }
 
@@ -527,32 +621,35 @@ static void coarse_setup_dense(fe_hierarchy* h, cudaStream_t s) {
   } else {
     launch_coarse_assemble_p3(L0, cs.dof2int, nci, cs.A, -1, s);
   }
-  for (int j = 0; j + 1 < nci; ++j) {
-    const int wl = std::min(w, nci - 1 - j);
-    dim3 blk(32, 8), grd(ceil_div(wl, 32), ceil_div(wl, 8));
-    k_chol_update<<<grd, blk, 0, s>>>(nci, w, j, cs.A);
-  }
-  LAUNCH_CHECK();
+  // L in the storage of the float-pair inverse, which is formed from Linv below (8-byte entries, rows of ld)
+  double* Lf = reinterpret_cast<double*>(cs.AinvDF.p);
   CUDA_CHECK(cudaMemsetAsync(cs.flag, 0, sizeof(int), s));
-  k_chol_scale<<<ceil_div((long long)nn, kBlock), kBlock, 0, s>>>(nci, w, cs.A, cs.t0, cs.flag);
-  LAUNCH_CHECK();
-  k_chol_diag<<<ceil_div(nci, kBlock), kBlock, 0, s>>>(nci, cs.A, cs.t0);
-  LAUNCH_CHECK();
+  for (int j = 0; j < nci; j += kPanel) {
+    const int rows = std::min(w, nci - j - std::min(kPanel, nci - j));  // rows of L below the panel's diagonal block
+    k_chol_panel<<<std::max(1, ceil_div(rows, kPanelRows)), kPanelRows * 32, 0, s>>>(nci, cs.ld, w, j, cs.A, Lf, cs.t0,
+                                                                                    cs.flag);
+    LAUNCH_CHECK();
+    if (rows > 0) {
+      const int t = ceil_div(rows, kUpdTile);
+      k_chol_update<<<dim3(t, t), kUpdTile * kUpdTile, 0, s>>>(nci, cs.ld, w, j, cs.A, Lf);
+      LAUNCH_CHECK();
+    }
+  }
   int hflag = 0;
   CUDA_CHECK(cudaMemcpyAsync(&hflag, cs.flag, sizeof(int), cudaMemcpyDeviceToHost, s));
   CUDA_CHECK(cudaStreamSynchronize(s));
   FE_REQUIRE(hflag == 0, FE_ERR_ARG, "coarse matrix is not positive definite");
   CUDA_CHECK(cudaMemsetAsync(cs.Linv, 0, sizeof(double) * nn, s));
   CUDA_CHECK(cudaMemsetAsync(cs.LinvT, 0, sizeof(double) * nn, s));
-  const int warps = 4;
-  const size_t shm = sizeof(double) * (size_t)(w + 1) * warps;
-  FE_REQUIRE(shm <= 200 * 1024, FE_ERR_UNSUPPORTED, "coarse band too wide");
-  if (shm > 48 * 1024) CUDA_CHECK(cudaFuncSetAttribute(k_tri_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm));
-  k_tri_inverse<<<ceil_div(nci, warps), warps * 32, shm, s>>>(nci, w, cs.A, cs.t0, cs.Linv, cs.LinvT);
+  const size_t shm = sizeof(double) * (size_t)((w + 63) & ~31) * kInvCols;
+  constexpr size_t kRingMax = 200 * 1024;
+  FE_REQUIRE(shm <= kRingMax, FE_ERR_UNSUPPORTED, "coarse band too wide");
+  CUDA_CHECK(cudaFuncSetAttribute(k_tri_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingMax));
+  CUDA_CHECK(cudaFuncSetAttribute(k_tri_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRingMax));
+  k_tri_forward<<<ceil_div(nci, kInvCols), kInvCols * 32, shm, s>>>(nci, w, cs.A, cs.t0, cs.Linv, cs.LinvT);
   LAUNCH_CHECK();
-  // A^-1 = L^-T L^-1 in FP64 into cs.A (the factor is no longer needed), then as scaled float pairs
-  const int tiles = ceil_div(nci, kGramTile);
-  k_inv_gram<<<dim3(tiles, tiles), dim3(kGramTile, 8), 0, s>>>(nci, cs.Linv, cs.A);
+  // A^-1 in FP64 into cs.A (L^T is no longer needed), then as scaled float pairs
+  k_tri_backward<<<ceil_div(nci, kInvCols), kInvCols * 32, shm, s>>>(nci, cs.ld, w, Lf, cs.t0, cs.LinvT, cs.A);
   LAUNCH_CHECK();
   CUDA_CHECK(cudaMemsetAsync(cs.flag, 0, sizeof(int), s));
   k_diag_exponent<<<ceil_div(nci, kBlock), kBlock, 0, s>>>(nci, cs.A, cs.flag);

@@ -246,6 +246,7 @@ struct Level {
   // vertex coordinates (uniform = 1 when every cell agrees) and keeps c for the operator kernels that then read
   // one value per cell instead of six.
   int uniform = 0;
+  int kuhn = 0;  // the geometry alone is (h / w) M in every cell (found with the first coefficient)
   // 1 when also the two tets of every pair with the same first axis (cells 6q + 2k, 6q + 2k + 1: they share a face)
   // have the same c, so that the FP64 P2 operator applies such pairs as one unit
   int pair_uniform = 0;
@@ -415,7 +416,7 @@ struct fe_hierarchy {
   } cgloop;
   DBuf<double> xcg, cgp;  // CG iterate of the graph loop; loop target
   DBuf<int> cgctl;        // loop counters
-  bool lmax_valid = false;
+  double* lmax_hist = nullptr;  // pinned: CG scalars of the eigenvalue estimates, [level][iteration][S_COUNT]
   int f64_mode = FE_F64_DOUBLE_FLOAT;  // arithmetic of FP64 operator applications
   int fuse_smoother = 0;               // Chebyshev update fused into the operator kernel (measured slower on GB300)
   int smoother = FE_SMOOTHER_JACOBI;   // preconditioner of the Chebyshev smoother
@@ -470,6 +471,8 @@ void launch_split_geometry(Level& L, cudaStream_t s);
 // Checks geo64 = c M cell by cell, fills c32 and cdf and sets L.uniform, L.pair_uniform, L.flux and L.kappa0
 // (synchronises s).  per_cell: treat every level as if the check had failed.
 void launch_uniform_geometry(Level& L, bool per_cell, int* dflag, cudaStream_t s);
+// The geometric factors of a level with L.kuhn for a new L.kappa, and the flags of launch_uniform_geometry.
+void launch_scale_geometry(Level& L, bool per_cell, int* dflag, cudaStream_t s);
 // b -= A g on interior rows and b = g on the boundary (inhomogeneous Dirichlet data, symmetric elimination)
 void launch_bc_lift(const Level& L, const double* g, double* b, cudaStream_t s);
 void launch_mass(const Level& L, const double* x, double* y, cudaStream_t s);

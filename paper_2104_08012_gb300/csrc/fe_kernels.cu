@@ -211,6 +211,34 @@ __global__ void k_uniform_geometry(int C, int Cs, const double* __restrict__ geo
   cdf[t] = make_float2(hi, (float)(c - (double)hi));
 }
 
+// A new coefficient on a level whose geometry has been found to be G = (h / w) M
+// in every cell (L.kuhn): every array of geometric factors is kappa times it, in
+// one pass over kappa instead of three over the vertex coordinates and each
+// other's results (bound by the 140 bytes per cell that it writes).  Same flag
+// bits as k_uniform_geometry.
+__global__ void k_scale_geometry(int C, int Cs, double hw, const double* __restrict__ kappa, double* __restrict__ geo64,
+                                 float* __restrict__ geo32, float2* __restrict__ geodf, float* __restrict__ c32,
+                                 float2* __restrict__ cdf, int* flag) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= C) return;
+  const double k = kappa[t], c = k * hw;
+  const float hi = (float)c, lo = (float)(c - (double)hi);
+  const float m[6] = {2.0f, -1.0f, 0.0f, 2.0f, -1.0f, 1.0f};  // powers of two: scaling by them is exact
+#pragma unroll
+  for (int a = 0; a < 6; ++a) {
+    const size_t i = (size_t)a * Cs + t;
+    geo64[i] = a == 5 ? c : a == 2 ? 0.0 : (a == 0 || a == 3) ? 2.0 * c : -c;
+    geo32[i] = m[a] * hi;
+    geodf[i] = make_float2(m[a] * hi, m[a] * lo);
+  }
+  c32[t] = hi;
+  cdf[t] = make_float2(hi, lo);
+  const bool ok = c >= 0x1p-100 && c <= 0x1p100;
+  const unsigned int mine = (ok ? 0u : 1u) | ((t & 1) && k != kappa[t - 1] ? 2u : 0u) | (k != kappa[0] ? 4u : 0u);
+  const unsigned int found = __reduce_or_sync(__activemask(), mine);
+  if (found & ~(unsigned int)*(volatile int*)flag) atomicOr(flag, (int)found);
+}
+
 // ------------------------------------------------------ operator apply
 // One thread per tet: gather the cell dofs through the cell->dof map
 // (coalesced: the map is stored [dof][cell]), contract with the cell's
@@ -632,6 +660,32 @@ __global__ void k_gradient(int C, int Cs, const int* __restrict__ map, const dou
 }
 
 // ------------------------------------------------------ mesh queries
+// P1 on Kuhn tets: along the tet's path of axis edges int_K grad lambda . grad u
+// = h / 6 times the sum of the three products of differences (10 FP64 operations
+// and no geometry, against about 150 with the metric of general tets).
+__global__ void k_gradient_p1(int N, int C, double h6, const double* __restrict__ u, const double* __restrict__ lam,
+                              double* __restrict__ g) {
+  const int c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= C) return;
+  const int q = c / 6, t = c - 6 * q, ci = q % N, cj = (q / N) % N, ck = q / (N * N);
+  const int n1 = N + 1, st[3] = {1, n1, n1 * n1};
+  int p0, p1, p2;
+  kuhn_perm(t, p0, p1, p2);
+  const int s0 = p0 == 0 ? st[0] : p0 == 1 ? st[1] : st[2], s1 = p1 == 0 ? st[0] : p1 == 1 ? st[1] : st[2];
+  const int v0 = ci + n1 * (cj + n1 * ck), v1 = v0 + s0, v2 = v1 + s1, v3 = v0 + 1 + n1 + n1 * n1;
+  // boundary dofs count as 0 (the origin of a cube is one at ci = 0, ..., its far corner at ci = N - 1, ...)
+  auto in = [&](int bx, int by, int bz) {
+    const int x = ci + bx, y = cj + by, z = ck + bz;
+    return x > 0 && x < N && y > 0 && y < N && z > 0 && z < N;
+  };
+  const bool b0 = in(0, 0, 0), b3 = in(1, 1, 1), b1 = in(p0 == 0, p0 == 1, p0 == 2), b2 = in(p2 != 0, p2 != 1, p2 != 2);
+  const double u0 = b0 ? __ldg(u + v0) : 0.0, u1 = b1 ? __ldg(u + v1) : 0.0, u2 = b2 ? __ldg(u + v2) : 0.0,
+               u3 = b3 ? __ldg(u + v3) : 0.0;
+  const double l0 = b0 ? __ldg(lam + v0) : 0.0, l1 = b1 ? __ldg(lam + v1) : 0.0, l2 = b2 ? __ldg(lam + v2) : 0.0,
+               l3 = b3 ? __ldg(lam + v3) : 0.0;
+  g[c] = h6 * fma(u1 - u0, l1 - l0, fma(u2 - u1, l2 - l1, (u3 - u2) * (l3 - l2)));
+}
+
 __global__ void k_dof_coords(Numbering num, int n, double* __restrict__ xyz) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
@@ -1219,6 +1273,16 @@ void launch_build_level(Level& L, cudaStream_t s) {
   LAUNCH_CHECK();
 }
 
+static void take_geometry_flags(Level& L, bool per_cell, int* dflag, cudaStream_t s) {
+  int hflag = 1;
+  CUDA_CHECK(cudaMemcpyAsync(&hflag, dflag, sizeof(int), cudaMemcpyDeviceToHost, s));
+  CUDA_CHECK(cudaMemcpyAsync(&L.kappa0, L.kappa, sizeof(double), cudaMemcpyDeviceToHost, s));
+  CUDA_CHECK(cudaStreamSynchronize(s));
+  L.uniform = (hflag & 1) == 0 && !per_cell ? 1 : 0;
+  L.pair_uniform = (hflag & 3) == 0 ? 1 : 0;
+  L.flux = !L.uniform || L.deg > 2 ? FLUX_NONE : (hflag & 4) == 0 ? FLUX_CONST : L.deg == 1 ? FLUX_VAR : FLUX_NONE;
+}
+
 void launch_uniform_geometry(Level& L, bool per_cell, int* dflag, cudaStream_t s) {
   if (!L.c32.p) {  // rows of Cs (a multiple of 128 cells): the tensor-core operator stages c32 by TMA tiles
     L.c32.alloc(L.Cs);
@@ -1227,13 +1291,17 @@ void launch_uniform_geometry(Level& L, bool per_cell, int* dflag, cudaStream_t s
   CUDA_CHECK(cudaMemsetAsync(dflag, 0, sizeof(int), s));
   k_uniform_geometry<<<ceil_div(L.C, kBlock), kBlock, 0, s>>>(L.C, L.Cs, L.geo64, L.kappa, L.c32, L.cdf, dflag);
   LAUNCH_CHECK();
-  int hflag = 1;
-  CUDA_CHECK(cudaMemcpyAsync(&hflag, dflag, sizeof(int), cudaMemcpyDeviceToHost, s));
-  CUDA_CHECK(cudaMemcpyAsync(&L.kappa0, L.kappa, sizeof(double), cudaMemcpyDeviceToHost, s));
-  CUDA_CHECK(cudaStreamSynchronize(s));
-  L.uniform = (hflag & 1) == 0 && !per_cell ? 1 : 0;
-  L.pair_uniform = (hflag & 3) == 0 ? 1 : 0;
-  L.flux = !L.uniform || L.deg > 2 ? FLUX_NONE : (hflag & 4) == 0 ? FLUX_CONST : L.deg == 1 ? FLUX_VAR : FLUX_NONE;
+  take_geometry_flags(L, per_cell, dflag, s);
+  L.kuhn = L.uniform || (per_cell && L.kuhn);
+}
+
+void launch_scale_geometry(Level& L, bool per_cell, int* dflag, cudaStream_t s) {
+  const double w = L.deg == 1 ? 6.0 : L.deg == 2 ? 120.0 : 161280.0;
+  CUDA_CHECK(cudaMemsetAsync(dflag, 0, sizeof(int), s));
+  k_scale_geometry<<<ceil_div(L.C, kBlock), kBlock, 0, s>>>(L.C, L.Cs, 1.0 / (w * L.N), L.kappa, L.geo64, L.geo32,
+                                                           L.geodf, L.c32, L.cdf, dflag);
+  LAUNCH_CHECK();
+  take_geometry_flags(L, per_cell, dflag, s);
 }
 
 void launch_geometry(Level& L, cudaStream_t s) {
@@ -1335,6 +1403,11 @@ void launch_diag(Level& L, double* diag, cudaStream_t s) {
 }
 
 void launch_gradient(const Level& L, const double* u, const double* lam, double* g, cudaStream_t s) {
+  if (L.deg == 1 && L.kuhn) {
+    k_gradient_p1<<<ceil_div(L.C, kBlock), kBlock, 0, s>>>(L.N, L.C, 1.0 / (6.0 * L.N), u, lam, g);
+    LAUNCH_CHECK();
+    return;
+  }
   by_degree(L.deg, [&](auto D) {
     k_gradient<D.value><<<ceil_div(L.C, kBlock), kBlock, 0, s>>>(L.C, L.Cs, L.map, L.vx, L.vy, L.vz, u, lam, g);
   });
