@@ -1292,6 +1292,7 @@ fe_hierarchy* hierarchy_create(int N0, int nrefine, int degree) {
     }
   }
   build_transfer_tables(h->tt, degree);
+  if (degree == 2) restrict_p2_prepare();
   for (int l = 0; l < h->nlev; ++l) {
     if (l > 0) build_level_transfer_index(h->L[l], h->L[l - 1], h->tt);
     launch_build_valence(h->L[l], s);

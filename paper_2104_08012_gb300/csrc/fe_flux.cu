@@ -37,7 +37,7 @@ struct Rows {
   const T* x;     // the operator's input (also the iterate that a Chebyshev step updates)
   T* out;         // APPLY: y; CHEB: the new iterate (another vector than x)
   const T* b;     // CHEB: right-hand side
-  const T* din;   // CHEB, c1 != 0: the previous direction
+  const T* din;   // CHEB: the previous direction (null: c1 = 0)
   T* dout;        // CHEB: the new direction (null: not stored)
   const T* dinv;  // CHEB on P1 with a coefficient per cell: inverse diagonal
   T c1, c2;
@@ -48,10 +48,11 @@ struct Rows {
 template <int EPI, typename T>
 struct RowIn {
   T b = T(0), d = T(0), x = T(0);
+  __device__ __forceinline__ RowIn() {}
   __device__ __forceinline__ RowIn(const Rows<T>& R, int i) {
     if constexpr (EPI == EPI_CHEB) {
       b = __ldg(R.b + i);
-      if (R.c1 != T(0)) d = R.din[i];
+      if (R.din) d = R.din[i];
       x = __ldg(R.x + i);
     }
   }
@@ -69,7 +70,7 @@ __device__ __forceinline__ void finish_row(const Rows<T>& R, const RowIn<EPI, T>
     R.out[i] = v * s;
   } else {
     const T r = fma_t(-v, s, in.b);
-    const T dn = R.c1 != T(0) ? fma_t(w, r, R.c1 * in.d) : w * r;
+    const T dn = R.din ? fma_t(w, r, R.c1 * in.d) : w * r;
     if (R.dout) R.dout[i] = dn;
     R.out[i] = in.x + dn;
   }
@@ -240,9 +241,14 @@ struct RowSum<double> {
 template <>
 struct RowSum<Pair32> {
   long long hi = 0, lo = 0;
+  // one 32 x 32 + 64 bit instruction per word (left to itself the compiler turns the small coefficients into sign
+  // extensions, shifts and carried additions, three instructions each)
+  static __device__ __forceinline__ void mad(long long& a, int k, int v) {
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a) : "r"(v), "r"(k));
+  }
   template <typename... A>
   __device__ __forceinline__ void add(int k, A... v) {  // sums of at most two staged values
-    ((hi += (long long)k * v.hi, lo += (long long)k * v.lo), ...);
+    ((mad(hi, k, v.hi), mad(lo, k, v.lo)), ...);
   }
 };
 
@@ -514,7 +520,7 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
       s64 = 64.0 * s1;
       s2 = pow2(max(-1022, ex - ea));
     }
-    const bool plain = passes == 1 && s2 == 1.0;
+    const bool plain = !FIX || (passes == 1 && E > 300 && E < 1900);  // one window, one factor
     for (int c = tid; c < S::own; c += S::threads) {
       const int a = c % S::TX, b = (c / S::TX) % S::TY, e = c / (S::TX * S::TY);
       const int vi = i0 + a, vj = j0 + b, vk = k0 + e;
@@ -532,8 +538,15 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
                     S::W * ((y >> 1) + S::H * (z >> 1))];
       };
       RowSum<V> rs[8];
+      RowIn<EPI, T> ins[8];  // FP32: every row's vectors in flight before the rows are formed
+      if constexpr (!FIX && EPI == EPI_CHEB) {
+#pragma unroll
+        for (int code = 0; code < 8; ++code)
+          if (((code & 1) || vi > 0) && ((code & 2) || vj > 0) && ((code & 4) || vk > 0))
+            ins[code] = RowIn<EPI, T>(R, G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk);
+      }
       if constexpr (!FIX) stencil_rows(rs, at, std::make_integer_sequence<int, 125>{});
-      auto row = [&](auto code_) {
+      auto row = [&](auto code_, auto plain_) {
         constexpr int code = decltype(code_)::value;
         if (!((code & 1) || vi > 0) || !((code & 2) || vj > 0) || !((code & 4) || vk > 0)) return;
         const int i = G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk;
@@ -545,7 +558,7 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
           const long long v = small ? (long long)((unsigned long long)r.hi << 30) + r.lo
                                     : (long long)((unsigned long long)r.hi << 24) + (r.lo >> 6);
           const double sv = small ? s1 : s64;
-          if (plain) {
+          if constexpr (decltype(plain_)::value) {
             finish_row<EPI>(R, in, i, (double)v, sv, R.wd[code]);
           } else {
             const double y = (double)v * sv * s2 + (pass > 0 ? R.out[i] : 0.0);
@@ -555,18 +568,23 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
               finish_row<EPI>(R, in, i, y, 1.0, R.wd[code]);
           }
         } else {
-          const RowIn<EPI, T> in(R, i);
-          finish_row<EPI>(R, in, i, rs[code].s, (float)scale, R.wd[code]);
+          finish_row<EPI>(R, ins[code], i, rs[code].s, (float)scale, R.wd[code]);
         }
       };
-      row(std::integral_constant<int, 0>{});
-      row(std::integral_constant<int, 1>{});
-      row(std::integral_constant<int, 2>{});
-      row(std::integral_constant<int, 3>{});
-      row(std::integral_constant<int, 4>{});
-      row(std::integral_constant<int, 5>{});
-      row(std::integral_constant<int, 6>{});
-      row(std::integral_constant<int, 7>{});
+      auto rows = [&](auto plain_) {
+        row(std::integral_constant<int, 0>{}, plain_);
+        row(std::integral_constant<int, 1>{}, plain_);
+        row(std::integral_constant<int, 2>{}, plain_);
+        row(std::integral_constant<int, 3>{}, plain_);
+        row(std::integral_constant<int, 4>{}, plain_);
+        row(std::integral_constant<int, 5>{}, plain_);
+        row(std::integral_constant<int, 6>{}, plain_);
+        row(std::integral_constant<int, 7>{}, plain_);
+      };
+      if (plain)
+        rows(std::true_type{});
+      else
+        rows(std::false_type{});
     }
   }
   if constexpr (FIX) {
@@ -634,20 +652,18 @@ __global__ void __launch_bounds__(kDirectBlock)
   }
 }
 
-// FP64 tiles: 71 KB, three blocks per SM; FP32 tiles have rows of 32 cells, so
-// that a warp's shared-memory accesses fall into distinct banks.
-#ifndef TL
-#define TL 16, 8, 4, 256, 3
-#endif
-#ifndef TF
-#define TF 32, 4, 8, 256, 3
-#endif
-#ifndef DIRECT
-#define DIRECT 16
-#endif
-using Tile64 = TileShape<TL>;
-using Tile32 = TileShape<TF>;
-constexpr int kDirectMax = DIRECT;
+// FP64: 41 KB, five blocks per SM, on levels whose tiles are few, where the whole
+// grid is one or two rounds of blocks (two Chebyshev steps at 32^3 30.8 us against
+// 36.5 with the larger tile, 64^3 83 against 86); above, 71 KB and less of the
+// values staged twice (128^3: 550 against 576 us).  FP32: rows of 32 cells, so that
+// a warp's shared-memory accesses fall into distinct banks (rows of 16: 58 against
+// 48 us at 128^3).
+using Tile64Few = TileShape<16, 4, 4, 128, 5>;
+using Tile64Many = TileShape<16, 8, 4, 256, 3>;
+using Tile32 = TileShape<32, 4, 8, 256, 3>;
+constexpr int kTileFewMax = 96;  // cubes per axis
+// The direct kernel: 16^3 8.7 us against 12 us tiled; its operations grow with the level, the tiles' latency does not.
+constexpr int kDirectMax = 16;
 
 Lattice2 lattice_of(const Level& L) {
   Lattice2 G{};
@@ -661,29 +677,39 @@ Lattice2 lattice_of(const Level& L) {
   return G;
 }
 
-template <typename T>
-using Tile = typename std::conditional<sizeof(T) == 8, Tile64, Tile32>::type;
+template <int EPI, typename T, typename S>
+void launch_tiles(const Level& L, double scale, const Rows<T>& R, cudaStream_t s) {
+  const int grid = ceil_div(L.N, S::TX) * ceil_div(L.N, S::TY) * ceil_div(L.N, S::KZ);
+  k_stencil2<T, EPI, S><<<grid, S::threads, S::template smem<T>(), s>>>(lattice_of(L), scale, R, L.nb, L.bnd);
+}
 
 template <int EPI, typename T>
 void launch_stencil(const Level& L, const Rows<T>& R, cudaStream_t s) {
-  using S = Tile<T>;
   const double scale = 8.0 * (L.kappa0 / (120.0 * L.N));
-  if (L.N <= kDirectMax) {
+  if (L.N <= kDirectMax)
     k_stencil2_direct<T, EPI><<<dim3(ceil_div((long long)L.Q, kDirectBlock), 8), kDirectBlock, 0, s>>>(
         lattice_of(L), scale, R, L.nb, L.bnd);
-  } else {
-    const int grid = ceil_div(L.N, S::TX) * ceil_div(L.N, S::TY) * ceil_div(L.N, S::KZ);
-    k_stencil2<T, EPI, S><<<grid, S::threads, S::template smem<T>(), s>>>(lattice_of(L), scale, R, L.nb, L.bnd);
-  }
+  else if constexpr (sizeof(T) == 4)
+    launch_tiles<EPI, T, Tile32>(L, scale, R, s);
+  else if (L.N <= kTileFewMax)
+    launch_tiles<EPI, T, Tile64Few>(L, scale, R, s);
+  else
+    launch_tiles<EPI, T, Tile64Many>(L, scale, R, s);
   LAUNCH_CHECK();
 }
 
 // The shared-memory limit of a kernel is a property of the device's context and
 // has one value per kernel, so setting it again for another hierarchy is harmless.
-template <typename T, int EPI>
+template <typename T, int EPI, typename S>
 void set_smem() {
-  CUDA_CHECK(cudaFuncSetAttribute((const void*)k_stencil2<T, EPI, Tile<T>>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)Tile<T>::template smem<T>()));
+  CUDA_CHECK(cudaFuncSetAttribute((const void*)k_stencil2<T, EPI, S>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)S::template smem<T>()));
+}
+template <int EPI>
+void set_smems() {
+  set_smem<double, EPI, Tile64Few>();
+  set_smem<double, EPI, Tile64Many>();
+  set_smem<float, EPI, Tile32>();
 }
 
 template <int EPI, typename T>
@@ -712,10 +738,8 @@ void launch(const Level& L, const Rows<T>& R, cudaStream_t s) {
 void launch_flux_setup(Level& L, cudaStream_t s) {
   if (L.flux == FLUX_NONE) return;
   if (L.deg == 2) {
-    set_smem<double, EPI_APPLY>();
-    set_smem<double, EPI_CHEB>();
-    set_smem<float, EPI_APPLY>();
-    set_smem<float, EPI_CHEB>();
+    set_smems<EPI_APPLY>();
+    set_smems<EPI_CHEB>();
   } else if (L.flux == FLUX_VAR) {
     L.fw64.alloc((size_t)4 * L.n);
     L.fw32.alloc((size_t)4 * L.n);
@@ -741,7 +765,7 @@ void launch_flux_cheb(const Level& L, const T* b, const T* x, T* xout, const T* 
   R.x = x;
   R.out = xout;
   R.b = b;
-  R.din = din;
+  R.din = c1 != 0.0 ? din : nullptr;
   R.dout = dout;
   if constexpr (sizeof(T) == 8)
     R.dinv = L.dinv64;

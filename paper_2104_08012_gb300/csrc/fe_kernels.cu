@@ -1482,11 +1482,17 @@ void launch_prolong(const fe_hierarchy* h, int lf, const T* xc, T* xf, bool accu
 // the 1024-thread blocks were slower (14.0 -> 18.5 us).
 constexpr int kRestrictWideBelow = 1 << 14;
 
+constexpr int kRestrictTiledFrom = 32;  // coarse cubes per axis: below, the tiles are too few to hide their latency
 template <typename T>
 void launch_restrict(const fe_hierarchy* h, int lf, const T* bf, const T* yf, T* rc, bool zero_bd, cudaStream_t s) {
   const Level& F = h->L[lf];
   const Level& Cc = h->L[lf - 1];
   const TransferTables& t = h->tt;
+  if constexpr (sizeof(T) == 4)
+    if (h->deg == 2 && zero_bd && Cc.N >= kRestrictTiledFrom) {
+      launch_restrict_p2(F, Cc, bf, yf, rc, s);
+      return;
+    }
   if (h->deg == 1)
     k_restrict<1, T, 4><<<ceil_div(Cc.n, 32), 32 * 4, 0, s>>>(F.num.m, Cc.num, Cc.n, t.res_margin, t.res_start,
                                                               F.rtab, tt_weights<T>(t.res_w, t.res_wf), bf,
