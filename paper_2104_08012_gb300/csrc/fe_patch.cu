@@ -211,22 +211,81 @@ __global__ void __launch_bounds__(kBlock) k_patch_apply_df(int P, int Pp, int Pp
   }
 }
 
-// P3 (65 slots, packed inverse patch-major [P][2145]): one warp per patch.  Each
-// lane owns rows lane, lane + 32 and lane + 64 (< 65); r = b - y is split into
-// float pairs with the warp's largest exponent and shared through shared
-// memory; z_i = sum_j (A_p^-1)_ij r_j reads the packed upper triangle, whose
-// 17 KB per patch the warp streams through L1.  T = double: float-pair
-// arithmetic; T = float: FP32 with the FP32 copy.
+// P3 (65 slots, packed inverse patch-major [P][2145]): one warp per patch.  r = b
+// - y is split into float pairs with the warp's largest exponent (T = double) or
+// taken as it is (T = float, with the FP32 copy of the inverse) and shared through
+// shared memory.  Lane l owns the columns l and l + 32: row i of the packed upper
+// triangle is read once, by coalesced loads, and each entry a_ij serves both z_j
+// (+= a_ij r_i, in the lane's own sums) and z_i (+= a_ij r_j, a partial sum per lane
+// and row, 32 rows at a time, which one exchange of halves over the warp turns into
+// the row sums of 32 lanes); column 64 is read by rows.  The first form gave every
+// lane whole rows: two loads per entry, half of them scattered, 65 steps for row 64
+// on one lane, and one dependent chain of 195 float-pair additions per warp: 53 us
+// at 8^3 and 16^3, where there are too few patches to hide it, and 115 us at 32^3,
+// whose 617 MB take 91 us at the copy bandwidth.
 constexpr int NS3 = 65, NP3 = NS3 * (NS3 + 1) / 2, kWarpsP3 = 4;
+constexpr int kRing = 8;  // rows of the triangle in flight per warp (cp.async; 6 blocks per SM measured best with 8)
+
 template <typename T>
-__global__ void __launch_bounds__(32 * kWarpsP3) k_patch_apply_p3(int P, const int* __restrict__ pdof,
+struct PatchNum;  // the arithmetic of the product
+template <>
+struct PatchNum<double> {
+  using V = fe_df::DF;
+  using E = float2;
+  static __device__ __forceinline__ V entry(E e) { return V(e.x, e.y); }
+  static __device__ __forceinline__ V zero() { return V(0.0f, 0.0f); }
+  static __device__ __forceinline__ V shfl_xor(V v, int m) {
+    return V(__shfl_xor_sync(0xffffffffu, v.hi, m), __shfl_xor_sync(0xffffffffu, v.lo, m));
+  }
+  static __device__ __forceinline__ V pick(bool c, V a, V b) { return V(c ? a.hi : b.hi, c ? a.lo : b.lo); }
+  static __device__ __forceinline__ V mul(V a, V b) { return fe_df::mul(a, b); }
+  static __device__ __forceinline__ V add(V a, V b) { return a + b; }
+};
+template <>
+struct PatchNum<float> {
+  using V = float;
+  using E = float;
+  static __device__ __forceinline__ V entry(E e) { return e; }
+  static __device__ __forceinline__ V zero() { return 0.0f; }
+  static __device__ __forceinline__ V shfl_xor(V v, int m) { return __shfl_xor_sync(0xffffffffu, v, m); }
+  static __device__ __forceinline__ V pick(bool c, V a, V b) { return c ? a : b; }
+  static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
+  static __device__ __forceinline__ V add(V a, V b) { return a + b; }
+};
+
+__device__ __forceinline__ void cp_async_entry(float2* smem, const float2* gmem) {
+  const unsigned int sa = (unsigned int)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(sa), "l"(gmem) : "memory");
+}
+__device__ __forceinline__ void cp_async_entry(float* smem, const float* gmem) {
+  const unsigned int sa = (unsigned int)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(sa), "l"(gmem) : "memory");
+}
+
+// s[k] of every lane, k = 0 .. 31 -> lane l returns the sum over the lanes of s[l].
+template <typename N, typename V>
+__device__ __forceinline__ V sum_transposed(V (&s)[32], int lane) {
+#pragma unroll
+  for (int h = 16; h > 0; h >>= 1) {
+    const bool up = (lane & h) != 0;
+#pragma unroll
+    for (int k = 0; k < h; ++k) s[k] = N::add(N::pick(up, s[k + h], s[k]), N::shfl_xor(N::pick(up, s[k], s[k + h]), h));
+  }
+  return s[0];
+}
+
+template <typename T>
+__global__ void __launch_bounds__(32 * kWarpsP3, 6) k_patch_apply_p3(int P, const int* __restrict__ pdof,
                                                                   const float2* __restrict__ pinvdf,
                                                                   const float* __restrict__ pinv32,
                                                                   const T* __restrict__ b, const T* __restrict__ y,
                                                                   T* __restrict__ z, int nb,
                                                                   const int* __restrict__ bnd) {
   using namespace fe_df;
-  __shared__ float2 rs[kWarpsP3][NS3];
+  using N = PatchNum<T>;
+  using V = typename N::V;
+  __shared__ V rs[kWarpsP3][NS3];
+  __shared__ typename N::E ring[kWarpsP3 * kRing * 64];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int v = blockIdx.x * kWarpsP3 + wib;
   // Dirichlet rows: z = r (a grid-stride loop over all threads)
@@ -249,44 +308,89 @@ __global__ void __launch_bounds__(32 * kWarpsP3) k_patch_apply_p3(int P, const i
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
   }
+  V r[3];
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     const int sl = lane + 32 * q;
-    if (sl < NS3) {
-      if constexpr (sizeof(T) == 8) {
-        DF d = split_scaled((double)rr[q], emax);
-        if (q == 0 && lane == 0 && emax == 0x7FF) d = DF(__int_as_float(0x7fc00000), 0.0f);
-        rs[wib][sl] = make_float2(d.hi, d.lo);
-      } else {
-        rs[wib][sl] = make_float2((float)rr[q], 0.0f);
-      }
+    if constexpr (sizeof(T) == 8) {
+      r[q] = split_scaled((double)rr[q], emax);
+      if (q == 0 && lane == 0 && emax == 0x7FF) r[q] = DF(__int_as_float(0x7fc00000), 0.0f);
+    } else {
+      r[q] = rr[q];
     }
+    if (sl < NS3) rs[wib][sl] = r[q];
   }
   __syncwarp();
-  const size_t base = (size_t)v * NP3;
-#pragma unroll
-  for (int q = 0; q < 3; ++q) {
-    const int i = lane + 32 * q;
-    if (i >= NS3) continue;
-    if constexpr (sizeof(T) == 8) {
-      DF acc(0.0f);
-#pragma unroll 5  // loads issued ahead of the dependent float-pair chain: 3.5% faster than a rolled loop
-      for (int j = 0; j < NS3; ++j) {
-        const int lo = min(i, j), hi = max(i, j);
-        const float2 e = __ldg(pinvdf + base + NS3 * lo - lo * (lo - 1) / 2 + (hi - lo));
-        const float2 r = rs[wib][j];
-        acc = acc + mul(DF(e.x, e.y), DF(r.x, r.y));
+  const typename N::E* a;
+  if constexpr (sizeof(T) == 8)
+    a = pinvdf + (size_t)v * NP3;
+  else
+    a = pinv32 + (size_t)v * NP3;
+  auto at = [&](int i, int j) { return N::entry(__ldg(a + NS3 * i - i * (i - 1) / 2 + (j - i))); };
+  // rows 0 .. 31 (columns lane and lane + 32) and 32 .. 63 (column lane + 32) through the lane's ring of kRing rows
+  using E = typename N::E;
+  auto* slot = ring + (size_t)wib * kRing * 64 + lane;
+  auto issue = [&](int i) {
+    if (i < 64) {
+      const E* row = a + NS3 * i - i * (i - 1) / 2 - i;
+      E* dst = slot + (i % kRing) * 64;
+      if (i < 32) {
+        if (lane >= i) cp_async_entry(dst, row + lane);
+        cp_async_entry(dst + 32, row + lane + 32);
+      } else if (lane + 32 >= i) {
+        cp_async_entry(dst + 32, row + lane + 32);
       }
-      if (dof[q] >= 0) atomicAdd(z + dof[q], (T)(widen_scaled(acc.hi, emax) + widen_scaled(acc.lo, emax)));
-    } else {
-      float acc = 0.0f;
-      for (int j = 0; j < NS3; ++j) {
-        const int lo = min(i, j), hi = max(i, j);
-        acc += __ldg(pinv32 + base + NS3 * lo - lo * (lo - 1) / 2 + (hi - lo)) * rs[wib][j].x;
-      }
-      if (dof[q] >= 0) atomicAdd(z + dof[q], (T)acc);
     }
+    cp_async_commit();
+  };
+#pragma unroll
+  for (int i = 0; i < kRing - 1; ++i) issue(i);
+  V z0 = N::zero(), z1 = N::zero();  // a_ij r_i of the lane's columns
+  V zi[2];
+  {
+    V s[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+      issue(i + kRing - 1);
+      cp_async_wait<kRing - 1>();
+      const V ri = rs[wib][i];
+      const V e0 = lane >= i ? N::entry(slot[(i % kRing) * 64]) : N::zero(), e1 = N::entry(slot[(i % kRing) * 64 + 32]);
+      s[i] = N::add(N::mul(e0, r[0]), N::mul(e1, r[1]));
+      z0 = N::add(z0, N::mul(N::pick(lane == i, N::zero(), e0), ri));
+      z1 = N::add(z1, N::mul(e1, ri));
+    }
+    zi[0] = sum_transposed<N>(s, lane);
   }
+  {
+    V s[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+      issue(i + 32 + kRing - 1);
+      cp_async_wait<kRing - 1>();
+      const V e = lane >= i ? N::entry(slot[((i + 32) % kRing) * 64 + 32]) : N::zero();
+      s[i] = N::mul(e, r[1]);
+      z1 = N::add(z1, N::mul(N::pick(lane == i, N::zero(), e), rs[wib][i + 32]));
+    }
+    zi[1] = sum_transposed<N>(s, lane);
+  }
+  // column 64: a_(i,64) for the lane's two rows, and its own row
+  const V c0 = at(lane, 64), c1 = at(lane + 32, 64), r64 = rs[wib][64];
+  z0 = N::add(N::add(z0, zi[0]), N::mul(c0, r64));
+  z1 = N::add(N::add(z1, zi[1]), N::mul(c1, r64));
+  V z2 = N::add(N::mul(c0, r[0]), N::mul(c1, r[1]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) z2 = N::add(z2, N::shfl_xor(z2, o));
+  z2 = N::add(z2, N::mul(at(64, 64), r64));
+  auto put = [&](int q, V val) {
+    if (dof[q] < 0) return;
+    if constexpr (sizeof(T) == 8)
+      atomicAdd(z + dof[q], widen_scaled(val.hi, emax) + widen_scaled(val.lo, emax));
+    else
+      atomicAdd(z + dof[q], val);
+  };
+  put(0, z0);
+  put(1, z1);
+  if (lane == 0) put(2, z2);
 }
 
 // Chebyshev step with a preconditioned residual z: d = c1 d + c2 z, x += d
