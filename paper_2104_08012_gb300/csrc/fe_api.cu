@@ -454,6 +454,8 @@ void apply_enqueue(const fe_hierarchy* h, int level, const void* x, void* y, int
   if (L.deg == 3) {  // P3: element through the gradient at the P2 nodes in FP64, float pairs (default), FP32 or bf16
     if (dtype == FE_F64 && h->f64_mode == FE_F64_NATIVE)
       launch_apply64(L, (const double*)x, (double*)y, s);
+    else if (dtype == FE_F64 && L.uniform)
+      launch_apply64_p3(L, (const double*)x, (double*)y, s);
     else if (dtype == FE_F64)
       launch_apply64_df3(L, (const double*)x, (double*)y, s);
     else if (dtype == FE_F32)

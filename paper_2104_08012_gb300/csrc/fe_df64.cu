@@ -439,11 +439,11 @@ __global__ void __launch_bounds__(kBlock, 2) k_apply_df2(int P, int Cs, const in
   }
 }
 
-// P3, one tet per thread (persistent grid-stride loop): the element through
-// the gradient at the P2 nodes (fe_p3.cuh) in float pairs, on the geometric
-// factors kappa G / 161280 split once per tet; dofs split and contributions
-// widened per tet as in k_apply_df.  UNI: geo is L.cdf (G = c M per cell).
-template <bool UNI>
+// P3 on levels whose G is not c M in every cell (or with FE_GEOMETRY_PER_CELL;
+// fe_p3int.cu otherwise), one tet per thread (persistent grid-stride loop): the
+// element through the gradient at the P2 nodes (fe_p3.cuh) in float pairs, on the
+// geometric factors kappa G / 161280 split once per tet; dofs split and
+// contributions widened per tet as in k_apply_df.
 __global__ void __launch_bounds__(kBlockP3, 2) k_apply_df3(int C, int Cs, const int* __restrict__ map,
                                                            const float2* __restrict__ geo,
                                                            const double* __restrict__ x, double* __restrict__ y,
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(kBlockP3, 2) k_apply_df3(int C, int Cs, const 
     }
     DF g[6];
 #pragma unroll
-    for (int a = 0; a < (UNI ? 1 : 6); ++a) {
+    for (int a = 0; a < 6; ++a) {
       const float2 v = __ldg(geo + (size_t)a * Cs + c);
       g[a] = DF(v.x, v.y);
     }
@@ -469,7 +469,7 @@ __global__ void __launch_bounds__(kBlockP3, 2) k_apply_df3(int C, int Cs, const 
 #pragma unroll
     for (int j = 0; j < ND; ++j) u[j] = split_scaled(xv[j], emax);
     if (emax == 0x7FF) u[0] = DF(__int_as_float(0x7fc00000), 0.0f);  // propagate NaN/inf dofs
-    fe_p3::p3_element_grad<fe_p3::DFOps, UNI>(u, g, out);
+    fe_p3::p3_element_grad<fe_p3::DFOps>(u, g, out);
 #pragma unroll
     for (int j = 0; j < ND; ++j) {
       const int m = __ldg(map + (size_t)j * Cs + c);
@@ -740,12 +740,9 @@ void launch_apply64_df3(const Level& L, const double* x, double* y, cudaStream_t
   FE_REQUIRE(L.deg == 3, FE_ERR_UNSUPPORTED, "the float-pair P3 kernel needs a degree-3 level");
   CUDA_CHECK(cudaMemsetAsync(y, 0, sizeof(double) * (size_t)L.n, s));
   static int g = 0;
-  if (!g) g = resident_grid(k_apply_df3<true>, kBlockP3, 1 << 30);
+  if (!g) g = resident_grid(k_apply_df3, kBlockP3, 1 << 30);
   const int grid = std::min(g, ceil_div(std::max(L.C, L.nb), kBlockP3));
-  if (L.uniform)
-    k_apply_df3<true><<<grid, kBlockP3, 0, s>>>(L.C, L.Cs, L.map, L.cdf, x, y, L.nb, L.bnd);
-  else
-    k_apply_df3<false><<<grid, kBlockP3, 0, s>>>(L.C, L.Cs, L.map, L.geodf, x, y, L.nb, L.bnd);
+  k_apply_df3<<<grid, kBlockP3, 0, s>>>(L.C, L.Cs, L.map, L.geodf, x, y, L.nb, L.bnd);
   LAUNCH_CHECK();
 }
 

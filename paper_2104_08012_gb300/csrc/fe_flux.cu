@@ -22,10 +22,13 @@
 #include <type_traits>
 #include <utility>
 
+#include "fe_fixed.cuh"
 #include "fe_internal.cuh"
 #include "fe_kuhn.h"
 
 namespace {
+
+using namespace fe_fixed;
 
 inline int ceil_div(long long a, int b) { return (int)((a + b - 1) / b); }
 
@@ -171,31 +174,7 @@ __global__ void k_edge_weights(int N, int n, const double* __restrict__ geo22, d
   w32[3 * m + i] = (float)dg;
 }
 
-// FP64 values as 64-bit integers of a common scale: with E the largest biased
-// exponent of a tile, |x| is cut into windows of TB + 1 bits below 2^(E - 1022);
-// window `pass` of x is returned with x's sign.  Sums of such integers wrap
-// modulo 2^64 and are exact as long as the final row fits.
-template <int TB>
-__device__ __forceinline__ long long fixed_window(unsigned int hi, unsigned int lo, int E, int pass) {
-  const int e = (int)((hi >> 20) & 0x7FFu);
-  if (e == 0 || e == 0x7FF) return 0;  // zero, subnormal (flushed), or not finite (handled by the caller)
-  const unsigned long long m = ((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
-  const unsigned long long M = m << (TB - 52);
-  const int r = (E - e) - pass * (TB + 1);
-  unsigned long long w;
-  if (r >= 0)
-    w = r < 64 ? M >> r : 0ull;
-  else
-    w = r > -64 ? (M << -r) & ((1ull << (TB + 1)) - 1) : 0ull;
-  return (hi >> 31) ? -(long long)w : (long long)w;
-}
-
-constexpr int kTop = 59;    // top bit of a staged value: |x| < 2^60 units
 constexpr int kRange = 15;  // bits by which a cell may lie below its tile's largest value in one pass
-
-__device__ __forceinline__ double pow2(int e) {  // 2^e, -1022 <= e <= 1023
-  return __hiloint2double((e + 1023) << 20, 0);
-}
 
 // ------------------------------------------- P2, one coefficient: stencils ---
 // With one c on the level the rows of A are eight constant stencils of 19 to 51
@@ -215,11 +194,6 @@ __device__ __forceinline__ double pow2(int e) {  // 2^e, -1022 <= e <= 1023
 // form 180.  What the integers cut off is below 2^-59 of the tile's largest
 // value; the cells that lie more than kRange bits below it are formed again from
 // the windows of the next lower bits, and the parts are added in FP64.
-struct Pair32 {  // hi 2^30 + lo
-  int hi, lo;
-};
-__device__ __forceinline__ Pair32 operator+(Pair32 a, Pair32 b) { return {a.hi + b.hi, a.lo + b.lo}; }
-
 template <typename V>
 struct RowSum;
 template <>
@@ -239,18 +213,7 @@ struct RowSum<double> {
   }
 };
 template <>
-struct RowSum<Pair32> {
-  long long hi = 0, lo = 0;
-  // one 32 x 32 + 64 bit instruction per word (left to itself the compiler turns the small coefficients into sign
-  // extensions, shifts and carried additions, three instructions each)
-  static __device__ __forceinline__ void mad(long long& a, int k, int v) {
-    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(a) : "r"(v), "r"(k));
-  }
-  template <typename... A>
-  __device__ __forceinline__ void add(int k, A... v) {  // sums of at most two staged values
-    ((mad(hi, k, v.hi), mad(lo, k, v.lo)), ...);
-  }
-};
+struct RowSum<Pair32> : PairSum {};
 
 // The row of the lattice point of parity code CODE in units of 8 c; at(x, y, z):
 // the value at that offset from the vertex of its cell, components in [-2, 2].
@@ -375,17 +338,6 @@ __device__ __forceinline__ void stencil_rows(RowSum<V> (&r)[8], At at, std::inte
   (point(std::integral_constant<int, I>{}, std::true_type{}), ...);
 }
 
-// x as hi 2^30 + lo of the scale E, both with the sign of x (the first window of
-// fixed_window in 30-bit halves).  A shift beyond 63 (zeros, far smaller values
-// and, with e > E, values that are not finite) gives 0; needs E >= 64.
-__device__ __forceinline__ Pair32 fixed_pair(double x, int E) {
-  const unsigned int xh = (unsigned int)__double2hiint(x), xl = (unsigned int)__double2loint(x);
-  const unsigned int r = min((unsigned int)(E - (int)((xh >> 20) & 0x7FFu)), 63u);
-  const unsigned long long m = ((unsigned long long)((xh & 0xFFFFFu) | 0x100000u) << 32) | xl;
-  const unsigned long long w = (m << (kTop - 52)) >> r;
-  const int sg = 1 | ((int)xh >> 31);
-  return {sg * (int)(w >> 30), sg * (int)((unsigned int)w & 0x3FFFFFFFu)};
-}
 // any window, any E
 __device__ __noinline__ Pair32 fixed_pair_window(double x, int E, int pass) {
   const unsigned int xh = (unsigned int)__double2hiint(x), xl = (unsigned int)__double2loint(x);

@@ -439,6 +439,8 @@ void launch_split_pairs(const Level& L, const double* x, cudaStream_t s);
 void launch_apply64_cube_df(const Level& L, const double* x, double* y, cudaStream_t s);
 void launch_apply64_df2(const Level& L, const double* x, double* y, cudaStream_t s);
 void launch_apply64_df3(const Level& L, const double* x, double* y, cudaStream_t s);
+// P3 on levels with L.uniform, by the integer element matrix (fe_p3int.cu)
+void launch_apply64_p3(const Level& L, const double* x, double* y, cudaStream_t s);
 void upload_p3_mass_table(const float* m3i);
 // The same operator kernels with the Chebyshev update fused (y = A x, then
 // d = c1 d + c2 D^-1 (b - y), x += d per dof, in one launch).

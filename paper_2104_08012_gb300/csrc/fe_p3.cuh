@@ -59,6 +59,54 @@ __host__ __device__ constexpr int dphi8(int i, int v, int n) {
   return 54 * node_l(n, o[0]) * node_l(n, o[1]);
 }
 
+// The integer element matrix of every Kuhn tet: with G = c M, M diagonal along
+// the tet's path of edges 01, 12, 23, A_K = 48 c K for c = kappa h / 161280 and
+//   K_ij = 3360 int_ref sum_p d_p phi_i d_p phi_j,  d_p = d/dlambda_(p+1) - d/dlambda_p,
+// from the tables above (64 * 2520 = 48 * 3360).  362 nonzeros, rows of |K| summing
+// to at most 15768.
+struct KuhnP3 {
+  int k[20][20];
+};
+__host__ __device__ constexpr int p2_mass_entry(int n, int m) {
+  if (n < 4 && m < 4) return n == m ? 6 : 1;
+  if (n >= 4 && m >= 4) return n == m ? 32 : n - 4 + m - 4 == 5 ? 8 : 16;
+  const int v = n < 4 ? n : m, e = (n < 4 ? m : n) - 4;
+  return ea(e) == v || eb(e) == v ? -4 : -6;
+}
+__host__ __device__ constexpr KuhnP3 make_kuhn_p3() {
+  KuhnP3 r{};
+  for (int p = 0; p < 3; ++p) {
+    int d[20][10] = {};
+    for (int i = 0; i < 20; ++i)
+      for (int n = 0; n < 10; ++n) d[i][n] = dphi8(i, p + 1, n) - dphi8(i, p, n);
+    for (int j = 0; j < 20; ++j) {
+      int w[10] = {};
+      for (int n = 0; n < 10; ++n)
+        for (int m = 0; m < 10; ++m) w[n] += p2_mass_entry(n, m) * d[j][m];
+      for (int i = 0; i < 20; ++i)
+        for (int n = 0; n < 10; ++n) r.k[i][j] += d[i][n] * w[n];
+    }
+  }
+  for (int i = 0; i < 20; ++i)
+    for (int j = 0; j < 20; ++j) r.k[i][j] = r.k[i][j] % 48 == 0 ? r.k[i][j] / 48 : 1 << 30;
+  return r;
+}
+constexpr KuhnP3 kKuhnP3 = make_kuhn_p3();
+__host__ __device__ constexpr bool kuhn_p3_ok() {
+  for (int i = 0; i < 20; ++i) {
+    int sum = 0, mag = 0;
+    for (int j = 0; j < 20; ++j) {
+      const int k = kKuhnP3.k[i][j];
+      if (k != kKuhnP3.k[j][i]) return false;
+      sum += k;
+      mag += k < 0 ? -k : k;
+    }
+    if (sum != 0 || mag > 15768) return false;
+  }
+  return true;
+}
+static_assert(kuhn_p3_ok(), "P3 Kuhn stiffness: integer, symmetric, zero row sums, bounded rows");
+
 // ------------------------------------------------------------ arithmetic
 template <typename T>
 struct PlainOps {

@@ -1,5 +1,6 @@
 """The operator in flux and stencil form (P1 on any coefficient, P2 on one coefficient per level): its tile edges,
-remainders, small-level kernel, value ranges and non-finite entries, and the Chebyshev step in the same launch."""
+remainders, small-level kernel, value ranges and non-finite entries, and the Chebyshev step in the same launch; the P3
+operator by integer sums; the FP32 P2 restriction from staged tiles."""
 import numpy as np
 import pytest
 
@@ -120,3 +121,34 @@ def test_chebyshev_steps_in_one_launch(fe, k, N0, coef, steps, f32):
         h.smooth(dt(b, d), x, level=1, steps=steps, dtype=fe.FE_F32 if f32 else fe.FE_F64)
         got = x.double().cpu().numpy()
         assert np.abs(got - ref).max() <= (1e-5 if f32 else 1e-12) * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("scale", [1e-300, 1e-200, 1e-8, 1.0, 1e200, 1e300])
+def test_p3_integer_element_value_range(fe, scale):
+    """P3 rows within 1e-14 of |A| |x| from 1e-300 to 1e300 (exact integer sums, one rounding per contribution, up to 24
+    contributions per row; 2 N = 6 extra ulps for the integers' cut below 2^-59), exact zeros, NaN dofs propagate."""
+    with fe.Hierarchy(3, 0, 3) as h:
+        kappa = np.exp(I.random_vector(h.n_cells(), 5))
+        h.set_coefficient(dt(kappa))
+        L = O.Level(3, 3, kappa)
+        x = I.random_vector(L.n, 77) * scale
+        x[::7] = 0.0
+        assert np.all(np.abs(apply(fe, h, x) - L.A @ x) <= 1e-14 * np.maximum(abs(L.A) @ np.abs(x), 1e-307))
+        assert not apply(fe, h, np.zeros(L.n)).any()
+        i = np.nonzero(~L.space.boundary)[0][7]
+        x[i] = np.nan
+        row = np.abs(L.A[i].toarray()[0])
+        assert np.isnan(apply(fe, h, x)[row > 1e-12 * row.max()]).all()
+
+
+@pytest.mark.parametrize("N0", [4, 5])
+def test_fp32_cycle_with_tiled_restriction_matches_fp64(fe, N0):
+    """The FP32 V-cycle restricts 64^3 (and 80^3: ragged tiles) with staged tiles; it equals the FP64 cycle to FP32
+    rounding (5e-6 of the largest entry, as every FP32 cycle here)."""
+    with fe.Hierarchy(N0, 4, 2) as h:
+        b = I.random_vector(h.n_dofs(), 3)
+        b[h.boundary_mask()] = 0.0
+        x, x32 = torch.empty(len(b), dtype=torch.float64, device=DEV), torch.empty(len(b), device=DEV)
+        h.vcycle(dt(b), x)
+        h.vcycle(dt(b, torch.float32), x32, dtype=fe.FE_F32)
+        assert (x32.double() - x).abs().max() <= 5e-6 * x.abs().max()
