@@ -47,6 +47,13 @@ struct BLevel {
   const double* detj;
   const int* bnd;
   double *b, *x, *y, *d, *w;
+  // P1 on Kuhn tets: rows of A from the edge weights fw ([4][n]: x, y, z edges, diagonal) or, without them, the one
+  // coefficient c1d (rows = 1; see fe_flux.cu).  No apply phase of a smoothing step then: the dof phase forms A x
+  // itself, from one vector to another (x -> y -> x in turn).
+  int rows;
+  const double* fw;
+  double c1d;
+  float2* xs;  // P2, one c per tet: x as float pairs, written with x for the operator (null: split per tet)
   double inv_theta, c1, c2;  // two Chebyshev steps: d0 = inv_theta D^-1 r0; d1 = c1 d0 + c2 D^-1 r1
 };
 
@@ -67,6 +74,7 @@ struct BProb {
   const double* LinvT;
   double *t0, *t1;
   double *xs, *p, *q, *rhs;  // solution, CG direction, A p, load vector
+  float2* ps;                // p as float pairs (with lev[].xs)
   const double* f;           // nodal right-hand side
 };
 
@@ -80,7 +88,9 @@ struct GridBar {
   int abort, pad;
 };
 
-enum Range { R_CELL = 0, R_DOF = 1, R_BND = 2, R_ROW = 3, R_KINDS = 4 };
+// R_CELL, R_BND: cells and boundary dofs of the problems whose operator runs over cells; R_AROW: dofs of those whose
+// operator runs over rows; R_MASS, R_RBND: every problem's cells and boundary dofs (load vector)
+enum Range { R_CELL = 0, R_DOF = 1, R_BND = 2, R_ROW = 3, R_AROW = 4, R_MASS = 5, R_RBND = 6, R_KINDS = 7 };
 
 struct Work {
   const int4* items;  // (problem, begin, end, level)
@@ -180,6 +190,26 @@ enum DofOp {
   OP_UPDATE_P      // beta = acc_rz/rz; p = z + beta p; q = 0
 };
 
+// Row i of A x for a P1 level with `rows` (boundary rows: identity).
+__device__ __forceinline__ double p1_row(const BLevel& L, const double* x, int i) {
+  const int N = L.N, n1 = N + 1, sz = n1 * n1, n = L.n;
+  const int X = i % n1, q = i / n1, Y = q % n1, Z = q / n1;
+  const double xi = x[i];
+  if (X == 0 || Y == 0 || Z == 0 || X == N || Y == N || Z == N) return xi;
+  const double xl = X > 1 ? x[i - 1] : 0.0, xr = X < N - 1 ? x[i + 1] : 0.0;
+  const double yl = Y > 1 ? x[i - n1] : 0.0, yr = Y < N - 1 ? x[i + n1] : 0.0;
+  const double zl = Z > 1 ? x[i - sz] : 0.0, zr = Z < N - 1 ? x[i + sz] : 0.0;
+  const double* w = L.fw;
+  if (!w) return L.c1d * fma(6.0, xi, -(((xl + xr) + (yl + yr)) + (zl + zr)));
+  double y = __ldg(w + 3 * (size_t)n + i) * xi;
+  y = fma(-__ldg(w + i - 1), xl, y);
+  y = fma(-__ldg(w + i), xr, y);
+  y = fma(-__ldg(w + n + i - n1), yl, y);
+  y = fma(-__ldg(w + n + i), yr, y);
+  y = fma(-__ldg(w + 2 * (size_t)n + i - sz), zl, y);
+  return fma(-__ldg(w + 2 * (size_t)n + i), zr, y);
+}
+
 // Prolongation of the coarse x at fine point i through the level's index
 // table (each entry's coarse dof an affine form of the base cube).
 template <int DEG>
@@ -253,32 +283,55 @@ __device__ void dof_phase(const Params& A, int level, int op, bool all_problems)
         } break;
         case OP_PRE0: {
           const double v = L.inv_theta * L.dinv[i] * L.b[i];
-          L.d[i] = v;
           L.x[i] = v;
-          L.y[i] = 0.0;
+          if (!L.rows) {
+            L.d[i] = v;
+            L.y[i] = 0.0;
+            if (L.xs) L.xs[i] = fe_df::split_pair(v);
+          }
         } break;
-        case OP_CHEB1_PRE: {
-          const double v = L.c1 * L.d[i] + L.c2 * L.dinv[i] * (L.b[i] - L.y[i]);
-          L.d[i] = v;
-          L.x[i] += v;
-          L.w[i] = 0.0;
-        } break;
+        case OP_CHEB1_PRE:
+          if (L.rows) {  // x -> y
+            const double x = L.x[i];
+            L.y[i] = x + (L.c1 * x + L.c2 * L.dinv[i] * (L.b[i] - p1_row(L, L.x, i)));
+          } else {
+            const double v = L.c1 * L.d[i] + L.c2 * L.dinv[i] * (L.b[i] - L.y[i]);
+            const double x = L.x[i] + v;
+            L.x[i] = x;
+            L.w[i] = 0.0;
+            if (L.xs) L.xs[i] = fe_df::split_pair(x);
+          }
+          break;
         case OP_PROLONG: {
           const double v = P.deg == 1 ? prolong_point<1>(P, L, P.lev[level - 1], i)
                                       : prolong_point<2>(P, L, P.lev[level - 1], i);
-          L.x[i] += v;
-          L.y[i] = 0.0;
+          if (L.rows) {  // y -> x
+            L.x[i] = L.y[i] + v;
+          } else {
+            const double x = L.x[i] + v;
+            L.x[i] = x;
+            L.y[i] = 0.0;
+            if (L.xs) L.xs[i] = fe_df::split_pair(x);
+          }
         } break;
-        case OP_CHEB0_POST: {
-          const double v = L.inv_theta * L.dinv[i] * (L.b[i] - L.y[i]);
-          L.d[i] = v;
-          L.x[i] += v;
-          L.w[i] = 0.0;
-        } break;
+        case OP_CHEB0_POST:
+          if (L.rows) {  // x -> y
+            const double v = L.inv_theta * L.dinv[i] * (L.b[i] - p1_row(L, L.x, i));
+            L.d[i] = v;
+            L.y[i] = L.x[i] + v;
+          } else {
+            const double v = L.inv_theta * L.dinv[i] * (L.b[i] - L.y[i]);
+            const double x = L.x[i] + v;
+            L.d[i] = v;
+            L.x[i] = x;
+            L.w[i] = 0.0;
+            if (L.xs) L.xs[i] = fe_df::split_pair(x);
+          }
+          break;
         case OP_CHEB1_POST: {
-          const double v = L.c1 * L.d[i] + L.c2 * L.dinv[i] * (L.b[i] - L.w[i]);
-          L.d[i] = v;
-          L.x[i] += v;
+          const double yi = L.rows ? p1_row(L, L.y, i) : L.w[i];  // rows: y -> x
+          const double v = L.c1 * L.d[i] + L.c2 * L.dinv[i] * (L.b[i] - yi);
+          L.x[i] = (L.rows ? L.y[i] : L.x[i]) + v;
         } break;
         case OP_RESTRICT:
           L.b[i] = P.deg == 1 ? restrict_point<1>(P, P.lev[level + 1], L, i)
@@ -294,6 +347,7 @@ __device__ void dof_phase(const Params& A, int level, int op, bool all_problems)
         case OP_P_FROM_Z:
           P.p[i] = L.x[i];
           P.q[i] = 0.0;
+          if (L.xs) P.ps[i] = fe_df::split_pair(L.x[i]);
           break;
         case OP_DOT_PQ:
           acc += P.p[i] * P.q[i];
@@ -304,10 +358,12 @@ __device__ void dof_phase(const Params& A, int level, int op, bool all_problems)
           L.b[i] = r;
           acc += r * r;
         } break;
-        case OP_UPDATE_P:
-          P.p[i] = L.x[i] + beta * P.p[i];
+        case OP_UPDATE_P: {
+          const double v = L.x[i] + beta * P.p[i];
+          P.p[i] = v;
           P.q[i] = 0.0;
-          break;
+          if (L.xs) P.ps[i] = fe_df::split_pair(v);
+        } break;
       }
     }
     if (op == OP_R_FROM_RHS || op == OP_DOT_RZ || op == OP_DOT_PQ || op == OP_UPDATE_XR) {
@@ -320,13 +376,14 @@ __device__ void dof_phase(const Params& A, int level, int op, bool all_problems)
   }
 }
 
-enum VecSel { V_X_TO_Y, V_X_TO_W, V_P_TO_Q, V_F_TO_RHS };
+// V_X_TO_W: the residual after pre-smoothing; V_X_TO_W_POST: the second post-smoothing step
+enum VecSel { V_X_TO_Y, V_X_TO_W, V_X_TO_W_POST, V_P_TO_Q, V_F_TO_RHS };
 
 template <int DEG>
 __device__ void apply_cells(const Params& A, const BProb& P, const BLevel& L, int c0, int c1, int sel) {
   constexpr int ND = DEG == 1 ? 4 : 10;
   const double* in = sel == V_P_TO_Q ? P.p : sel == V_F_TO_RHS ? P.f : L.x;
-  double* out = sel == V_X_TO_Y ? L.y : sel == V_X_TO_W ? L.w : sel == V_P_TO_Q ? P.q : P.rhs;
+  double* out = sel == V_X_TO_Y ? L.y : sel == V_P_TO_Q ? P.q : sel == V_F_TO_RHS ? P.rhs : L.w;
   const double* mref = DEG == 1 ? A.mref1 : A.mref2;
   for (int c = c0 + threadIdx.x; c < c1; c += blockDim.x) {
     int idx[ND];
@@ -348,6 +405,45 @@ __device__ void apply_cells(const Params& A, const BProb& P, const BLevel& L, in
         atomicAdd(out + idx[i], s * a);
       }
     } else if (A.df) {
+      if constexpr (DEG == 2) {
+        if (L.xs) {  // the pairs that the dof phases wrote, rescaled by a power of two (as in k_apply_lp)
+          const float2* xs = sel == V_P_TO_Q ? P.ps : L.xs;
+          float2 xv[ND];
+          unsigned int mb = 0u;
+#pragma unroll
+          for (int j = 0; j < ND; ++j) xv[j] = idx[j] >= 0 ? xs[idx[j]] : make_float2(0.0f, 0.0f);
+#pragma unroll
+          for (int j = 0; j < ND; ++j) mb = max(mb, __float_as_uint(xv[j].x) & 0x7FFFFFFFu);
+          if (mb == 0u) continue;  // every dof is zero
+          const int ef = (int)(mb >> 23);
+          if (ef != 0xFF) {  // (a marker: some dof does not fit an unscaled pair)
+            fe_df::DF ud[ND];
+#pragma unroll
+            for (int j = 0; j < ND; ++j) ud[j] = fe_df::DF(xv[j].x, xv[j].y);
+            const float f = __uint_as_float((unsigned int)(254 - ef) << 23);
+            const float2 v = L.cdf[c];
+            const unsigned int cb = __float_as_uint(v.x);
+            const int ec = (int)((cb >> 23) & 0xFFu);
+            const fe_df::DF cs(__fmul_rn(__uint_as_float((cb & 0x807FFFFFu) | (126u << 23)), f),
+                               __fmul_rn(__fmul_rn(v.y, __uint_as_float((unsigned int)(253 - ec) << 23)), f));
+            float la[10], lb[10], lc[10];
+            fe_df::p2_kuhn_split(ud, cs, la, lb, lc);
+            const int w = ec + ef + 896 - 124;
+            if (w >= 127 && w <= 1918) {
+              const unsigned int kexp = (unsigned int)(w - 127) << 20;
+              fe_df::p2_kuhn_apply(la, lb, lc, [&](int j, fe_df::DF t) {
+                if (idx[j] >= 0)
+                  atomicAdd(out + idx[j], fe_df::widen_in_range(t.hi, kexp) + fe_df::widen_in_range(t.lo, kexp));
+              });
+            } else {
+              fe_df::p2_kuhn_apply(la, lb, lc, [&](int j, fe_df::DF t) {
+                if (idx[j] >= 0) atomicAdd(out + idx[j], fe_df::widen_scaled(t.hi, w) + fe_df::widen_scaled(t.lo, w));
+              });
+            }
+            continue;
+          }
+        }
+      }
 #pragma unroll
       for (int j = 0; j < ND; ++j) u[j] = idx[j] >= 0 ? in[idx[j]] : 0.0;
       const int emax = fe_df::block_exponent<ND>(u);
@@ -401,34 +497,43 @@ __device__ void apply_cells(const Params& A, const BProb& P, const BLevel& L, in
   }
 }
 
-// Operator application on `level`: cell items (atomic scatter) and boundary
-// items (identity rows; for the load vector, zero Dirichlet rows) in one phase.
+// Operator application on `level`: cell items (atomic scatter), boundary items
+// (identity rows) and row items in one phase; for the load vector the cells of
+// every problem.  The smoother's applications skip the problems whose dof phases
+// form the rows themselves.
 __device__ void apply_phase(const Params& A, int level, int sel, bool all_problems) {
   const Work& W = A.W;
-  const int nc = W.end[R_CELL][level] - W.beg[R_CELL][level];
-  const int nbi = W.end[R_BND][level] - W.beg[R_BND][level];
-  for (int t = blockIdx.x; t < nc + (sel == V_F_TO_RHS ? 0 : nbi); t += gridDim.x) {
-    const bool is_cell = t < nc;
-    const int4 item = W.items[is_cell ? W.beg[R_CELL][level] + t : W.beg[R_BND][level] + (t - nc)];
+  const int kc = sel == V_F_TO_RHS ? R_MASS : R_CELL;
+  const int nc = W.end[kc][level] - W.beg[kc][level];
+  const int nbi = sel == V_F_TO_RHS ? 0 : W.end[R_BND][level] - W.beg[R_BND][level];
+  const int nr = sel == V_X_TO_W || sel == V_P_TO_Q ? W.end[R_AROW][level] - W.beg[R_AROW][level] : 0;
+  for (int t = blockIdx.x; t < nc + nbi + nr; t += gridDim.x) {
+    const int4 item = W.items[t < nc         ? W.beg[kc][level] + t
+                              : t < nc + nbi ? W.beg[R_BND][level] + (t - nc)
+                                             : W.beg[R_AROW][level] + (t - nc - nbi)];
     const BProb& P = A.prob[item.x];
     if (!all_problems && !A.sc[item.x].active) continue;
     const BLevel& L = P.lev[level];
-    if (is_cell) {
+    if (t < nc) {
       if (P.deg == 1)
         apply_cells<1>(A, P, L, item.y, item.z, sel);
       else
         apply_cells<2>(A, P, L, item.y, item.z, sel);
-    } else {
+    } else if (t < nc + nbi) {
       const double* in = sel == V_P_TO_Q ? P.p : L.x;
-      double* out = sel == V_X_TO_Y ? L.y : sel == V_X_TO_W ? L.w : P.q;
+      double* out = sel == V_X_TO_Y ? L.y : sel == V_P_TO_Q ? P.q : L.w;
       for (int k = item.y + threadIdx.x; k < item.z; k += blockDim.x) out[L.bnd[k]] = in[L.bnd[k]];
+    } else {  // the pre-smoothed iterate lies in y
+      const double* in = sel == V_P_TO_Q ? P.p : L.y;
+      double* out = sel == V_P_TO_Q ? P.q : L.w;
+      for (int i = item.y + threadIdx.x; i < item.z; i += blockDim.x) out[i] = p1_row(L, in, i);
     }
   }
 }
 
 __device__ void zero_rhs_boundary(const Params& A, int level) {
   const Work& W = A.W;
-  for (int it = W.beg[R_BND][level] + blockIdx.x; it < W.end[R_BND][level]; it += gridDim.x) {
+  for (int it = W.beg[R_RBND][level] + blockIdx.x; it < W.end[R_RBND][level]; it += gridDim.x) {
     const int4 item = W.items[it];
     const BProb& P = A.prob[item.x];
     const BLevel& L = P.lev[level];
@@ -489,7 +594,7 @@ __device__ bool vcycle(const Params& A, uint64_t& tl) {
     if (!pbar(A, FE_PHASE_SMOOTH, l, tl)) return false;
     dof_phase(A, l, OP_CHEB0_POST, false);
     if (!pbar(A, FE_PHASE_SMOOTH, l, tl)) return false;
-    apply_phase(A, l, V_X_TO_W, false);
+    apply_phase(A, l, V_X_TO_W_POST, false);
     if (!pbar(A, FE_PHASE_SMOOTH, l, tl)) return false;
     dof_phase(A, l, OP_CHEB1_POST, false);
     if (!pbar(A, FE_PHASE_SMOOTH, l, tl)) return false;
@@ -602,6 +707,7 @@ struct fe_batch {
   Work work{};
   Schedule sched;
   bool tuned = false;
+  std::vector<char> row_form;  // per problem and level, as the work lists were built
   int sms = 148;
   std::vector<const double*> f_ptrs;
   std::vector<double*> u_ptrs;
@@ -616,7 +722,21 @@ struct fe_batch {
 
 namespace {
 
+// Whether level l's operator runs over rows (P1 in the float-pair modes, where it has the edge form).
+// The mode of the whole batch is its first problem's.
+bool batch_native(const fe_batch* B) { return B->hs[0]->f64_mode == FE_F64_NATIVE; }
+bool batch_rows(const fe_batch* B, const fe_hierarchy* h, int l) {
+  return h->deg == 1 && !batch_native(B) && h->L[l].flux != FLUX_NONE;
+}
+std::vector<char> batch_row_form(const fe_batch* B) {
+  std::vector<char> rows;
+  for (const fe_hierarchy* h : B->hs)
+    for (int l = 0; l < B->nlev; ++l) rows.push_back(batch_rows(B, h, l));
+  return rows;
+}
+
 void build_items(fe_batch* B) {
+  B->row_form = batch_row_form(B);
   std::vector<int4> it;
   Work W{};
   const int P = (int)B->hs.size();
@@ -629,10 +749,14 @@ void build_items(fe_batch* B) {
     W.end[kind][l] = (int)it.size();
   };
   for (int l = 0; l < B->nlev; ++l) {
-    blocks(R_CELL, l, B->sched.cell_block, [](fe_hierarchy* h, int l) { return h->L[l].C; });
+    blocks(R_CELL, l, B->sched.cell_block, [B](fe_hierarchy* h, int l) { return batch_rows(B, h, l) ? 0 : h->L[l].C; });
+    blocks(R_BND, l, B->sched.dof_block, [B](fe_hierarchy* h, int l) { return batch_rows(B, h, l) ? 0 : h->L[l].nb; });
+    blocks(R_AROW, l, B->sched.cell_block, [B](fe_hierarchy* h, int l) { return batch_rows(B, h, l) ? h->L[l].n : 0; });
     blocks(R_DOF, l, B->sched.dof_block, [](fe_hierarchy* h, int l) { return h->L[l].n; });
-    blocks(R_BND, l, B->sched.dof_block, [](fe_hierarchy* h, int l) { return h->L[l].nb; });
   }
+  const int fine = B->nlev - 1;
+  blocks(R_MASS, fine, B->sched.cell_block, [](fe_hierarchy* h, int l) { return h->L[l].C; });
+  blocks(R_RBND, fine, B->sched.dof_block, [](fe_hierarchy* h, int l) { return h->L[l].nb; });
   blocks(R_ROW, 0, 64, [](fe_hierarchy* h, int) { return h->cs.nci; });
   B->items.alloc(it.size());
   CUDA_CHECK(cudaMemcpy(B->items.p, it.data(), sizeof(int4) * it.size(), cudaMemcpyHostToDevice));
@@ -662,6 +786,10 @@ void fill_problems(fe_batch* B, double cheb_lo, double cheb_hi) {
       D.geodf = L.geodf;
       D.cdf = L.cdf;
       D.uniform = L.uniform;
+      D.rows = batch_rows(B, h, l);
+      D.fw = L.flux == FLUX_VAR ? L.fw64.p : nullptr;
+      D.c1d = L.kappa0 / L.N;
+      D.xs = L.deg == 2 && L.uniform && !batch_native(B) ? L.xs64.p : nullptr;
       D.rtab = L.rtab;
       D.ptab = L.ptab;
       D.dinv = L.dinv64;
@@ -697,6 +825,7 @@ void fill_problems(fe_batch* B, double cheb_lo, double cheb_hi) {
     P.p = h->p;
     P.q = h->q;
     P.rhs = h->b;
+    P.ps = h->ps;
     P.f = B->f_ptrs.empty() ? nullptr : B->f_ptrs[p];
   }
   CUDA_CHECK(cudaMemcpy(B->dprob.p, hp.data(), sizeof(BProb) * hp.size(), cudaMemcpyHostToDevice));
@@ -734,7 +863,7 @@ Params make_params(fe_batch* B, const fe_solver_opts& o) {
   A.mref2 = B->mref2;
   A.nprob = (int)B->hs.size();
   A.nlev = B->nlev;
-  A.df = B->hs[0]->f64_mode != FE_F64_NATIVE;
+  A.df = !batch_native(B);
   A.max_it = o.max_it;
   A.rtol = o.rtol;
   A.timeout_ns = o.wait_timeout_us > 0 ? (unsigned long long)o.wait_timeout_us * 1000ull : 5000000000ull;
@@ -896,6 +1025,7 @@ int fe_solve_batched(fe_batch* B, const double* const* f_nodal, double* const* u
       FE_REQUIRE(cudaPointerGetAttributes(&a, u[p]) == cudaSuccess && a.type == cudaMemoryTypeDevice, FE_ERR_ARG,
                  "batched vectors must be device pointers");
     }
+    if (batch_row_form(B) != B->row_form) build_items(B);  // a mode or geometry form changed since
     fill_problems(B, o.cheb_lo, o.cheb_hi);
     if (!B->tuned && o.use_graph && !o.profile) autotune(B, o, s);
     const double ms = run_solve(B, o, s);
