@@ -353,6 +353,7 @@ struct GraphCache {
   cudaStream_t stream = nullptr;
   int steps = 0;  // smoother parameters baked into the captured launches
   double lo = 0, hi = 0;
+  int calls = 0;  // fe_vcycle calls since the last invalidation
   int extra = 0;  // another baked parameter (V-cycles per level of the full-multigrid graph)
 };
 

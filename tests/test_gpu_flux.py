@@ -152,3 +152,32 @@ def test_fp32_cycle_with_tiled_restriction_matches_fp64(fe, N0):
         h.vcycle(dt(b), x)
         h.vcycle(dt(b, torch.float32), x32, dtype=fe.FE_F32)
         assert (x32.double() - x).abs().max() <= 5e-6 * x.abs().max()
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_vcycle_replayed_and_captured(fe, dtype):
+    """The V-cycle's later calls replay its graph: with new inputs, other buffers and a changed coefficient they equal the
+    first call's result for those inputs (bitwise up to the order of atomic additions, 1e-13 / 1e-5 of the largest entry),
+    also inside a graph that the caller captures."""
+    d = torch.float64 if dtype == "f64" else torch.float32
+    code, tol = (fe.FE_F64, 1e-13) if dtype == "f64" else (fe.FE_F32, 1e-5)
+    kappas = [np.ones(6 * 16 ** 3), np.exp(I.random_vector(6 * 16 ** 3, 5))]
+    with fe.Hierarchy(4, 2, 2) as h, fe.Hierarchy(4, 2, 2) as fresh:
+        b = [dt(I.random_vector(h.n_dofs(), s), d) for s in (1, 2, 3)]
+        for kappa in kappas:
+            h.set_coefficient(dt(kappa))
+            for i in range(3):
+                fresh.set_coefficient(dt(kappa))  # its next call is a first one
+                x, ref = torch.empty_like(b[i]), torch.empty_like(b[i])
+                h.vcycle(b[i], x, dtype=code)
+                fresh.vcycle(b[i], ref, dtype=code)
+                assert (x - ref).abs().max() <= tol * ref.abs().max()
+        y, stream = torch.empty_like(b[0]), torch.cuda.Stream()
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream):
+            h.vcycle(b[2], y, dtype=code, stream=stream)
+        y.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert (y - ref).abs().max() <= tol * ref.abs().max()
