@@ -608,7 +608,10 @@ __device__ bool any_active(const Params& A) {
   return false;
 }
 
-__global__ void __launch_bounds__(kThreads) k_batched_pcg(Params A) {
+// Registers for three blocks per SM: the element phases wait for their gathers, and 24 warps hide more than the spills
+// cost (2, 3 and 4 blocks: 64.1, 56.7 and 55.5 ms for 64 problems, 30.8, 29.6 and 31.3 for 16, 18.5, 18.7 and 19.1
+// for 4, where the grid's barriers are the time).
+__global__ void __launch_bounds__(kThreads, 3) k_batched_pcg(Params A) {
   const int fine = A.nlev - 1;
   const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
   uint64_t tl = now_ns();  // profile clock of block 0
