@@ -625,14 +625,20 @@ static void vcycle_level(fe_hierarchy* h, int l, int dtype, cudaStream_t s) {
     PhaseScope ps(FE_PHASE_SMOOTH, l, s);
     smooth_enqueue<T>(h, l, b, x, y, d, g_sp.steps, g_sp.lo, g_sp.hi, true, dtype, s, false, true);
   }
+  // FP32: y = b - A x in the operator's epilogue, so that the restriction stages one vector, asynchronously, instead of
+  // two (P2 128^3 -> 64^3: 131 -> 48 us).  The FP64 restriction takes 43 us at 64^3 either way.
+  const bool residual = sizeof(T) == 4 && use_flux(h, l, rdt);
   {
     PhaseScope ps(FE_PHASE_APPLY, l, s);
-    apply_enqueue(h, l, x, y, rdt, s, xs);
+    if (residual)
+      launch_flux_residual<T>(L, b, x, y, s);
+    else
+      apply_enqueue(h, l, x, y, rdt, s, xs);
   }
   Level& Lc = h->L[l - 1];
   {
     PhaseScope ps(FE_PHASE_TRANSFER, l, s);
-    launch_restrict<T>(h, l, b, y, lv_b<T>(Lc), true, s);
+    launch_restrict<T>(h, l, residual ? y : b, residual ? nullptr : y, lv_b<T>(Lc), true, s);
   }
   vcycle_level<T>(h, l - 1, dtype, s);
   {
@@ -742,11 +748,14 @@ static void fmg_enqueue(fe_hierarchy* h, const double* b, int cycles, cudaStream
       launch_prolong<double>(h, l, h->L[l - 1].fx64, L.fx64, false, s);
     }
     for (int c = 0; c < cycles; ++c) {
-      {
+      if (use_flux(h, l, FE_F64)) {
         PhaseScope ps(FE_PHASE_APPLY, l, s);
-        apply_enqueue(h, l, L.fx64, L.y64, FE_F64, s);
-      }
-      {
+        launch_flux_residual<double>(L, L.fb64, L.fx64, L.b64, s);
+      } else {
+        {
+          PhaseScope ps(FE_PHASE_APPLY, l, s);
+          apply_enqueue(h, l, L.fx64, L.y64, FE_F64, s);
+        }
         PhaseScope ps(FE_PHASE_BLAS1, l, s);
         launch_sub64(L.n, L.fb64, L.y64, L.b64, s);
       }

@@ -33,13 +33,13 @@ using namespace fe_fixed;
 inline int ceil_div(long long a, int b) { return (int)((a + b - 1) / b); }
 
 // What a kernel does with its row y_i of A x.
-enum Epilogue { EPI_APPLY = 0, EPI_CHEB = 1 };
+enum Epilogue { EPI_APPLY = 0, EPI_CHEB = 1, EPI_RESIDUAL = 2 };
 
 template <typename T>
 struct Rows {
   const T* x;     // the operator's input (also the iterate that a Chebyshev step updates)
-  T* out;         // APPLY: y; CHEB: the new iterate (another vector than x)
-  const T* b;     // CHEB: right-hand side
+  T* out;         // APPLY: y; CHEB: the new iterate (another vector than x); RESIDUAL: b - y
+  const T* b;     // CHEB, RESIDUAL: right-hand side
   const T* din;   // CHEB: the previous direction (null: c1 = 0)
   T* dout;        // CHEB: the new direction (null: not stored)
   const T* dinv;  // CHEB on P1 with a coefficient per cell: inverse diagonal
@@ -53,8 +53,8 @@ struct RowIn {
   T b = T(0), d = T(0), x = T(0);
   __device__ __forceinline__ RowIn() {}
   __device__ __forceinline__ RowIn(const Rows<T>& R, int i) {
+    if constexpr (EPI != EPI_APPLY) b = __ldg(R.b + i);
     if constexpr (EPI == EPI_CHEB) {
-      b = __ldg(R.b + i);
       if (R.din) d = R.din[i];
       x = __ldg(R.x + i);
     }
@@ -64,13 +64,15 @@ struct RowIn {
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
-// Row y_i = s v; Chebyshev: d = c1 d + w (b - y), x += d with w = c2 / A_ii.
+// Row y_i = s v; residual: b - y; Chebyshev: d = c1 d + w (b - y), x += d with w = c2 / A_ii.
 // FP64 operations are scarce (2 per clock and SM), so the scaling of y and the
 // diagonal are folded: 4 of them per row with a previous direction.
 template <int EPI, typename T>
 __device__ __forceinline__ void finish_row(const Rows<T>& R, const RowIn<EPI, T>& in, int i, T v, T s, T w) {
   if constexpr (EPI == EPI_APPLY) {
     R.out[i] = v * s;
+  } else if constexpr (EPI == EPI_RESIDUAL) {
+    R.out[i] = fma_t(-v, s, in.b);
   } else {
     const T r = fma_t(-v, s, in.b);
     const T dn = R.din ? fma_t(w, r, R.c1 * in.d) : w * r;
@@ -346,14 +348,6 @@ __device__ __noinline__ Pair32 fixed_pair_window(double x, int E, int pass) {
   return {sg * (int)(w >> 30), sg * (int)(w & 0x3FFFFFFF)};
 }
 
-template <int BYTES>
-__device__ __forceinline__ void cp_async_or_zero(void* smem, const void* gmem, bool valid) {
-  const unsigned int sa = (unsigned int)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(sa), "l"(gmem), "n"(BYTES),
-               "r"(valid ? BYTES : 0)
-               : "memory");
-}
-
 template <int TX_, int TY_, int KZ_, int THREADS_, int BLOCKS_>
 struct TileShape {  // BLOCKS: resident blocks per SM that the registers are limited for
   static constexpr int blocks = BLOCKS_;
@@ -491,7 +485,7 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
       };
       RowSum<V> rs[8];
       RowIn<EPI, T> ins[8];  // FP32: every row's vectors in flight before the rows are formed
-      if constexpr (!FIX && EPI == EPI_CHEB) {
+      if constexpr (!FIX && EPI != EPI_APPLY) {
 #pragma unroll
         for (int code = 0; code < 8; ++code)
           if (((code & 1) || vi > 0) && ((code & 2) || vj > 0) && ((code & 4) || vk > 0))
@@ -692,6 +686,7 @@ void launch_flux_setup(Level& L, cudaStream_t s) {
   if (L.deg == 2) {
     set_smems<EPI_APPLY>();
     set_smems<EPI_CHEB>();
+    set_smems<EPI_RESIDUAL>();
   } else if (L.flux == FLUX_VAR) {
     L.fw64.alloc((size_t)4 * L.n);
     L.fw32.alloc((size_t)4 * L.n);
@@ -709,6 +704,17 @@ void launch_flux_apply(const Level& L, const T* x, T* y, cudaStream_t s) {
 }
 template void launch_flux_apply<double>(const Level&, const double*, double*, cudaStream_t);
 template void launch_flux_apply<float>(const Level&, const float*, float*, cudaStream_t);
+
+template <typename T>
+void launch_flux_residual(const Level& L, const T* b, const T* x, T* r, cudaStream_t s) {
+  Rows<T> R{};
+  R.x = x;
+  R.b = b;
+  R.out = r;
+  launch<EPI_RESIDUAL>(L, R, s);
+}
+template void launch_flux_residual<double>(const Level&, const double*, const double*, double*, cudaStream_t);
+template void launch_flux_residual<float>(const Level&, const float*, const float*, float*, cudaStream_t);
 
 template <typename T>
 void launch_flux_cheb(const Level& L, const T* b, const T* x, T* xout, const T* din, T* dout, double c1, double c2,

@@ -199,6 +199,14 @@ __device__ __forceinline__ void cp_async16(void* smem, const void* gmem, int byt
   const unsigned int sa = (unsigned int)__cvta_generic_to_shared(smem);
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(sa), "l"(gmem), "r"(bytes) : "memory");
 }
+// BYTES (4 or 8) from gmem, or zeros
+template <int BYTES>
+__device__ __forceinline__ void cp_async_or_zero(void* smem, const void* gmem, bool valid) {
+  const unsigned int sa = (unsigned int)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(sa), "l"(gmem), "n"(BYTES),
+               "r"(valid ? BYTES : 0)
+               : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 // Until at most N of this thread's most recent groups are still in flight.
@@ -457,6 +465,8 @@ void launch_apply_cheb64_cube_df(const Level& L, const double* b, double* x, dou
 void launch_flux_setup(Level& L, cudaStream_t s);
 template <typename T>
 void launch_flux_apply(const Level& L, const T* x, T* y, cudaStream_t s);
+template <typename T>  // r = b - A x
+void launch_flux_residual(const Level& L, const T* b, const T* x, T* r, cudaStream_t s);
 template <typename T>
 void launch_flux_cheb(const Level& L, const T* b, const T* x, T* xout, const T* din, T* dout, double c1, double c2,
                       cudaStream_t s);

@@ -11,8 +11,9 @@
 // memory, split by the fine coordinates modulo 4 so that a warp's accesses are
 // contiguous, and the weights are immediate operands.  Two threads serve a cell:
 // one the vertex row (125 weights), one the seven others (150).  At 128^3 -> 64^3
-// the gathers took 215 us against 20 us for the two vectors' bytes; with all of the solve around it
-// the mixed-precision solve of that size went from 12.6 to 10.9 ms.
+// the gathers took 215 us, staging b and y through registers 131 us, and with the
+// residual left by the operator one vector staged by asynchronous copies 48 us
+// (its bytes: 11 us).
 // FP64 keeps the table-driven form: its 4.3 + 2.4 (residuals of the extra layer)
 // operations per fine dof bind it to the FP64 pipe (64^3: 60 against 45 us).
 #include <utility>
@@ -107,14 +108,16 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
     for (int code = 0; code < 8; ++code) {
       const int px = code & 1, py = code >> 1 & 1, pz = code >> 2;
       const int i = F.off[code] + ci + F.sy[code] * cj + F.sz[code] * ck;
-      float val = 0.0f;
-      if (in && ci + px <= F.N && cj + py <= F.N && ck + pz <= F.N) {
-        val = __ldg(b + i);
-        if (y) val -= __ldg(y + i);
-      }
-      at[S::S * (px + 4 * py + 16 * pz)] = val;
+      const bool ok = in && ci + px <= F.N && cj + py <= F.N && ck + pz <= F.N;
+      float* to = at + S::S * (px + 4 * py + 16 * pz);
+      if (!y)  // one vector: every copy in flight at once
+        cp_async_or_zero<4>(to, b + (ok ? i : 0), ok);
+      else
+        *to = ok ? __ldg(b + i) - __ldg(y + i) : 0.0f;
     }
   }
+  cp_async_commit();
+  cp_async_wait_all();
   __syncthreads();
   const int c = tid % S::own;
   const int a = c % S::TX, bb = (c / S::TX) % S::TY, e = c / (S::TX * S::TY);

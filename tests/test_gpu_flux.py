@@ -154,6 +154,27 @@ def test_fp32_cycle_with_tiled_restriction_matches_fp64(fe, N0):
         assert (x32.double() - x).abs().max() <= 5e-6 * x.abs().max()
 
 
+@pytest.mark.parametrize("k,N0,levels,coef", [(1, 3, 2, "field"), (2, 2, 2, "one"), (2, 3, 3, "constant"), (2, 3, 2, "field"),
+                                              (3, 2, 2, "field")])
+@pytest.mark.parametrize("f32", [False, True])
+def test_cycle_residuals_match_oracle(fe, k, N0, levels, coef, f32):
+    """Cycles whose operator leaves b - A x for the restriction (small and tiled levels, 24 cubes the largest) equal the
+    oracle's: 1e-11 of the largest entry as for the cycles' parity tests, FP32 1e-5 (condition of the coarse solve)."""
+    with fe.Hierarchy(N0, levels, k) as h:
+        kappa = np.exp(I.random_vector(h.n_cells(), 5)) if coef == "field" else np.full(
+            h.n_cells(), 1.0 if coef == "one" else 0.7)
+        h.set_coefficient(dt(kappa))
+        oh = O.Hierarchy(N0, levels, k, kappa)
+        for l in range(levels + 1):
+            oh.lmax[l] = h.lambda_max(l)
+        b = I.random_vector(h.n_dofs(), 6)
+        b[h.boundary_mask()] = 0.0
+        ref = oh.vcycle(b)
+        x = torch.empty(len(b), dtype=torch.float32 if f32 else torch.float64, device=DEV)
+        h.vcycle(dt(b, x.dtype), x, dtype=fe.FE_F32 if f32 else fe.FE_F64)
+        assert np.abs(x.double().cpu().numpy() - ref).max() <= (1e-5 if f32 else 1e-11) * np.abs(ref).max()
+
+
 @pytest.mark.parametrize("dtype", ["f64", "f32"])
 def test_vcycle_replayed_and_captured(fe, dtype):
     """The V-cycle's later calls replay its graph: with new inputs, other buffers and a changed coefficient they equal the
