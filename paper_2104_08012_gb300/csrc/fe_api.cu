@@ -625,9 +625,9 @@ static void vcycle_level(fe_hierarchy* h, int l, int dtype, cudaStream_t s) {
     PhaseScope ps(FE_PHASE_SMOOTH, l, s);
     smooth_enqueue<T>(h, l, b, x, y, d, g_sp.steps, g_sp.lo, g_sp.hi, true, dtype, s, false, true);
   }
-  // FP32: y = b - A x in the operator's epilogue, so that the restriction stages one vector, asynchronously, instead of
-  // two (P2 128^3 -> 64^3: 131 -> 48 us).  The FP64 restriction takes 43 us at 64^3 either way.
-  const bool residual = sizeof(T) == 4 && use_flux(h, l, rdt);
+  // y = b - A x in the operator's epilogue, so that the restriction stages one vector, asynchronously, instead of two
+  // (P2 FP32 128^3 -> 64^3: 131 -> 48 us; FP64 64^3 -> 32^3: 43 -> 30 us)
+  const bool residual = use_flux(h, l, rdt);
   {
     PhaseScope ps(FE_PHASE_APPLY, l, s);
     if (residual)

@@ -508,9 +508,10 @@ void launch_prolong(const fe_hierarchy* h, int lf, const T* xc, T* xf, bool accu
 // rc = P^T (bf - yf), or P^T bf when yf is null
 template <typename T>
 void launch_restrict(const fe_hierarchy* h, int lf, const T* bf, const T* yf, T* rc, bool zero_bd, cudaStream_t s);
-// The same for FP32 P2 vectors with the coarse boundary rows 0 (fe_restrict.cu); restrict_p2_prepare once per device
+// The same for P2 vectors with the coarse boundary rows 0 (fe_restrict.cu); restrict_p2_prepare once per device
 // and hierarchy.
-void launch_restrict_p2(const Level& F, const Level& Cc, const float* b, const float* y, float* rc, cudaStream_t s);
+template <typename T>
+void launch_restrict_p2(const Level& F, const Level& Cc, const T* b, const T* y, T* rc, cudaStream_t s);
 void restrict_p2_prepare();
 
 // Vector kernels

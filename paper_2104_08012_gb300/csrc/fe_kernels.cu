@@ -1488,11 +1488,11 @@ void launch_restrict(const fe_hierarchy* h, int lf, const T* bf, const T* yf, T*
   const Level& F = h->L[lf];
   const Level& Cc = h->L[lf - 1];
   const TransferTables& t = h->tt;
-  if constexpr (sizeof(T) == 4)
-    if (h->deg == 2 && zero_bd && Cc.N >= kRestrictTiledFrom) {
-      launch_restrict_p2(F, Cc, bf, yf, rc, s);
-      return;
-    }
+  // (the entry point restricts one vector too)
+  if (h->deg == 2 && zero_bd && Cc.N >= kRestrictTiledFrom && (sizeof(T) == 4 || !yf)) {
+    launch_restrict_p2<T>(F, Cc, bf, yf, rc, s);
+    return;
+  }
   if (h->deg == 1)
     k_restrict<1, T, 4><<<ceil_div(Cc.n, 32), 32 * 4, 0, s>>>(F.num.m, Cc.num, Cc.n, t.res_margin, t.res_start,
                                                               F.rtab, tt_weights<T>(t.res_w, t.res_wf), bf,

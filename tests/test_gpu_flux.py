@@ -175,6 +175,26 @@ def test_cycle_residuals_match_oracle(fe, k, N0, levels, coef, f32):
         assert np.abs(x.double().cpu().numpy() - ref).max() <= (1e-5 if f32 else 1e-11) * np.abs(ref).max()
 
 
+@pytest.mark.parametrize("N0", [4, 5])
+def test_fp64_tiled_restriction_matches_table(fe, N0):
+    """The FP64 restriction to 32^3 and 40^3 (ragged tiles) by staged tiles (boundary rows zeroed) equals the table-driven
+    one (boundary rows kept): two sums of at most 125 terms, weights and values at most 1, differ by at most
+    2 * 125 * 125 * 2^-53; a NaN reaches exactly the same rows."""
+    with fe.Hierarchy(N0, 4, 2) as h:
+        r = dt(I.random_vector(h.n_dofs(), 3))
+        inner = torch.from_numpy(~h.boundary_mask(3)).to(DEV)
+        tiled, table = (torch.empty(h.n_dofs(3), dtype=torch.float64, device=DEV) for _ in range(2))
+        for bad in (None, 12345):
+            if bad is not None:
+                r[bad] = float("nan")
+            h.restrict(r, tiled, 4, zero_boundary=True)
+            h.restrict(r, table, 4, zero_boundary=False)
+            assert not tiled[~inner].any()
+            a, b = tiled[inner], table[inner]
+            assert torch.equal(torch.isnan(a), torch.isnan(b))
+            assert (a - b).nan_to_num().abs().max() <= 2 * 125 * 125 * 2.0 ** -53
+
+
 @pytest.mark.parametrize("dtype", ["f64", "f32"])
 def test_vcycle_replayed_and_captured(fe, dtype):
     """The V-cycle's later calls replay its graph: with new inputs, other buffers and a changed coefficient they equal the
