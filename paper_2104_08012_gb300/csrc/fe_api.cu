@@ -358,13 +358,10 @@ static double lmax_of(const double* hist) {
   return tridiag_max_eig(a, off);
 }
 
-// meanwhile(): work on another stream that the host can drive while the iterations run.
-template <typename F>
-static void estimate_lmax(fe_hierarchy* h, cudaStream_t s, F&& meanwhile) {
+static void estimate_lmax(fe_hierarchy* h, cudaStream_t s) {
   constexpr size_t per = (size_t)(kLmaxSteps + 1) * S_COUNT;
   if (!h->lmax_hist) CUDA_CHECK(cudaMallocHost(&h->lmax_hist, sizeof(double) * per * FE_MAX_LEVELS));
   for (int l = 0; l < h->nlev; ++l) enqueue_lmax(h, l, h->lmax_hist + per * l, s);
-  meanwhile();
   CUDA_CHECK(cudaStreamSynchronize(s));
   for (int l = 0; l < h->nlev; ++l) h->L[l].lmax = lmax_of(h->lmax_hist + per * l);
 }
@@ -1177,20 +1174,8 @@ static void set_coefficient_impl(fe_hierarchy* h, const double* kappa, cudaStrea
   }
   if (h->smoother == FE_SMOOTHER_PATCH && h->deg >= 2)
     for (int l = 1; l < h->nlev; ++l) launch_patch_setup(h->L[l], s);
-  // The coarse factorisation and the eigenvalue estimates are both chains of small kernels and share no buffers (the
-  // factorisation reads level 0's coefficients and writes h->cs): side by side they take the longer one's time (P1 96^3:
-  // 5.8 and 4.5 ms).  Everything before is complete on s when the side stream starts; both are waited for here.
-  if (h->nlev > 1 && !h->side) CUDA_CHECK(cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking));
-  CUDA_CHECK(cudaStreamSynchronize(s));
-  try {
-    estimate_lmax(h, s, [&] {
-      if (h->nlev > 1) coarse_setup(h, h->side);
-    });
-  } catch (...) {  // leave nothing in flight on either stream
-    cudaStreamSynchronize(s);
-    if (h->side) cudaStreamSynchronize(h->side);
-    throw;
-  }
+  estimate_lmax(h, s);
+  if (h->nlev > 1) coarse_setup(h, s);
   invalidate_graphs(h);
   CUDA_CHECK(cudaStreamSynchronize(s));
 }
@@ -1407,7 +1392,6 @@ void fe_hierarchy_destroy(fe_hierarchy* h) {
   for (auto& L : h->L) bf16_forget_level(&L);
   red_free(h->red);
   if (h->lmax_hist) cudaFreeHost(h->lmax_hist);
-  if (h->side) cudaStreamDestroy(h->side);
   delete h;
 }
 
@@ -1537,7 +1521,7 @@ int fe_set_smoother(fe_hierarchy* h, int smoother) {
           L.z32.alloc(L.n);
         }
       }
-    estimate_lmax(h, s, [] {});
+    estimate_lmax(h, s);
     invalidate_graphs(h);
     CUDA_CHECK(cudaStreamSynchronize(s));
   }

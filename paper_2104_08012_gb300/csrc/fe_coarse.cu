@@ -790,9 +790,8 @@ void coarse_setup(fe_hierarchy* h, cudaStream_t s) {
     if (cs.band > nci - 1) cs.band = nci - 1;
     cs.ci.alloc(nci);
     cs.dof2int.alloc(L0.n);
-    CUDA_CHECK(cudaMemcpyAsync(cs.ci, ci.data(), sizeof(int) * nci, cudaMemcpyHostToDevice, s));
-    CUDA_CHECK(cudaMemcpyAsync(cs.dof2int, d2i.data(), sizeof(int) * L0.n, cudaMemcpyHostToDevice, s));
-    CUDA_CHECK(cudaStreamSynchronize(s));
+    CUDA_CHECK(cudaMemcpy(cs.ci, ci.data(), sizeof(int) * nci, cudaMemcpyHostToDevice));
+    CUDA_CHECK(cudaMemcpy(cs.dof2int, d2i.data(), sizeof(int) * L0.n, cudaMemcpyHostToDevice));
     cs.t0.alloc(nci);
     cs.t1.alloc(nci);
     cs.flag.alloc(1);

@@ -425,7 +425,6 @@ struct fe_hierarchy {
   } cgloop;
   DBuf<double> xcg, cgp;  // CG iterate of the graph loop; loop target
   DBuf<int> cgctl;        // loop counters
-  cudaStream_t side = nullptr;  // the coarse factorisation of a set-up, beside the eigenvalue estimates
   double* lmax_hist = nullptr;  // pinned: CG scalars of the eigenvalue estimates, [level][iteration][S_COUNT]
   int f64_mode = FE_F64_DOUBLE_FLOAT;  // arithmetic of FP64 operator applications
   int fuse_smoother = 0;               // Chebyshev update fused into the operator kernel (measured slower on GB300)
