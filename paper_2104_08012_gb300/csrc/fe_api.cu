@@ -448,18 +448,28 @@ static bool presplit(const fe_hierarchy* h, int l) {
          !(h->smoother == FE_SMOOTHER_PATCH && h->deg >= 2 && l >= 1 && L.pdof.p);
 }
 
+// Whether the operator of this precision on level l adds element contributions to a y that it needs zero and that an
+// earlier kernel can have zeroed (OperatorNext).
+static bool scatters(const fe_hierarchy* h, int l, int dtype) {
+  const Level& L = h->L[l];
+  if (use_flux(h, l, dtype) || (h->fuse_smoother && L.deg <= 2)) return false;
+  if (dtype == FE_F64)
+    return L.deg == 3 ? L.uniform && h->f64_mode != FE_F64_NATIVE : L.deg == 2 && h->f64_mode == FE_F64_DOUBLE_FLOAT;
+  return dtype == FE_F32;
+}
+
 void apply_enqueue(const fe_hierarchy* h, int level, const void* x, void* y, int dtype, cudaStream_t s,
-                   const float2* xs) {
+                   const float2* xs, bool y_zero) {
   const Level& L = h->L[level];
   if (L.deg == 3) {  // P3: element through the gradient at the P2 nodes in FP64, float pairs (default), FP32 or bf16
     if (dtype == FE_F64 && h->f64_mode == FE_F64_NATIVE)
       launch_apply64(L, (const double*)x, (double*)y, s);
     else if (dtype == FE_F64 && L.uniform)
-      launch_apply64_p3(L, (const double*)x, (double*)y, s);
+      launch_apply64_p3(L, (const double*)x, (double*)y, s, y_zero);
     else if (dtype == FE_F64)
       launch_apply64_df3(L, (const double*)x, (double*)y, s);
     else if (dtype == FE_F32)
-      launch_apply32(L, (const float*)x, (float*)y, s);
+      launch_apply32(L, (const float*)x, (float*)y, s, y_zero);
     else if (dtype == FE_BF16)
       apply_bf16_enqueue(L, (const float*)x, (float*)y, s);
     else
@@ -481,11 +491,11 @@ void apply_enqueue(const fe_hierarchy* h, int level, const void* x, void* y, int
   else if (dtype == FE_F64 && h->f64_mode != FE_F64_NATIVE && cube)
     launch_apply64_cube_df(L, (const double*)x, (double*)y, s);
   else if (dtype == FE_F64 && h->f64_mode != FE_F64_NATIVE)
-    launch_apply64_df(L, (const double*)x, (double*)y, s, h->f64_mode == FE_F64_DOUBLE_FLOAT ? xs : nullptr);
+    launch_apply64_df(L, (const double*)x, (double*)y, s, h->f64_mode == FE_F64_DOUBLE_FLOAT ? xs : nullptr, y_zero);
   else if (dtype == FE_F64)
     launch_apply64(L, (const double*)x, (double*)y, s);
   else if (dtype == FE_F32)
-    launch_apply32(L, (const float*)x, (float*)y, s);
+    launch_apply32(L, (const float*)x, (float*)y, s, y_zero);
   else if (dtype == FE_BF16)
     apply_bf16_enqueue(L, (const float*)x, (float*)y, s);
   else
@@ -498,8 +508,8 @@ void apply_enqueue(const fe_hierarchy* h, int level, const void* x, void* y, int
 // operator kernel and the vector kernel.
 template <typename T>
 static void apply_cheb_enqueue(fe_hierarchy* h, int l, const T* b, T* x, T* y, T* d, double c1, double c2,
-                               bool store_d, int dtype, cudaStream_t s, const float2* xs_in = nullptr,
-                               float2* xs_out = nullptr) {
+                               bool store_d, int dtype, cudaStream_t s, const float2* xs_in, bool y_zero,
+                               OperatorNext<T> next) {
   Level& L = h->L[l];
   if (h->fuse_smoother && L.cnt_tet.p && L.deg <= 2) {
     const bool cube = h->f64_mode == FE_F64_DOUBLE_FLOAT_CUBE || (h->f64_mode == FE_F64_DOUBLE_FLOAT && L.deg == 1);
@@ -518,20 +528,22 @@ static void apply_cheb_enqueue(fe_hierarchy* h, int l, const T* b, T* x, T* y, T
       }
     }
   }
-  apply_enqueue(h, l, x, y, dtype, s, xs_in);
-  launch_cheb_step<T>(L.n, b, y, lv_dinv<T>(L), x, d, c1, c2, false, s, store_d, xs_out);
+  apply_enqueue(h, l, x, y, dtype, s, xs_in, y_zero);
+  launch_cheb_step<T>(L.n, b, y, lv_dinv<T>(L), x, d, c1, c2, false, s, store_d, next);
 }
 
 // Chebyshev iterations on level l (the level smoother of Section 3): the
 // three-term Chebyshev semi-iteration for the preconditioned operator on
 // [lo, hi] * lambda_max, theta = centre, delta = half-width of the interval.
-// xs_fresh_in: L.xs64 holds x as float pairs on entry (FP64, presplit levels);
-// xs_after: leave L.xs64 current with the smoothed x (an operator application
-// reads it next).
+// ready_in: the kernel that wrote x has prepared its operator application (L.xs64
+// holds x as float pairs on presplit levels, y is zero where scatters());
+// ready_after: prepare the same for the residual of the smoothed x (in FP32 for
+// bf16 smoothing).
 template <typename T>
 static void smooth_enqueue(fe_hierarchy* h, int l, const T* b, T* x, T* y, T* d, int steps, double lo, double hi,
-                           bool x_zero, int dtype, cudaStream_t s, bool xs_fresh_in = false, bool xs_after = false) {
+                           bool x_zero, int dtype, cudaStream_t s, bool ready_in = false, bool ready_after = false) {
   Level& L = h->L[l];
+  const bool sc = scatters(h, l, dtype), sc_after = ready_after && scatters(h, l, dtype == FE_BF16 ? FE_F32 : dtype);
   const double a = lo * L.lmax, bmax = hi * L.lmax;
   const double theta = 0.5 * (bmax + a), delta = 0.5 * (bmax - a), sigma = theta / delta;
   double rho = 1.0 / sigma;
@@ -540,13 +552,14 @@ static void smooth_enqueue(fe_hierarchy* h, int l, const T* b, T* x, T* y, T* d,
     for (int k = 0; k < steps; ++k) {
       const bool last = k + 1 == steps;
       const bool from_zero = k == 0 && x_zero;
-      if (!from_zero) apply_enqueue(h, l, x, y, dtype, s);
-      launch_patch_apply<T>(L, b, from_zero ? nullptr : y, z, h->f64_mode != FE_F64_NATIVE, s);
+      if (!from_zero) apply_enqueue(h, l, x, y, dtype, s, nullptr, sc && (k > 0 || ready_in));
+      launch_patch_apply<T>(L, b, from_zero ? nullptr : y, z, h->f64_mode != FE_F64_NATIVE, s, k > 0);
+      T* yz = (last ? sc_after : sc) ? y : nullptr;
       if (k == 0) {
-        launch_cheb_pc<T>(L.n, z, x, d, 0.0, 1.0 / theta, from_zero, !last, s);
+        launch_cheb_pc<T>(L.n, z, x, d, 0.0, 1.0 / theta, from_zero, !last, s, yz, !last);
       } else {
         const double rn = 1.0 / (2.0 * sigma - rho);
-        launch_cheb_pc<T>(L.n, z, x, d, rn * rho, 2.0 * rn / delta, false, !last, s);
+        launch_cheb_pc<T>(L.n, z, x, d, rn * rho, 2.0 * rn / delta, false, !last, s, yz, !last);
         rho = rn;
       }
     }
@@ -589,16 +602,19 @@ static void smooth_enqueue(fe_hierarchy* h, int l, const T* b, T* x, T* y, T* d,
     if (dtype == FE_F64 && presplit(h, l)) xs = L.xs64.p;
   for (int k = 0; k < steps; ++k) {
     const bool last = k + 1 == steps;  // its direction d is not used again
-    float2* xs_out = (!last || xs_after) ? xs : nullptr;
-    const float2* xs_in = (k > 0 || xs_fresh_in) ? xs : nullptr;
+    const bool ready = k > 0 || ready_in;
+    const float2* xs_in = ready ? xs : nullptr;
+    OperatorNext<T> next;
+    if (!last || ready_after) next.xs = xs;
+    if (last ? sc_after : sc) next.y = y;
     if (k == 0) {
       if (x_zero)
-        launch_cheb_step<T>(L.n, b, nullptr, lv_dinv<T>(L), x, d, 0.0, 1.0 / theta, true, s, !last, xs_out);
+        launch_cheb_step<T>(L.n, b, nullptr, lv_dinv<T>(L), x, d, 0.0, 1.0 / theta, true, s, !last, next);
       else
-        apply_cheb_enqueue<T>(h, l, b, x, y, d, 0.0, 1.0 / theta, !last, dtype, s, xs_in, xs_out);
+        apply_cheb_enqueue<T>(h, l, b, x, y, d, 0.0, 1.0 / theta, !last, dtype, s, xs_in, sc && ready, next);
     } else {
       const double rn = 1.0 / (2.0 * sigma - rho);
-      apply_cheb_enqueue<T>(h, l, b, x, y, d, rn * rho, 2.0 * rn / delta, !last, dtype, s, xs_in, xs_out);
+      apply_cheb_enqueue<T>(h, l, b, x, y, d, rn * rho, 2.0 * rn / delta, !last, dtype, s, xs_in, sc && ready, next);
       rho = rn;
     }
   }
@@ -630,7 +646,7 @@ static void vcycle_level(fe_hierarchy* h, int l, int dtype, cudaStream_t s) {
     if (residual)
       launch_flux_residual<T>(L, b, x, y, s);
     else
-      apply_enqueue(h, l, x, y, rdt, s, xs);
+      apply_enqueue(h, l, x, y, rdt, s, xs, scatters(h, l, rdt));
   }
   Level& Lc = h->L[l - 1];
   {
@@ -640,10 +656,13 @@ static void vcycle_level(fe_hierarchy* h, int l, int dtype, cudaStream_t s) {
   vcycle_level<T>(h, l - 1, dtype, s);
   {
     PhaseScope ps(FE_PHASE_TRANSFER, l, s);
-    launch_prolong<T>(h, l, lv_x<T>(Lc), x, true, s, xs);
+    OperatorNext<T> next;
+    next.xs = xs;
+    if (scatters(h, l, dtype)) next.y = y;
+    launch_prolong<T>(h, l, lv_x<T>(Lc), x, true, s, next);
   }
   PhaseScope ps(FE_PHASE_SMOOTH, l, s);
-  smooth_enqueue<T>(h, l, b, x, y, d, g_sp.steps, g_sp.lo, g_sp.hi, false, dtype, s, xs != nullptr, false);
+  smooth_enqueue<T>(h, l, b, x, y, d, g_sp.steps, g_sp.lo, g_sp.hi, false, dtype, s, true, false);
 }
 
 // Enqueue one fine-level V-cycle (reads L.b of the finest level, writes
@@ -1475,8 +1494,8 @@ int fe_apply_operator(const fe_hierarchy* hc, int level, const void* x, void* y,
     const double* xd = stage_in<double>(h, 0, (const double*)x, L.n, s);
     double* yd = stage_out<double>(h, 1, (double*)y, L.n);
     if (presplit(h, level)) {  // the solver's operator: x split into float pairs first
-      launch_split_pairs(L, xd, s);
-      apply_enqueue(h, level, xd, yd, dtype, s, L.xs64.p);
+      launch_split_pairs(L, xd, yd, s);
+      apply_enqueue(h, level, xd, yd, dtype, s, L.xs64.p, true);
     } else {
       apply_enqueue(h, level, xd, yd, dtype, s);
     }

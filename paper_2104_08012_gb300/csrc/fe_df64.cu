@@ -704,8 +704,8 @@ static void apply_df_geo(const Level& L, const double* x, const float2* xs, doub
 
 template <bool FUSE>
 static void apply_df(const Level& L, const double* x, const float2* xs, double* y, const ChebFuse<double>& cf,
-                     cudaStream_t s) {
-  CUDA_CHECK(cudaMemsetAsync(y, 0, sizeof(double) * (size_t)L.n, s));
+                     cudaStream_t s, bool y_zero = false) {
+  if (!y_zero) CUDA_CHECK(cudaMemsetAsync(y, 0, sizeof(double) * (size_t)L.n, s));
   if constexpr (FUSE) {
     if (L.deg == 1)
       apply_df_launch<1, true, false, false>(L, x, nullptr, y, cf, s);
@@ -750,19 +750,22 @@ void launch_apply64_cube_df(const Level& L, const double* x, double* y, cudaStre
   apply_cube_df<false>(L, x, y, ChebFuse<double>{}, s);
 }
 
-void launch_apply64_df(const Level& L, const double* x, double* y, cudaStream_t s, const float2* xs) {
-  apply_df<false>(L, x, xs, y, ChebFuse<double>{}, s);
+void launch_apply64_df(const Level& L, const double* x, double* y, cudaStream_t s, const float2* xs, bool y_zero) {
+  apply_df<false>(L, x, xs, y, ChebFuse<double>{}, s, y_zero);
 }
 
-__global__ void k_split_pairs(int n, const double* __restrict__ x, float2* __restrict__ xs) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) xs[i] = split_pair(x[i]);
+__global__ void k_split_pairs(int n, const double* __restrict__ x, float2* __restrict__ xs, double* __restrict__ y) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    xs[i] = split_pair(x[i]);
+    y[i] = 0.0;
+  }
 }
 
-void launch_split_pairs(const Level& L, const double* x, cudaStream_t s) {
+void launch_split_pairs(const Level& L, const double* x, double* y, cudaStream_t s) {
   FE_REQUIRE(L.xs64.p, FE_ERR_UNSUPPORTED, "this level keeps no float-pair copy of x");
   static int g = 0;
   if (!g) g = resident_grid(k_split_pairs, kBlock, 1 << 30);
-  k_split_pairs<<<std::min(g, std::max(1, ceil_div(L.n, kBlock))), kBlock, 0, s>>>(L.n, x, L.xs64.p);
+  k_split_pairs<<<std::min(g, std::max(1, ceil_div(L.n, kBlock))), kBlock, 0, s>>>(L.n, x, L.xs64.p, y);
   LAUNCH_CHECK();
 }
 

@@ -439,17 +439,19 @@ struct fe_hierarchy {
 void launch_build_level(Level& L, cudaStream_t s);
 void launch_geometry(Level& L, cudaStream_t s);
 void launch_apply64(const Level& L, const double* x, double* y, cudaStream_t s);
-void launch_apply32(const Level& L, const float* x, float* y, cudaStream_t s);
+// y_zero: y is zero already (an OperatorNext of the kernel that wrote x)
+void launch_apply32(const Level& L, const float* x, float* y, cudaStream_t s, bool y_zero = false);
 // xs (optional): x as unscaled float pairs (split_pair), gathered instead of x
-void launch_apply64_df(const Level& L, const double* x, double* y, cudaStream_t s, const float2* xs = nullptr);
+void launch_apply64_df(const Level& L, const double* x, double* y, cudaStream_t s, const float2* xs = nullptr,
+                       bool y_zero = false);
 // x as the float pairs the pre-split P2 operator gathers (into L.xs64), for an application whose input no vector
-// kernel has split.
-void launch_split_pairs(const Level& L, const double* x, cudaStream_t s);
+// kernel has split; y = 0 with it.
+void launch_split_pairs(const Level& L, const double* x, double* y, cudaStream_t s);
 void launch_apply64_cube_df(const Level& L, const double* x, double* y, cudaStream_t s);
 void launch_apply64_df2(const Level& L, const double* x, double* y, cudaStream_t s);
 void launch_apply64_df3(const Level& L, const double* x, double* y, cudaStream_t s);
 // P3 on levels with L.uniform, by the integer element matrix (fe_p3int.cu)
-void launch_apply64_p3(const Level& L, const double* x, double* y, cudaStream_t s);
+void launch_apply64_p3(const Level& L, const double* x, double* y, cudaStream_t s, bool y_zero = false);
 void upload_p3_mass_table(const float* m3i);
 // The same operator kernels with the Chebyshev update fused (y = A x, then
 // d = c1 d + c2 D^-1 (b - y), x += d per dof, in one launch).
@@ -475,11 +477,13 @@ void launch_coarse_assemble_p3(const Level& L0, const int* dof2int, int nci, dou
 // Vertex-star patch smoother (fe_patch.cu; P3 setup in fe_kernels.cu)
 void launch_patch_setup(Level& L, cudaStream_t s);
 void launch_patch_setup_p3(Level& L, cudaStream_t s);
+// z_zero: z is zero already
 template <typename T>
-void launch_patch_apply(const Level& L, const T* b, const T* y, T* z, bool df, cudaStream_t s);
+void launch_patch_apply(const Level& L, const T* b, const T* y, T* z, bool df, cudaStream_t s, bool z_zero = false);
+// y (optional) = 0 for the next operator application, and zero_z: z = 0 after its use for the next product
 template <typename T>
-void launch_cheb_pc(int n, const T* z, T* x, T* d, double c1, double c2, bool first_from_zero, bool store_d,
-                    cudaStream_t s);
+void launch_cheb_pc(int n, T* z, T* x, T* d, double c1, double c2, bool first_from_zero, bool store_d, cudaStream_t s,
+                    T* y = nullptr, bool zero_z = false);
 void launch_split_geometry(Level& L, cudaStream_t s);
 // Checks geo64 = c M cell by cell, fills c32 and cdf and sets L.uniform, L.pair_uniform, L.flux and L.kappa0
 // (synchronises s).  per_cell: treat every level as if the check had failed.
@@ -499,11 +503,18 @@ void launch_centroids(const Level& L, double* xyz, cudaStream_t s);
 void launch_bmask(const Level& L, unsigned char* m, cudaStream_t s);
 void launch_coarsen_kappa(const Level& Lc, const Level& Lf, const int* children, cudaStream_t s);
 int launch_check_positive(const double* v, int n, int* dflag, cudaStream_t s);
+// What the kernel that writes a vector x leaves ready for the operator application that reads it next: x as unscaled
+// float pairs (xs, FP64) and the output that the operator's contributions are added to set to zero (y).  A separate
+// fill costs a launch, 1.2 to 1.5 us and the gap before the next one, per application: P2 40^3 V-cycle 12 of 53 launches.
+template <typename T>
+struct OperatorNext {
+  float2* xs = nullptr;
+  T* y = nullptr;
+};
 // Transfers
-// xs (optional, FP64): also write the result as unscaled float pairs
 template <typename T>
 void launch_prolong(const fe_hierarchy* h, int lf, const T* xc, T* xf, bool accumulate, cudaStream_t s,
-                    float2* xs = nullptr);
+                    OperatorNext<T> next = {});
 // rc = P^T (bf - yf), or P^T bf when yf is null
 template <typename T>
 void launch_restrict(const fe_hierarchy* h, int lf, const T* bf, const T* yf, T* rc, bool zero_bd, cudaStream_t s);
@@ -514,10 +525,10 @@ void launch_restrict_p2(const Level& F, const Level& Cc, const T* b, const T* y,
 void restrict_p2_prepare();
 
 // Vector kernels
-// xs (optional, FP64): also write the new x as unscaled float pairs
+// next.y may be y
 template <typename T>
 void launch_cheb_step(int n, const T* b, const T* y, const T* dinv, T* x, T* d, double c1, double c2, bool first_from_zero,
-                      cudaStream_t s, bool store_d = true, float2* xs = nullptr);
+                      cudaStream_t s, bool store_d = true, OperatorNext<T> next = {});
 // p = z and ps = split_pair(z)
 void launch_copy_split(int n, const double* z, double* p, float2* ps, cudaStream_t s);
 template <typename Ti, typename To>
@@ -563,8 +574,9 @@ void hierarchy_destroy(fe_hierarchy* h);
 template <typename T>
 void vcycle_enqueue(fe_hierarchy* h, int dtype, cudaStream_t s);  // reads L.b of the finest level, writes L.x
 // xs (optional): FP64 x as unscaled float pairs, current with x (the float-pair P2 kernel gathers it)
+// y_zero: y is zero already (used where scatters(h, level, dtype))
 void apply_enqueue(const fe_hierarchy* h, int level, const void* x, void* y, int dtype, cudaStream_t s,
-                   const float2* xs = nullptr);
+                   const float2* xs = nullptr, bool y_zero = false);
 void apply_bf16_enqueue(const Level& L, const float* x, float* y, cudaStream_t s);
 bool bf16_supported();
 int bf16_take_error(cudaStream_t s);      // nonzero if a tensor-core launch gave up a bounded wait

@@ -745,6 +745,13 @@ __global__ void k_check_positive(const double* __restrict__ v, int n, int* __res
   if (!(a > 0.0) || !isfinite(a)) atomicOr(flag, 1);
 }
 
+template <typename T>
+__device__ __forceinline__ void put_next(const OperatorNext<T>& next, int i, T v) {
+  if constexpr (sizeof(T) == 8)
+    if (next.xs) next.xs[i] = fe_df::split_pair(v);
+  if (next.y) next.y[i] = T(0);
+}
+
 // ----------------------------------------------------------- transfers
 // Prolongation: fine lattice point L splits as L = 2k*c + o (c the coarse cube,
 // o in [0,2k)^3); the class o selects a stencil of (coarse lattice point
@@ -754,7 +761,7 @@ __global__ void k_check_positive(const double* __restrict__ v, int n, int* __res
 template <int DEG, typename T>
 __global__ void k_prolong(Numbering nf, int n_f, const int* __restrict__ start, const int4* __restrict__ tab,
                           const T* __restrict__ w, const T* __restrict__ xc, T* __restrict__ xf, int accumulate,
-                          float2* __restrict__ xs) {
+                          OperatorNext<T> next) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_f) return;
   int x, y, z;
@@ -780,8 +787,7 @@ __global__ void k_prolong(Numbering nf, int n_f, const int* __restrict__ start, 
   }
   const T v = accumulate ? xf[i] + s : s;
   xf[i] = v;
-  if constexpr (sizeof(T) == 8)
-    if (xs) xs[i] = fe_df::split_pair(v);  // the operator's next input, ready as a float pair
+  put_next(next, i, v);
 }
 
 // P2 prolongation per coarse cube and fine row: a thread takes coarse cube
@@ -831,13 +837,12 @@ __device__ __forceinline__ T pro_sum(const T (&v)[27], std::integer_sequence<int
 }
 template <int OX, int OY, int OZ, typename T>
 __device__ __forceinline__ void pro_point(const T (&v)[27], int base0, int base1, T* __restrict__ xf, int accumulate,
-                                          float2* __restrict__ xs) {
+                                          const OperatorNext<T>& next) {
   const T s = pro_sum<OX, OY, OZ, T>(v, std::make_integer_sequence<int, 27>{});
   const int i = (OX & 1 ? base1 : base0) + (OX >> 1);
   const T r = accumulate ? xf[i] + s : s;
   xf[i] = r;
-  if constexpr (sizeof(T) == 8)
-    if (xs) xs[i] = fe_df::split_pair(r);  // the operator's next input, ready as a float pair
+  put_next(next, i, r);
 }
 template <int OY, int OZ, typename T, int... N>
 __device__ __forceinline__ void pro_loads(const Numbering& nc, int cx, int cy, int cz, const T* __restrict__ xc,
@@ -848,7 +853,7 @@ __device__ __forceinline__ void pro_loads(const Numbering& nc, int cx, int cy, i
 template <int OY, int OZ, typename T>
 __device__ __forceinline__ void pro_row(const Numbering& nc, const Numbering& nf, int Nc, int cx, int cy, int cz,
                                         const T* __restrict__ xc, T* __restrict__ xf, int accumulate,
-                                        float2* __restrict__ xs) {
+                                        const OperatorNext<T>& next) {
   T v[27];
   pro_loads<OY, OZ>(nc, cx, cy, cz, xc, v, std::make_integer_sequence<int, 27>{});
   // fine dofs of the row: parity class by ox & 1, the y and z parts fixed
@@ -856,32 +861,32 @@ __device__ __forceinline__ void pro_row(const Numbering& nc, const Numbering& nf
   constexpr int c0 = p2_class(0, OY & 1, OZ & 1), c1 = p2_class(1, OY & 1, OZ & 1);
   const int base0 = nf.off[c0] + 2 * cx + nf.sx[c0] * (fy + nf.sy[c0] * fz);
   const int base1 = nf.off[c1] + 2 * cx + nf.sx[c1] * (fy + nf.sy[c1] * fz);
-  pro_point<0, OY, OZ>(v, base0, base1, xf, accumulate, xs);
-  pro_point<1, OY, OZ>(v, base0, base1, xf, accumulate, xs);
-  pro_point<2, OY, OZ>(v, base0, base1, xf, accumulate, xs);
-  pro_point<3, OY, OZ>(v, base0, base1, xf, accumulate, xs);
-  if (cx == Nc - 1) pro_point<4, OY, OZ>(v, base0, base1, xf, accumulate, xs);
+  pro_point<0, OY, OZ>(v, base0, base1, xf, accumulate, next);
+  pro_point<1, OY, OZ>(v, base0, base1, xf, accumulate, next);
+  pro_point<2, OY, OZ>(v, base0, base1, xf, accumulate, next);
+  pro_point<3, OY, OZ>(v, base0, base1, xf, accumulate, next);
+  if (cx == Nc - 1) pro_point<4, OY, OZ>(v, base0, base1, xf, accumulate, next);
 }
 
 template <int R, typename T>
 __device__ __forceinline__ void pro_row_dispatch(int row, const Numbering& nc, const Numbering& nf, int Nc, int cx,
-                                                 int cy, int cz, const T* xc, T* xf, int accumulate, float2* xs) {
+                                                 int cy, int cz, const T* xc, T* xf, int accumulate, const OperatorNext<T>& next) {
   if (row == R)
-    pro_row<R % 5, R / 5, T>(nc, nf, Nc, cx, cy, cz, xc, xf, accumulate, xs);
+    pro_row<R % 5, R / 5, T>(nc, nf, Nc, cx, cy, cz, xc, xf, accumulate, next);
   else if constexpr (R + 1 < 25)
-    pro_row_dispatch<R + 1, T>(row, nc, nf, Nc, cx, cy, cz, xc, xf, accumulate, xs);
+    pro_row_dispatch<R + 1, T>(row, nc, nf, Nc, cx, cy, cz, xc, xf, accumulate, next);
 }
 
 template <typename T>
 __global__ void __launch_bounds__(128) k_prolong_cube(Numbering nc, Numbering nf, int Nc, int nby,
                                                       const T* __restrict__ xc, T* __restrict__ xf, int accumulate,
-                                                      float2* __restrict__ xs) {
+                                                      OperatorNext<T> next) {
   const int row = blockIdx.y / nby;  // uniform per block
   const int cx = blockIdx.x * 32 + threadIdx.x, cy = (blockIdx.y - row * nby) * 4 + threadIdx.y, cz = blockIdx.z;
   if (cx >= Nc || cy >= Nc) return;
   const int oy = row % 5, oz = row / 5;
   if ((oy == 4 && cy != Nc - 1) || (oz == 4 && cz != Nc - 1)) return;
-  pro_row_dispatch<0, T>(row, nc, nf, Nc, cx, cy, cz, xc, xf, accumulate, xs);
+  pro_row_dispatch<0, T>(row, nc, nf, Nc, cx, cy, cz, xc, xf, accumulate, next);
 }
 
 // Restriction = exact transpose: coarse point Lc gathers fine points
@@ -943,9 +948,9 @@ __global__ void __launch_bounds__(32 * TPC) k_restrict(int mf, Numbering nc, int
 // Chebyshev step: d = c1 d + c2 D^-1 (b - y); x += d  (y = A x).  With
 // first_from_zero (x = 0, y unused): d = c2 D^-1 b; x = d.
 template <typename T>
-__global__ void k_cheb_step(int n, const T* __restrict__ b, const T* __restrict__ y, const T* __restrict__ dinv,
+__global__ void k_cheb_step(int n, const T* __restrict__ b, const T* y, const T* __restrict__ dinv,
                             T* __restrict__ x, T* __restrict__ d, T c1, T c2, int first_from_zero, int store_d,
-                            float2* __restrict__ xs) {
+                            OperatorNext<T> next) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   T xn;
@@ -959,16 +964,15 @@ __global__ void k_cheb_step(int n, const T* __restrict__ b, const T* __restrict_
     xn = x[i] + dn;
   }
   x[i] = xn;
-  if constexpr (sizeof(T) == 8)
-    if (xs) xs[i] = fe_df::split_pair(xn);  // the operator's next input, ready as a float pair
+  put_next(next, i, xn);
 }
 
 // The FP64 step with two dofs per thread: 16-byte loads and stores (every
 // pointer 16-byte aligned), so a warp keeps twice the bytes in flight per
 // load instruction; the last thread takes the odd dof of an odd n.
-__global__ void k_cheb_step2(int n, const double* __restrict__ b, const double* __restrict__ y,
+__global__ void k_cheb_step2(int n, const double* __restrict__ b, const double* y,
                              const double* __restrict__ dinv, double* __restrict__ x, double* __restrict__ d, double c1,
-                             double c2, int first_from_zero, int store_d, float2* __restrict__ xs) {
+                             double c2, int first_from_zero, int store_d, OperatorNext<double> next) {
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   const int i = 2 * t;
   if (i >= n) return;
@@ -984,7 +988,7 @@ __global__ void k_cheb_step2(int n, const double* __restrict__ b, const double* 
       xn = x[i] + dn;
     }
     x[i] = xn;
-    if (xs) xs[i] = fe_df::split_pair(xn);
+    put_next(next, i, xn);
     return;
   }
   const double2 bb = *reinterpret_cast<const double2*>(b + i), dd = *reinterpret_cast<const double2*>(dinv + i);
@@ -1002,9 +1006,10 @@ __global__ void k_cheb_step2(int n, const double* __restrict__ b, const double* 
     xn = make_double2(xo.x + dn.x, xo.y + dn.y);
   }
   *reinterpret_cast<double2*>(x + i) = xn;
-  if (xs) {
+  if (next.y) *reinterpret_cast<double2*>(next.y + i) = make_double2(0.0, 0.0);
+  if (next.xs) {
     const float2 p0 = fe_df::split_pair(xn.x), p1 = fe_df::split_pair(xn.y);
-    *reinterpret_cast<float4*>(xs + i) = make_float4(p0.x, p0.y, p1.x, p1.y);
+    *reinterpret_cast<float4*>(next.xs + i) = make_float4(p0.x, p0.y, p1.x, p1.y);
   }
 }
 
@@ -1313,8 +1318,8 @@ void launch_geometry(Level& L, cudaStream_t s) {
 }
 
 template <typename T>
-static void apply_impl(const Level& L, const T* geo, const T* x, T* y, cudaStream_t s) {
-  CUDA_CHECK(cudaMemsetAsync(y, 0, sizeof(T) * (size_t)L.n, s));
+static void apply_impl(const Level& L, const T* geo, const T* x, T* y, cudaStream_t s, bool y_zero = false) {
+  if (!y_zero) CUDA_CHECK(cudaMemsetAsync(y, 0, sizeof(T) * (size_t)L.n, s));
   const int Cpad = ceil_div(L.C, kBlock) * kBlock;
   const int grid = ceil_div((long long)Cpad + L.nb, kBlock);
   by_degree(L.deg, [&](auto D) {
@@ -1327,8 +1332,9 @@ static void apply_impl(const Level& L, const T* geo, const T* x, T* y, cudaStrea
 }
 
 template <bool FUSE>
-static void apply_cube32(const Level& L, const float* x, float* y, const ChebFuse<float>& cf, cudaStream_t s) {
-  CUDA_CHECK(cudaMemsetAsync(y, 0, sizeof(float) * (size_t)L.n, s));
+static void apply_cube32(const Level& L, const float* x, float* y, const ChebFuse<float>& cf, cudaStream_t s,
+                         bool y_zero = false) {
+  if (!y_zero) CUDA_CHECK(cudaMemsetAsync(y, 0, sizeof(float) * (size_t)L.n, s));
   const int Qpad = ceil_div(L.Q, kCubeBlock) * kCubeBlock;
   const int grid = ceil_div((long long)Qpad + L.nb, kCubeBlock);
   // c32 rows start at multiples of 24 bytes per cube: the UNI kernel's float2 loads stay 8-byte aligned
@@ -1373,11 +1379,11 @@ void launch_build_valence(Level& L, cudaStream_t s) {
 }
 
 void launch_apply64(const Level& L, const double* x, double* y, cudaStream_t s) { apply_impl<double>(L, L.geo64, x, y, s); }
-void launch_apply32(const Level& L, const float* x, float* y, cudaStream_t s) {
+void launch_apply32(const Level& L, const float* x, float* y, cudaStream_t s, bool y_zero) {
   if (L.deg == 3)  // P3: one thread per tet (a P3 cube holds 64 dofs and 6 x 20 x 20 products)
-    apply_impl<float>(L, L.geo32, x, y, s);
+    apply_impl<float>(L, L.geo32, x, y, s, y_zero);
   else
-    apply_cube32<false>(L, x, y, ChebFuse<float>{}, s);
+    apply_cube32<false>(L, x, y, ChebFuse<float>{}, s, y_zero);
 }
 
 void launch_mass(const Level& L, const double* x, double* y, cudaStream_t s) {
@@ -1453,7 +1459,8 @@ template <>
 const float* tt_weights<float>(const DBuf<double>&, const DBuf<float>& wf) { return wf.p; }
 
 template <typename T>
-void launch_prolong(const fe_hierarchy* h, int lf, const T* xc, T* xf, bool accumulate, cudaStream_t s, float2* xs) {
+void launch_prolong(const fe_hierarchy* h, int lf, const T* xc, T* xf, bool accumulate, cudaStream_t s,
+                    OperatorNext<T> next) {
   const Level& F = h->L[lf];
   const TransferTables& t = h->tt;
   // the per-cube kernel's blocks span 32 cubes along x: on coarse levels with
@@ -1463,14 +1470,14 @@ void launch_prolong(const fe_hierarchy* h, int lf, const T* xc, T* xf, bool accu
     const Level& Cl = h->L[lf - 1];
     const int Nc = Cl.N, nby = ceil_div(Nc, 4);
     const dim3 grid(ceil_div(Nc, 32), nby * 25, Nc), block(32, 4);
-    k_prolong_cube<T><<<grid, block, 0, s>>>(Cl.num, F.num, Nc, nby, xc, xf, accumulate, xs);
+    k_prolong_cube<T><<<grid, block, 0, s>>>(Cl.num, F.num, Nc, nby, xc, xf, accumulate, next);
     LAUNCH_CHECK();
     return;
   }
   by_degree(h->deg, [&](auto D) {
     k_prolong<D.value, T><<<ceil_div(F.n, kBlock), kBlock, 0, s>>>(F.num, F.n, t.pro_start, F.ptab,
                                                                   tt_weights<T>(t.pro_w, t.pro_wf), xc, xf, accumulate,
-                                                                  xs);
+                                                                  next);
   });
   LAUNCH_CHECK();
 }
@@ -1512,33 +1519,35 @@ void launch_restrict(const fe_hierarchy* h, int lf, const T* bf, const T* yf, T*
   LAUNCH_CHECK();
 }
 
-template void launch_prolong<double>(const fe_hierarchy*, int, const double*, double*, bool, cudaStream_t, float2*);
-template void launch_prolong<float>(const fe_hierarchy*, int, const float*, float*, bool, cudaStream_t, float2*);
+template void launch_prolong<double>(const fe_hierarchy*, int, const double*, double*, bool, cudaStream_t,
+                                     OperatorNext<double>);
+template void launch_prolong<float>(const fe_hierarchy*, int, const float*, float*, bool, cudaStream_t,
+                                    OperatorNext<float>);
 template void launch_restrict<double>(const fe_hierarchy*, int, const double*, const double*, double*, bool,
                                       cudaStream_t);
 template void launch_restrict<float>(const fe_hierarchy*, int, const float*, const float*, float*, bool, cudaStream_t);
 
 template <typename T>
 void launch_cheb_step(int n, const T* b, const T* y, const T* dinv, T* x, T* d, double c1, double c2,
-                      bool first_from_zero, cudaStream_t s, bool store_d, float2* xs) {
+                      bool first_from_zero, cudaStream_t s, bool store_d, OperatorNext<T> next) {
   if constexpr (sizeof(T) == 8) {
     auto a16 = [](const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; };
-    if (a16(b) && a16(y) && a16(dinv) && a16(x) && a16(d) && a16(xs)) {  // null pointers count as aligned
+    if (a16(b) && a16(y) && a16(dinv) && a16(x) && a16(d) && a16(next.xs) && a16(next.y)) {  // null pointers count as aligned
       k_cheb_step2<<<ceil_div(ceil_div(n, 2), kBlock), kBlock, 0, s>>>(n, (const double*)b, (const double*)y,
                                                                       (const double*)dinv, (double*)x, (double*)d, c1,
-                                                                      c2, first_from_zero ? 1 : 0, store_d ? 1 : 0, xs);
+                                                                      c2, first_from_zero ? 1 : 0, store_d ? 1 : 0, next);
       LAUNCH_CHECK();
       return;
     }
   }
   k_cheb_step<T><<<ceil_div(n, kBlock), kBlock, 0, s>>>(n, b, y, dinv, x, d, (T)c1, (T)c2, first_from_zero ? 1 : 0,
-                                                        store_d ? 1 : 0, xs);
+                                                        store_d ? 1 : 0, next);
   LAUNCH_CHECK();
 }
 template void launch_cheb_step<double>(int, const double*, const double*, const double*, double*, double*, double,
-                                       double, bool, cudaStream_t, bool, float2*);
+                                       double, bool, cudaStream_t, bool, OperatorNext<double>);
 template void launch_cheb_step<float>(int, const float*, const float*, const float*, float*, float*, double, double,
-                                      bool, cudaStream_t, bool, float2*);
+                                      bool, cudaStream_t, bool, OperatorNext<float>);
 
 template <typename Ti, typename To>
 void launch_convert(int n, const Ti* in, To* out, cudaStream_t s) {

@@ -83,8 +83,8 @@ __global__ void __launch_bounds__(kBlock, 3)
 
 }  // namespace
 
-void launch_apply64_p3(const Level& L, const double* x, double* y, cudaStream_t s) {
-  CUDA_CHECK(cudaMemsetAsync(y, 0, sizeof(double) * (size_t)L.n, s));
+void launch_apply64_p3(const Level& L, const double* x, double* y, cudaStream_t s, bool y_zero) {
+  if (!y_zero) CUDA_CHECK(cudaMemsetAsync(y, 0, sizeof(double) * (size_t)L.n, s));
   static int g = 0;
   if (!g) g = resident_grid(k_apply_p3_int, kBlock, 1 << 30);
   const int grid = std::max(1, std::min(g, (std::max(L.C, L.nb) + kBlock - 1) / kBlock));

@@ -396,13 +396,15 @@ __global__ void __launch_bounds__(32 * kWarpsP3, 6) k_patch_apply_p3(int P, cons
 // Chebyshev step with a preconditioned residual z: d = c1 d + c2 z, x += d
 // (first_from_zero: x = d = c2 z).
 template <typename T>
-__global__ void k_cheb_pc(int n, const T* __restrict__ z, T* __restrict__ x, T* __restrict__ d, T c1, T c2,
-                          int first_from_zero, int store_d) {
+__global__ void k_cheb_pc(int n, T* __restrict__ z, T* __restrict__ x, T* __restrict__ d, T c1, T c2,
+                          int first_from_zero, int store_d, T* __restrict__ y, int zero_z) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const T dn = (c1 != T(0) && !first_from_zero ? c1 * d[i] : T(0)) + c2 * z[i];
   if (store_d) d[i] = dn;
   x[i] = first_from_zero ? dn : x[i] + dn;
+  if (y) y[i] = T(0);
+  if (zero_z) z[i] = T(0);
 }
 
 template <typename T>
@@ -440,9 +442,9 @@ void launch_patch_setup(Level& L, cudaStream_t s) {
 }
 
 template <typename T>
-void launch_patch_apply(const Level& L, const T* b, const T* y, T* z, bool df, cudaStream_t s) {
+void launch_patch_apply(const Level& L, const T* b, const T* y, T* z, bool df, cudaStream_t s, bool z_zero) {
   const int P = L.V, Pp = (P + 127) / 128 * 128, Ppad = ceil_div(P, kBlock) * kBlock;
-  CUDA_CHECK(cudaMemsetAsync(z, 0, sizeof(T) * (size_t)L.n, s));
+  if (!z_zero) CUDA_CHECK(cudaMemsetAsync(z, 0, sizeof(T) * (size_t)L.n, s));
   if (L.deg == 3) {  // P3: the FP64 product always in float pairs
     (void)df;
     k_patch_apply_p3<T><<<ceil_div(P, kWarpsP3), 32 * kWarpsP3, 0, s>>>(P, L.pdof, L.pinvdf, L.pinv32, b, y, z, L.nb,
@@ -464,14 +466,15 @@ void launch_patch_apply(const Level& L, const T* b, const T* y, T* z, bool df, c
 }
 
 template <typename T>
-void launch_cheb_pc(int n, const T* z, T* x, T* d, double c1, double c2, bool first_from_zero, bool store_d,
-                    cudaStream_t s) {
+void launch_cheb_pc(int n, T* z, T* x, T* d, double c1, double c2, bool first_from_zero, bool store_d, cudaStream_t s,
+                    T* y, bool zero_z) {
   k_cheb_pc<T><<<ceil_div(n, kBlock), kBlock, 0, s>>>(n, z, x, d, (T)c1, (T)c2, first_from_zero ? 1 : 0,
-                                                      store_d ? 1 : 0);
+                                                      store_d ? 1 : 0, y, zero_z ? 1 : 0);
   LAUNCH_CHECK();
 }
 
-template void launch_patch_apply<double>(const Level&, const double*, const double*, double*, bool, cudaStream_t);
-template void launch_patch_apply<float>(const Level&, const float*, const float*, float*, bool, cudaStream_t);
-template void launch_cheb_pc<double>(int, const double*, double*, double*, double, double, bool, bool, cudaStream_t);
-template void launch_cheb_pc<float>(int, const float*, float*, float*, double, double, bool, bool, cudaStream_t);
+template void launch_patch_apply<double>(const Level&, const double*, const double*, double*, bool, cudaStream_t, bool);
+template void launch_patch_apply<float>(const Level&, const float*, const float*, float*, bool, cudaStream_t, bool);
+template void launch_cheb_pc<double>(int, double*, double*, double*, double, double, bool, bool, cudaStream_t, double*,
+                                     bool);
+template void launch_cheb_pc<float>(int, float*, float*, float*, double, double, bool, bool, cudaStream_t, float*, bool);
