@@ -21,51 +21,54 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
-// Block-reduce NV values; in the last block of the grid, thread 0 returns
-// true with the grid totals in out[].
+// Sums of NV values over the block, in thread 0.  Every FP64 instruction of a warp
+// holds its scheduler's FP64 pipe for 64 clocks, so shuffling all 16 warps down to
+// one value each (5 such instructions per warp and value, 1.3 us for the two blocks
+// of an SM) costs more than the loads of a short vector: here the values meet in
+// shared memory, 4 warps add four each, one warp four more, and only that one
+// shuffles (11 instructions in a row instead of 25 to 45; P1 16^3 solve 702 -> 676
+// us, P1 96^3 gradient 20.6 -> 20.1 ms).
 template <int NV>
-__device__ bool grid_reduce(double (&v)[NV], double* __restrict__ partials, unsigned int* __restrict__ counter,
-                            double (&out)[NV]) {
-  __shared__ double sh[NV][kRedBlock / 32];
-  __shared__ bool last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int nw = kRedBlock / 32;
+__device__ __forceinline__ void block_sum(double (&v)[NV], double (&sh)[NV][kRedBlock]) {
+  const int t = threadIdx.x;
 #pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    const double s = warp_sum(v[k]);
-    if (lane == 0) sh[k][warp] = s;
+  for (int k = 0; k < NV; ++k) sh[k][t] = v[k];
+  __syncthreads();
+  if (t < kRedBlock / 4) {
+    constexpr int q = kRedBlock / 4;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) sh[k][t] = (sh[k][t] + sh[k][t + q]) + (sh[k][t + 2 * q] + sh[k][t + 3 * q]);
   }
   __syncthreads();
-  if (warp == 0) {
+  if (t < 32) {
+    static_assert(kRedBlock / 4 == 128, "four values per lane");
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double s = lane < nw ? sh[k][lane] : 0.0;
-      s = warp_sum(s);
-      if (lane == 0) partials[k * gridDim.x + blockIdx.x] = s;
-    }
-    if (lane == 0) {
-      __threadfence();
-      const unsigned int ticket = atomicAdd(counter, 1u);
-      last = (ticket == gridDim.x - 1);
-    }
+    for (int k = 0; k < NV; ++k) v[k] = warp_sum((sh[k][t] + sh[k][t + 32]) + (sh[k][t + 64] + sh[k][t + 96]));
+  }
+}
+
+// Reduces NV values; in the last block of the grid, thread 0 returns true with
+// the grid totals in v[].
+template <int NV>
+__device__ bool grid_reduce(double (&v)[NV], double* __restrict__ partials, unsigned int* __restrict__ counter) {
+  __shared__ double sh[NV][kRedBlock];
+  __shared__ bool last;
+  block_sum(v, sh);
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int k = 0; k < NV; ++k) partials[k * gridDim.x + blockIdx.x] = v[k];
+    __threadfence();
+    last = atomicAdd(counter, 1u) == gridDim.x - 1;
   }
   __syncthreads();
   if (!last) return false;
   __threadfence();
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
-    double s = 0.0;
-    for (int i = threadIdx.x; i < (int)gridDim.x; i += kRedBlock) s += __ldcg(partials + k * gridDim.x + i);
-    s = warp_sum(s);
-    __syncthreads();
-    if (lane == 0) sh[k][warp] = s;
-    __syncthreads();
-    if (warp == 0) {
-      double t = lane < nw ? sh[k][lane] : 0.0;
-      t = warp_sum(t);
-      if (lane == 0) out[k] = t;
-    }
+    v[k] = 0.0;
+    for (int i = threadIdx.x; i < (int)gridDim.x; i += kRedBlock) v[k] += __ldcg(partials + k * gridDim.x + i);
   }
+  block_sum(v, sh);
   if (threadIdx.x == 0) *counter = 0u;
   return threadIdx.x == 0;
 }
@@ -131,18 +134,16 @@ template <typename T>
 __global__ void __launch_bounds__(kRedBlock) k_dot(int n, const T* __restrict__ a, const T* __restrict__ b,
                                                    double* partials, unsigned int* counter, double* scal, int slot) {
   double v[1] = {slice_dot(n, a, b)};
-  double out[1];
-  if (grid_reduce<1>(v, partials, counter, out)) scal[slot] = out[0];
+  if (grid_reduce<1>(v, partials, counter)) scal[slot] = v[0];
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kRedBlock) k_cg_alpha(int n, const T* __restrict__ p, const T* __restrict__ q,
                                                         double* partials, unsigned int* counter, double* scal) {
   double v[1] = {slice_dot(n, p, q)};
-  double out[1];
-  if (grid_reduce<1>(v, partials, counter, out)) {
-    scal[S_PQ] = out[0];
-    scal[S_ALPHA] = scal[S_RZ] / out[0];
+  if (grid_reduce<1>(v, partials, counter)) {
+    scal[S_PQ] = v[0];
+    scal[S_ALPHA] = scal[S_RZ] / v[0];
   }
 }
 
@@ -178,15 +179,17 @@ __global__ void __launch_bounds__(kRedBlock)
     for (int u = 0; u < kUnroll; ++u) one(i + u * G, xv[u], pv[u], rv[u], qv[u]);
   }
   for (; i < n; i += G) one(i, x[i], p[i], r[i], q[i]);
+  if (!dinv) {
+    double v[1] = {rr.value()};
+    if (grid_reduce<1>(v, partials, counter)) scal[S_RR] = v[0];
+    return;
+  }
   double v[2] = {rr.value(), rz.value()};
-  double out[2];
-  if (grid_reduce<2>(v, partials, counter, out)) {
-    scal[S_RR] = out[0];
-    if (dinv) {
-      scal[S_RZNEW] = out[1];
-      scal[S_BETA] = out[1] / scal[S_RZ];
-      scal[S_RZ] = out[1];
-    }
+  if (grid_reduce<2>(v, partials, counter)) {
+    scal[S_RR] = v[0];
+    scal[S_RZNEW] = v[1];
+    scal[S_BETA] = v[1] / scal[S_RZ];
+    scal[S_RZ] = v[1];
   }
 }
 
@@ -194,11 +197,10 @@ template <typename T>
 __global__ void __launch_bounds__(kRedBlock) k_cg_beta(int n, const T* __restrict__ r, const T* __restrict__ z,
                                                        double* partials, unsigned int* counter, double* scal) {
   double v[1] = {slice_dot(n, r, z)};
-  double out[1];
-  if (grid_reduce<1>(v, partials, counter, out)) {
-    scal[S_RZNEW] = out[0];
-    scal[S_BETA] = out[0] / scal[S_RZ];
-    scal[S_RZ] = out[0];
+  if (grid_reduce<1>(v, partials, counter)) {
+    scal[S_RZNEW] = v[0];
+    scal[S_BETA] = v[0] / scal[S_RZ];
+    scal[S_RZ] = v[0];
   }
 }
 
