@@ -1486,7 +1486,9 @@ void launch_prolong(const fe_hierarchy* h, int lf, const T* xc, T* xf, bool accu
 // points instead of 8: with fewer blocks than SMs there, a P2 vertex's 125
 // entries in chains of 16 per thread left them latency-bound (P2 16^3 -> 8^3,
 // 4,913 coarse dofs: 16.5 -> 9.1 us).  At 35,937 coarse dofs (32^3 -> 16^3)
-// the 1024-thread blocks were slower (14.0 -> 18.5 us).
+// the 1024-thread blocks were slower (14.0 -> 18.5 us).  P3, whose points gather up
+// to 343 entries, takes 32 and 16 warps (8, 16 and 32: 20.9, 12.3 and 11.4 us to
+// 4^3, 37.5, 23.6 and 21.5 to 8^3, 75, 73 and 92 to 16^3).
 constexpr int kRestrictWideBelow = 1 << 14;
 
 constexpr int kRestrictTiledFrom = 32;  // coarse cubes per axis: below, the tiles are too few to hide their latency
@@ -1512,10 +1514,14 @@ void launch_restrict(const fe_hierarchy* h, int lf, const T* bf, const T* yf, T*
     k_restrict<2, T, 8><<<ceil_div(Cc.n, 32), 32 * 8, 0, s>>>(F.num.m, Cc.num, Cc.n, t.res_margin, t.res_start,
                                                               F.rtab, tt_weights<T>(t.res_w, t.res_wf), bf,
                                                               yf, rc, zero_bd);
+  else if (Cc.n < kRestrictWideBelow)
+    k_restrict<3, T, 32><<<ceil_div(Cc.n, 32), 32 * 32, 0, s>>>(F.num.m, Cc.num, Cc.n, t.res_margin, t.res_start,
+                                                                F.rtab, tt_weights<T>(t.res_w, t.res_wf), bf,
+                                                                yf, rc, zero_bd);
   else
-    k_restrict<3, T, 8><<<ceil_div(Cc.n, 32), 32 * 8, 0, s>>>(F.num.m, Cc.num, Cc.n, t.res_margin, t.res_start,
-                                                              F.rtab, tt_weights<T>(t.res_w, t.res_wf), bf,
-                                                              yf, rc, zero_bd);
+    k_restrict<3, T, 16><<<ceil_div(Cc.n, 32), 32 * 16, 0, s>>>(F.num.m, Cc.num, Cc.n, t.res_margin, t.res_start,
+                                                                F.rtab, tt_weights<T>(t.res_w, t.res_wf), bf,
+                                                                yf, rc, zero_bd);
   LAUNCH_CHECK();
 }
 

@@ -195,6 +195,18 @@ def test_fp64_tiled_restriction_matches_table(fe, N0):
             assert (a - b).nan_to_num().abs().max() <= 2 * 125 * 125 * 2.0 ** -53
 
 
+@pytest.mark.parametrize("N0", [2, 8, 9])
+def test_p3_restriction_is_the_transpose(fe, N0):
+    """P3 restriction by 32 warps per 32 coarse points (8^3, 15,625 points, the largest) and by 16 (9^3): (P c) . r = c . (R r)
+    to the rounding of sums of n terms, each entry of at most 343 (1e-12 of the norms' product)."""
+    with fe.Hierarchy(N0, 1, 3) as h:
+        r, c = dt(I.random_vector(h.n_dofs(), 3)), dt(I.random_vector(h.n_dofs(0), 4))
+        rc, pc = torch.empty_like(c), torch.empty_like(r)
+        h.restrict(r, rc, 1, zero_boundary=False)
+        h.prolong(c, pc, 1)
+        assert abs(float(pc @ r - c @ rc)) <= 1e-12 * float(pc.norm() * r.norm())
+
+
 @pytest.mark.parametrize("dtype", ["f64", "f32"])
 def test_vcycle_replayed_and_captured(fe, dtype):
     """The V-cycle's later calls replay its graph: with new inputs, other buffers and a changed coefficient they equal the
