@@ -36,25 +36,21 @@ WORKLOAD = {"workload": "poisson_p2_unitcube64_gmg4_fp64", "mesh": "UnitCubeMesh
             "degree": 2, "levels": 4, "coarse_mesh": 8, "cells": 1572864, "dofs": 2146689, "rtol": 1e-8,
             "preconditioner": "GMG V(2,2) Chebyshev-Jacobi + FP64 Cholesky coarse", "l2_between_steps": "flushed"}
 F64_MODE = 1  # FE_F64_DOUBLE_FLOAT: the library default for FP64 operator applications
-# Algorithmic bytes per dof of one matrix-free application (each array counted once; P2, kappa = 1):
-# x read + y write (8 + 8 in FP64, 4 + 4 in FP32), tet->dof map (0.75 tets/dof x 10 x 4 B = 30 B),
-# vertex coordinates (1/8 vertex per dof x 24 B = 3 B).
-BYTES_PER_DOF_P2 = {"f64": 49.0, "f32": 41.0}
+# Algorithmic bytes per dof of one matrix-free application (each array counted once; P2, kappa = 1): by rows x read +
+# y write (8 + 8 in FP64, 4 + 4 in FP32); the element form (bf16) also the tet->dof map (0.75 tets/dof x 10 x 4 B =
+# 30 B) and the vertex coordinates (1/8 vertex per dof x 24 B = 3 B).
+BYTES_PER_DOF_P2 = {"f64": 16.0, "f32": 8.0, "bf16": 41.0}
 # DRAM bytes per launch of the FP64 operator kernel on this workload (dram__bytes_read.sum +
 # dram__bytes_write.sum from one ncu capture of the finest level's applications inside a V-cycle of the
-# P2 64^3 hierarchy, the kernel the CG iterations run; mean of 2 launches), keyed by FP64 mode; None where
-# the kernel changed after the last capture.
-TRAFFIC = {0: None, 1: 116.4e6, 2: None}
-# Arithmetic of one P2 element application (c, d, S, four G-products, transpose),
-# per tet: 151 flops in the FP64 formula with a general G (an FMA counts 2).  With
-# the geometric matrix shared by every Kuhn tet (G = c M) the element matrix is
-# c times one integer matrix K (82 nonzeros), applied by fixed-point limbs to
-# the two tets that share a face as one unit (14 dofs, 136 nonzero integers):
-# per pair 674 FP32 operations (an add, mul or FMA counts 1) = 14 products c x
-# as float pairs x 4, their cut into three limbs x 8 additions, 136 x 3 FMAs,
-# and per row one TwoSum (6) and one addition; 337 per tet.
+# P2 64^3 hierarchy, the kernel the CG iterations run; mean of 2 launches), keyed by FP64 mode (1:
+# x read once, y and the halo re-reads stay in L2); None where there is no capture.
+TRAFFIC = {0: None, 1: 17.6e6, 2: None}
+# Native FP64 P2 element application (c, d, S, four G-products, transpose), per tet:
+# 151 flops (an FMA counts 2).  By rows (k_stencil2): 177 instructions per dof
+# counted by ncu (smsp__inst_executed x 32 / dofs), staging and conversion of the
+# tile's halo included.
 FLOPS_PER_CELL_P2_F64 = 151
-OPS_PER_CELL_P2_DF = 337
+OPS_PER_DOF_P2_ROWS = 177
 # Operations of one P3 element application through the gradient at the P2 nodes (fe_p3.cuh; an FMA counts 1):
 # 206 additions, 165 multiplications, 284 FMAs, 22 negations (counted by tests/test_p3_element_host.py)
 OPS_PER_CELL_P3 = 677
@@ -184,8 +180,8 @@ def extras(fe, I, h, dev, stream, flush):
             for _ in range(3):
                 h.apply_operator(x, y, dtype=dt, stream=stream)
             ms = time_launches(lambda: h.apply_operator(x, y, dtype=dt, stream=stream), stream, 10, flush)
-        byt = apply_bytes_per_launch(n, C, 10, vb, gb, cube)
-        sb = BYTES_PER_DOF_P2["f64" if vb == 8 else "f32"] * n
+        sb = BYTES_PER_DOF_P2[name.split("_")[0]] * n
+        byt = apply_bytes_per_launch(n, C, 10, vb, gb, cube) if dt == fe.FE_BF16 else sb
         mv[name] = {"ms": ms, "GDoF_per_s": n / (ms * 1e-3) / 1e9,
                     "hbm_frac_survey_bytes": sb / (ms * 1e-3) / 1e9 / peak,
                     "GB_per_s_kernel_bytes": byt / (ms * 1e-3) / 1e9,
@@ -261,15 +257,13 @@ def extras(fe, I, h, dev, stream, flush):
         for _ in range(3):
             h2.apply_operator(x32, y32, dtype=fe.FE_F32, stream=stream)
         ms = time_launches(lambda: h2.apply_operator(x32, y32, dtype=fe.FE_F32, stream=stream), stream, 10, flush)
-    byt = apply_bytes_per_launch(n2, h2.n_cells(), 10, 4, 4, cube_map=True)
-    sb = BYTES_PER_DOF_P2["f32"] * n2
+    byt = sb = BYTES_PER_DOF_P2["f32"] * n2
     out["matvec_p2_128cubed_f32"] = {"ms": ms, "GDoF_per_s": n2 / (ms * 1e-3) / 1e9,
                                      "hbm_frac_survey_bytes": sb / (ms * 1e-3) / 1e9 / peak,
                                      "survey_bytes_per_dof": BYTES_PER_DOF_P2["f32"],
                                      "kernel_bytes_per_dof": byt / n2, "GB_per_s_kernel_bytes": byt / (ms * 1e-3) / 1e9,
                                      "hbm_frac_kernel_bytes": byt / (ms * 1e-3) / 1e9 / peak,
-                                     "kernel_bytes_model": "x 4 + y zero-fill and write 8 + cube->dof map 27 x 4 per "
-                                                           "cube + per-tet geometric factors 6 x 4 per tet",
+                                     "kernel_bytes_model": "x 4 + y 4 per dof (rows: no map, no geometry)",
                                      "hbm_peak_gbs": peak, "hbm_peak_source": src}
     del x32, y32
     for name, prec in (("f64", fe.FE_PREC_F64), ("mixed_f32", fe.FE_PREC_MIXED_F32),
@@ -362,7 +356,7 @@ def extras(fe, I, h, dev, stream, flush):
     except Exception as exc:
         p3["quadrature_load_vector"] = {"error": repr(exc)[:300]}
     p3["element_ops_per_tet"] = ops_per_cell
-    p3["apply_f64"]["arithmetic"] = "float pairs on the FP32 pipes (k_apply_df3)"
+    p3["apply_f64"]["arithmetic"] = "integer element matrix in exact 60-bit sums (k_apply_p3_int)"
     p3["apply_f64_native"]["arithmetic"] = "FP64 (k_apply<3, double>)"
     # FP64 issue rate in operations: half the nominal flop rate (an FMA is 2 flops)
     p3["apply_f64_native"]["frac_of_nominal_fp64_rate"] = p3["apply_f64_native"]["element_T_ops_per_s"] / (
@@ -759,13 +753,12 @@ def run_ours(args, rank, world, local_rank, oracle=None):
     byt = BYTES_PER_DOF_P2["f64"] * n
     achieved_gbs = byt / (apply_ms * 1e-3) / 1e9
     if F64_MODE == fe.FE_F64_DOUBLE_FLOAT:
-        kname = ("k_apply_lp<KuhnPair> (FP64 operator on the FP32 pipes: exact fixed-point limbs of c x against the "
-                 "integer stiffness of the two Kuhn tets that share a face, applied as one unit of 14 dofs; "
-                 "persistent, map rows staged in shared memory by cp.async)")
-        ops, opeak, ounit = OPS_PER_CELL_P2_DF * C, FP32_PEAK_TOPS, "T FP32 op/s"
-        oderiv = ("337 FP32 operations per tet of the limb element (674 per pair) x cells / launch duration, against the "
-                  "nominal FP32 issue rate 152 SMs x 128 lanes x 1 op/clk x 2.07 GHz = 40.3 T op/s (no measured FP32 "
-                  "peak exists)")
+        kname = ("k_stencil2<double, APPLY> (P2 operator of one coefficient by rows: eight integer stencils on a "
+                 "tile's values, staged once in shared memory as pairs of 30-bit integers; exact 64-bit sums, one "
+                 "rounding per row)")
+        ops, opeak, ounit = OPS_PER_DOF_P2_ROWS * n, FP32_PEAK_TOPS, "T op/s"
+        oderiv = ("177 instructions per dof (ncu: 11.9 M warp instructions for 2.15 M dofs) / launch duration, against "
+                  "the nominal issue rate 152 SMs x 128 lanes x 1 op/clk x 2.07 GHz = 40.3 T op/s")
     else:
         kname = "k_apply<2,double> (native FP64 operator)"
         ops, opeak, ounit = FLOPS_PER_CELL_P2_F64 * C, FP64_PEAK_TFLOPS, "TFLOP/s"
@@ -775,11 +768,11 @@ def run_ours(args, rank, world, local_rank, oracle=None):
         "metric": "Poisson GMG-CG solve DoF/s at 1e-8 residual",
         "value": value, "unit": "DoF/s", "n_gpus": world, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": t_ms / args.steps, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": "f64 (operator on the FP32 pipes, ~47-bit)" if F64_MODE == fe.FE_F64_DOUBLE_FLOAT else "f64",
+        "dtype": "f64 (operator in exact 60-bit integer sums)" if F64_MODE == fe.FE_F64_DOUBLE_FLOAT else "f64",
         "data": "synthetic (manufactured sin-product right-hand side, kappa = 1)",
         "config": dict(WORKLOAD, parallelism=f"replicas{world}",
-                       f64_operator="P2 element as exact fixed-point limbs of float-pair products on the FP32 "
-                                    "pipes (~47-bit); FP64 vectors, reductions, transfers, smoother updates, coarse "
+                       f64_operator="P2 rows as exact sums of 60-bit integers on the integer pipes, one FP64 "
+                                    "rounding per row; FP64 vectors, reductions, transfers, smoother updates, coarse "
                                     "Cholesky"
                        if F64_MODE == 1 else "native FP64"),
         "iterations": stats[-1].iterations, "rel_residual": stats[-1].rel_residual,
@@ -791,11 +784,10 @@ def run_ours(args, rank, world, local_rank, oracle=None):
                      "frac": achieved_gbs / peak_hbm, "frac_hbm": achieved_gbs / peak_hbm,
                      "traffic": TRAFFIC.get(F64_MODE), "apply_ms": apply_ms,
                      "algorithmic_bytes_per_launch": byt, "bytes_per_dof": BYTES_PER_DOF_P2["f64"],
-                     "bytes_model": "x read 8 + y write 8 + tet->dof map 30 + vertex coordinates 3 B per dof (P2, "
-                                    "kappa = 1)",
+                     "bytes_model": "x read 8 + y write 8 B per dof (P2, kappa = 1, rows: no map, no geometry)",
                      "peak_source": f"{hsrc} copy bandwidth (MEASURED_PEAKS.json hbm_gbs)" if hsrc == "measured"
                      else "fallback 6.8 TB/s",
-                     "limiter": "instruction issue and gather latency, not DRAM (ncu: issue 65%, FP64 pipe 48%)",
+                     "limiter": "latency of staging and of the FP64 pipe at 15 to 24 warps per SM, not DRAM (ncu: DRAM 7%)",
                      "alu_issue_view_nominal": {"achieved": ops / (apply_ms * 1e-3) / 1e12, "peak": opeak,
                                                 "unit": ounit, "frac": ops / (apply_ms * 1e-3) / 1e12 / opeak,
                                                 "derivation": oderiv},

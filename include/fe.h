@@ -81,7 +81,9 @@ extern "C" {
 #define FE_F64_DOUBLE_FLOAT 1       /* float-pair (hi + lo, ~48-bit) arithmetic on the FP32 pipes, FP64 in and
                                        out, with the faster layout per degree (P1: per cube, P2: per tet); on
                                        Kuhn tets (G = c M) the P2 element is c times one integer matrix, applied
-                                       to exact fixed-point FP32 limbs of the float-pair products c x */
+                                       to exact fixed-point FP32 limbs of the float-pair products c x; P1 on
+                                       such tets by FP64 rows, P2 with one coefficient by integer stencils and
+                                       P3 by its integer element matrix, in exact 60-bit integer sums */
 #define FE_F64_DOUBLE_FLOAT_TET 2   /* the same arithmetic, one thread per tet (persistent, prefetching) */
 #define FE_F64_DOUBLE_FLOAT_CUBE 3  /* the same arithmetic, one thread per cube (27/8 dofs split and scattered once) */
 #define FE_F64_DOUBLE_FLOAT_PAIR 4  /* P2: the same arithmetic, two tets per thread in packed FP32x2 instructions */
@@ -216,9 +218,13 @@ int fe_set_coefficient(fe_hierarchy* h, const double* kappa_cells, void* stream)
 /* y = A_l x on `level`, matrix-free: for every tet K, y_K += kappa_K
  * int_K grad(u) . grad(v) applied to the gathered dofs x_K, scatter-added
  * into y; boundary rows give y_i = x_i and boundary entries of x are treated
- * as 0 in interior rows.  dtype FE_F64: x, y double (P2 in the default FP64
- * mode: x is first split into the float pairs that the solver's operator
- * gathers, held by the hierarchy, then applied by that operator).  FE_F32: float.
+ * as 0 in interior rows.  dtype FE_F64: x, y double.  FE_F32: float.  In FP32 and
+ * in the default FP64 mode, levels whose Kuhn tets all have G = c M apply P1 by
+ * vertex rows (edge weights of the six axis neighbours) and P2 with one
+ * coefficient by eight integer stencils (FP64: exact integer sums of a tile's
+ * values), with the same result up to rounding; P2 with a varying coefficient
+ * splits x first into the float pairs that the solver's operator gathers, held
+ * by the hierarchy.
  * FE_BF16: float vectors, each dof entering as two bf16 terms (16 significant
  * bits) contracted on the tensor cores with FP32 accumulation: per tile of 128
  * cells one GEMM against the reference stiffness tables (one combined table
@@ -300,7 +306,8 @@ int fe_coarse_info(const fe_hierarchy* h, long long* n_interior, int* bandwidth,
  * x += d to that dof, so no separate vector kernel streams y, x and d again.
  * On GB300 the countdown atomics (one per scattered value, with the result
  * returned) cost about three times the operator itself, so the default is the
- * operator kernel followed by one vector kernel.  The fused forms exist for
+ * operator kernel followed by one vector kernel (and, where the operator runs by
+ * rows, one launch from one vector to another without countdowns).  The fused forms exist for
  * the FP32 operator and the float-pair FP64 operators; native-FP64 and bf16
  * smoothing always use two kernels.  Results agree up to the rounding order
  * of the atomic sums. */

@@ -3,8 +3,8 @@
 // reductions.
 //
 // Every reduction runs on a fixed grid (ReduceCtx::grid blocks): each block
-// reduces its grid-stride slice with warp shuffles, writes one partial, and
-// the last block to arrive (atomic ticket) sums the partials in index order
+// reduces its grid-stride slice through shared memory, writes one partial, and
+// the last block to arrive (atomic ticket) sums the partials in a fixed order
 // and derives the CG scalars (alpha, beta, ...) in device memory, so the
 // recurrences never wait for the host.  Sums are accumulated in FP64 for
 // every vector type.

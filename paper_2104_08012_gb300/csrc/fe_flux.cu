@@ -302,7 +302,8 @@ __host__ __device__ constexpr bool stencil_uses(int ox, int oy, int oz) {
     if (stencil_coef(code, ox, oy, oz) != 0) return true;
   return false;
 }
-static_assert(stencil_coef(0, 0, 0, 0) == 54 && stencil_coef(3, 1, 1, 0) == 48 && stencil_coef(1, 1, 0, 0) == 56 && stencil_coef(7, 1, 1, 1) == 48 &&
+static_assert(stencil_coef(0, 0, 0, 0) == 54 && stencil_coef(3, 1, 1, 0) == 48 &&
+                  stencil_coef(1, 1, 0, 0) == 56 && stencil_coef(7, 1, 1, 1) == 48 &&
                   stencil_coef(0, 2, 1, 1) == 1 && stencil_coef(3, 0, 0, -1) == 4,
               "P2 Kuhn stencils");
 

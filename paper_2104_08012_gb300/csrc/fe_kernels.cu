@@ -1497,7 +1497,7 @@ void launch_restrict(const fe_hierarchy* h, int lf, const T* bf, const T* yf, T*
   const Level& F = h->L[lf];
   const Level& Cc = h->L[lf - 1];
   const TransferTables& t = h->tt;
-  // (the entry point restricts one vector too)
+  // FP64 stages one vector only: the residual that the operator left, or a caller's vector (fe_restrict.cu)
   if (h->deg == 2 && zero_bd && Cc.N >= kRestrictTiledFrom && (sizeof(T) == 4 || !yf)) {
     launch_restrict_p2<T>(F, Cc, bf, yf, rc, s);
     return;

@@ -220,9 +220,10 @@ __global__ void __launch_bounds__(kBlock) k_patch_apply_df(int P, int Pp, int Pp
 // and row, 32 rows at a time, which one exchange of halves over the warp turns into
 // the row sums of 32 lanes); column 64 is read by rows.  The first form gave every
 // lane whole rows: two loads per entry, half of them scattered, 65 steps for row 64
-// on one lane, and one dependent chain of 195 float-pair additions per warp: 53 us
-// at 8^3 and 16^3, where there are too few patches to hide it, and 115 us at 32^3,
-// whose 617 MB take 91 us at the copy bandwidth.
+// on one lane, and one dependent chain of 195 float-pair additions per warp: 18, 46
+// and 281 us at 8^3, 16^3 and 32^3, this form 9, 31 and 201.  It is bound by issue:
+// 4.4 k instructions per patch, 136 us at 32^3 (whose 617 MB take 91 us at the copy
+// bandwidth).
 constexpr int NS3 = 65, NP3 = NS3 * (NS3 + 1) / 2, kWarpsP3 = 4;
 constexpr int kRing = 8;  // rows of the triangle in flight per warp (cp.async; 6 blocks per SM measured best with 8)
 
