@@ -1558,6 +1558,7 @@ int fe_set_geometry_form(fe_hierarchy* h, int form) {
     launch_flux_setup(h->L[l], nullptr);
   }
   invalidate_graphs(h);
+  CUDA_CHECK(cudaStreamSynchronize(nullptr));  // streams created as non-blocking do not wait for the default stream
   API_END
 }
 
