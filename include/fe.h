@@ -224,7 +224,8 @@ int fe_set_coefficient(fe_hierarchy* h, const double* kappa_cells, void* stream)
  * coefficient by eight integer stencils (FP64: exact integer sums of a tile's
  * values), with the same result up to rounding; P2 with a varying coefficient
  * splits x first into the float pairs that the solver's operator gathers, held
- * by the hierarchy.
+ * by the hierarchy.  Every FP64 row of the stencils is within 1e-14 of its own
+ * sum of |A_ij| |x_j|, whatever the values elsewhere are.
  * FE_BF16: float vectors, each dof entering as two bf16 terms (16 significant
  * bits) contracted on the tensor cores with FP32 accumulation: per tile of 128
  * cells one GEMM against the reference stiffness tables (one combined table

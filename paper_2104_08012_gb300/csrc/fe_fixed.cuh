@@ -9,25 +9,6 @@ namespace fe_fixed {
 
 constexpr int kTop = 59;  // top bit of a value: |x| < 2^60 units
 
-// FP64 values as 64-bit integers of a common scale: with E the largest biased
-// exponent of a tile, |x| is cut into windows of TB + 1 bits below 2^(E - 1022);
-// window `pass` of x is returned with x's sign.  Sums of such integers wrap
-// modulo 2^64 and are exact as long as the final row fits.
-template <int TB>
-__device__ __forceinline__ long long fixed_window(unsigned int hi, unsigned int lo, int E, int pass) {
-  const int e = (int)((hi >> 20) & 0x7FFu);
-  if (e == 0 || e == 0x7FF) return 0;  // zero, subnormal (flushed), or not finite (handled by the caller)
-  const unsigned long long m = ((unsigned long long)((hi & 0xFFFFFu) | 0x100000u) << 32) | lo;
-  const unsigned long long M = m << (TB - 52);
-  const int r = (E - e) - pass * (TB + 1);
-  unsigned long long w;
-  if (r >= 0)
-    w = r < 64 ? M >> r : 0ull;
-  else
-    w = r > -64 ? (M << -r) & ((1ull << (TB + 1)) - 1) : 0ull;
-  return (hi >> 31) ? -(long long)w : (long long)w;
-}
-
 __device__ __forceinline__ double pow2(int e) {  // 2^e, -1022 <= e <= 1023
   return __hiloint2double((e + 1023) << 20, 0);
 }
@@ -51,9 +32,9 @@ struct PairSum {
   }
 };
 
-// x as hi 2^30 + lo of the scale E, both with the sign of x (the first window of
-// fixed_window in 30-bit halves).  A shift beyond 63 (zeros, far smaller values
-// and, with e > E, values that are not finite) gives 0; needs E >= 64.
+// x as hi 2^30 + lo in units of 2^(E - 1023 - kTop), E the largest biased exponent of a tile, both with the sign of x,
+// what lies below a unit cut off.  A shift beyond 63 (zeros, far smaller values and, with e > E, values that are not
+// finite) gives 0; needs E >= 64.
 __device__ __forceinline__ Pair32 fixed_pair(double x, int E) {
   const unsigned int xh = (unsigned int)__double2hiint(x), xl = (unsigned int)__double2loint(x);
   const unsigned int r = min((unsigned int)(E - (int)((xh >> 20) & 0x7FFu)), 63u);

@@ -18,6 +18,7 @@
 // x is read as 0 on and outside the boundary.  An interior row only couples to
 // points of tets that exist, so edges of the domain need no special case.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <type_traits>
 #include <utility>
@@ -176,8 +177,6 @@ __global__ void k_edge_weights(int N, int n, const double* __restrict__ geo22, d
   w32[3 * m + i] = (float)dg;
 }
 
-constexpr int kRange = 15;  // bits by which a cell may lie below its tile's largest value in one pass
-
 // ------------------------------------------- P2, one coefficient: stencils ---
 // With one c on the level the rows of A are eight constant stencils of 19 to 51
 // small integers times 8 c, one per parity
@@ -193,9 +192,17 @@ constexpr int kRange = 15;  // bits by which a cell may lie below its tile's lar
 // row is rounded once, by one int64 -> FP64 conversion and one multiplication.
 // The FP64 pipe (2 operations per clock and SM) would need 23 operations per row,
 // the element-by-element form on the FP32 pipes 453 instructions per dof, this
-// form 180.  What the integers cut off is below 2^-59 of the tile's largest
-// value; the cells that lie more than kRange bits below it are formed again from
-// the windows of the next lower bits, and the parts are added in FP64.
+// form 180.  What the integers cut off a value is below 2^-59 of the tile's scale
+// 2^E.  They form the rows whose |A| |x| is large enough that less than 2^-47 of
+// it is lost (row_kept).  The others, where values of very different size meet, and
+// the rows of tiles whose scale is near the ends of the FP64 range are formed
+// separately, each from a scale of its own: a thread marks them, the block stages the
+// tile once more, and its warps take 32 cells of one stencil in turn.  P2 64^3: 26.8
+// us without such rows (the test costs nothing there, 1 to 2 us of the 45 of a
+// Chebyshev step), 33 with a single value in a vector of zeros, 119 to 127 where
+// all rows of most tiles are such rows (values of 2^-60 .. 1 in every tile,
+// exp(-200 r^2)); 24^3: 10.4, 21 and 37 us.  In FP64 the same rows took 185 us
+// (64^3) and 48 (24^3), in windows of the next lower bits of the whole tile 120 and 74.
 template <typename V>
 struct RowSum;
 template <>
@@ -215,7 +222,14 @@ struct RowSum<double> {
   }
 };
 template <>
-struct RowSum<Pair32> : PairSum {};
+struct RowSum<Pair32> : PairSum {
+  // |hi|, |lo| < 216 * 2^30: the sum as one int64, or in units of 64 where hi is large
+  __device__ __forceinline__ bool fits() const { return (unsigned long long)(hi + (1ll << 32)) < (1ull << 33); }
+  __device__ __forceinline__ double value(bool fits) const {
+    return (double)(fits ? (long long)((unsigned long long)hi << 30) + lo
+                         : (long long)((unsigned long long)hi << 24) + (lo >> 6));
+  }
+};
 
 // The row of the lattice point of parity code CODE in units of 8 c; at(x, y, z):
 // the value at that offset from the vertex of its cell, components in [-2, 2].
@@ -266,6 +280,19 @@ __device__ __forceinline__ RowSum<V> stencil_row(At at) {
     r.add(1, t(1, 1, 2));
   }
   return r;
+}
+
+// f(code) for the eight parity codes as constants
+template <typename F>
+__device__ __forceinline__ void for_codes(F&& f) {
+  f(std::integral_constant<int, 0>{});
+  f(std::integral_constant<int, 1>{});
+  f(std::integral_constant<int, 2>{});
+  f(std::integral_constant<int, 3>{});
+  f(std::integral_constant<int, 4>{});
+  f(std::integral_constant<int, 5>{});
+  f(std::integral_constant<int, 6>{});
+  f(std::integral_constant<int, 7>{});
 }
 
 // The coefficient (in units of 8 c) of the lattice point at offset (ox, oy, oz)
@@ -341,14 +368,48 @@ __device__ __forceinline__ void stencil_rows(RowSum<V> (&r)[8], At at, std::inte
   (point(std::integral_constant<int, I>{}, std::true_type{}), ...);
 }
 
-// any window, any E
-__device__ __noinline__ Pair32 fixed_pair_window(double x, int E, int pass) {
-  const unsigned int xh = (unsigned int)__double2hiint(x), xl = (unsigned int)__double2loint(x);
-  const long long w = fixed_window<kTop>(xh & 0x7FFFFFFFu, xl, E, pass);
-  const int sg = 1 | ((int)xh >> 31);
-  return {sg * (int)(w >> 30), sg * (int)(w & 0x3FFFFFFF)};
+// The same stencils as lists, for the rows with a scale of their own: few as a rule, and eight stencils unrolled a
+// second time would be fetched for each of them (FP64 64^3: 372 us).
+template <int CODE, int I>
+constexpr int kCoef = stencil_coef(CODE, I % 5 - 2, I / 5 % 5 - 2, I / 25 - 2);
+struct StencilList {
+  int n, sum, k[51], point[51];  // points, sum of |k|; coefficients, offsets as (x + 2) + 5 (y + 2) + 25 (z + 2)
+};
+template <int CODE, int... I>
+constexpr StencilList stencil_list(std::integer_sequence<int, I...>) {
+  StencilList L{};
+  auto point = [&L](int k, int i) {
+    if (k == 0) return;
+    L.sum += k < 0 ? -k : k;
+    L.k[L.n] = k;
+    L.point[L.n++] = i;
+  };
+  (point(kCoef<CODE, I>, I), ...);
+  return L;
+}
+template <int CODE>
+constexpr StencilList kList = stencil_list<CODE>(std::make_integer_sequence<int, 125>{});
+
+// Whether less than 2^-47 of a row's |A| |x| is cut off (at most the sum of |k| times 2^-59 of the scale): its own value
+// is at least 2^-kOwnBits of the scale, or the sum of |k| |x| over it and its six axis neighbours is large enough.  The
+// second test keeps the rows beside the corners of a smooth field, 2^-11.4 of the largest value in a tile of 16 x 4 x 4
+// cells at a corner of the domain.
+constexpr int kOwnBits = 10;
+template <int CODE, typename At>
+__device__ __forceinline__ bool row_kept(At at, int own) {
+  constexpr int X = CODE & 1, Y = CODE >> 1 & 1, Z = CODE >> 2, sum = kList<CODE>.sum;
+  constexpr int k = stencil_coef(CODE, X, Y, Z), kx = -stencil_coef(CODE, X - 1, Y, Z),
+                ky = -stencil_coef(CODE, X, Y - 1, Z), kz = -stencil_coef(CODE, X, Y, Z - 1);
+  static_assert(sum <= 216 && sum <= k << (12 - kOwnBits), "own value");
+  static_assert(kx > 0 && ky > 0 && kz > 0, "axis neighbours");
+  auto two = [&](int x, int y, int z) {
+    return (abs(at(X + x, Y + y, Z + z).hi) >> 9) + (abs(at(X - x, Y - y, Z - z).hi) >> 9);
+  };
+  // 2^E: hi = 2^29
+  return k * (own >> 9) + kx * two(1, 0, 0) + ky * two(0, 1, 0) + kz * two(0, 0, 1) >= sum << 8;
 }
 
+constexpr int kListStride = 56;
 template <int TX_, int TY_, int KZ_, int THREADS_, int BLOCKS_>
 struct TileShape {  // BLOCKS: resident blocks per SM that the registers are limited for
   static constexpr int blocks = BLOCKS_;
@@ -356,7 +417,7 @@ struct TileShape {  // BLOCKS: resident blocks per SM that the registers are lim
   static constexpr int W = TX + 2, H = TY + 2, D = KZ + 2, cells = W * H * D, own = TX * TY * KZ;
   template <typename T>
   static constexpr size_t smem() {
-    return (size_t)cells * (8 * sizeof(T) + (sizeof(T) == 8 ? 2 : 0));
+    return (size_t)cells * (8 * sizeof(T) + (sizeof(T) == 8 ? 2 : 0)) + (sizeof(T) == 8 ? own + 4 * 8 * kListStride : 0);
   }
 };
 
@@ -364,26 +425,85 @@ struct Lattice2 {  // the P2 numbering per parity code px + 2 py + 4 pz: first d
   int N, off[8], sy[8], sz[8];
 };
 
+// The lists with the points' places in a staged tile, relative to the cell's: the number of points, then place * 256
+// + (k & 255), the last point again with k = 0 up to whole groups of four.
+struct TileLists {
+  int p[8 * kListStride];
+};
+template <typename S, int... CODE>
+constexpr TileLists tile_lists(std::integer_sequence<int, CODE...>) {
+  TileLists L{};
+  auto list = [&L](int* p, const StencilList& a) {
+    p[0] = (a.n + 3) / 4 * 4;
+    for (int i = 0; i < p[0]; ++i) {
+      const int q = i < a.n ? i : a.n - 1;
+      const int x = a.point[q] % 5 - 2, y = a.point[q] / 5 % 5 - 2, z = a.point[q] / 25 - 2;
+      const int cls = (x & 1) | ((y & 1) << 1) | ((z & 1) << 2);
+      p[4 + i] = (cls * S::cells + (x >> 1) + S::W * ((y >> 1) + S::H * (z >> 1))) * 256 + (i < a.n ? a.k[q] & 255 : 0);
+    }
+  };
+  (list(L.p + CODE * kListStride, kList<CODE>), ...);
+  return L;
+}
+template <typename S>
+__device__ const TileLists d_lists = tile_lists<S>(std::make_integer_sequence<int, 8>{});
+
+// f(k, x) for the points of list p (in shared memory) of the staged cell.
+template <typename F>
+__device__ __forceinline__ void for_list(const int* p, const double* cell, F&& f) {
+  const int4* a4 = reinterpret_cast<const int4*>(p + 4);
+  const int n4 = p[0] / 4;
+#pragma unroll 2
+  for (int q = 0; q < n4; ++q) {
+    const int4 a = a4[q];
+    const double v0 = cell[a.x >> 8], v1 = cell[a.y >> 8], v2 = cell[a.z >> 8], v3 = cell[a.w >> 8];
+    f((int)(signed char)a.x, v0);
+    f((int)(signed char)a.y, v1);
+    f((int)(signed char)a.z, v2);
+    f((int)(signed char)a.w, v3);
+  }
+}
+
+// The row of list p at the staged cell in units of u, from the scale of its own largest value; scale: of the matrix.
+__device__ __forceinline__ double listed_row(const int* p, const double* cell, double scale, double& u) {
+  int er = 0;
+  for_list(p, cell, [&](int, double v) { er = max(er, (__double2hiint(v) >> 20) & 0x7FF); });
+  u = 1.0;
+  if (er == 0 || er == 0x7FF) return er ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;
+  RowSum<Pair32> r;
+  for_list(p, cell, [&](int k, double v) { r.add((__double2hiint(v) >> 20) & 0x7FF ? k : 0, fixed_pair(v, er)); });
+  const bool fits = r.fits();
+  const int ex = er - 1023 - kTop + (fits ? 0 : 6);  // the integers' unit
+  if (er <= 300 || er >= 1900) return r.value(fits) * scale * pow2(ex / 2) * pow2(ex - ex / 2);  // (2^ex out of range)
+  u = __hiloint2double(__double2hiint(scale) + ex * (1 << 20), __double2loint(scale));
+  return r.value(fits);
+}
+
 template <typename T, int EPI, typename S>
 __global__ void __launch_bounds__(S::threads, S::blocks)
-    k_stencil2(Lattice2 G, double scale, Rows<T> R, int nb, const int* __restrict__ bnd) {
+    k_stencil2(const __grid_constant__ Lattice2 G, double scale, const __grid_constant__ Rows<T> R, int nb,
+               const int* __restrict__ bnd) {
   constexpr bool FIX = sizeof(T) == 8;
   using V = typename std::conditional<FIX, Pair32, float>::type;
   static_assert(sizeof(V) == sizeof(T), "staged in place");
+  static_assert(S::own % S::threads == 0 && S::own / S::threads <= 4, "marks of a thread's rows in one word");
   extern __shared__ __align__(16) unsigned char smem[];
   T* raw = reinterpret_cast<T*>(smem);  // [8][cells]
   V* xs = reinterpret_cast<V*>(smem);
   unsigned short* se = reinterpret_cast<unsigned short*>(smem + (size_t)S::cells * 8 * sizeof(T));  // exponents
-  __shared__ int s_max, s_min, s_bad;
+  static_assert(S::cells % 8 == 0, "16-byte aligned lists");
+  int* lists = reinterpret_cast<int*>(se + S::cells);  // [8][kListStride]
+  unsigned char* marks = reinterpret_cast<unsigned char*>(lists + 8 * kListStride);  // [own]
+  __shared__ int s_max, s_bad;
   const int tid = threadIdx.x, N = G.N;
   const int ntx = (N + S::TX - 1) / S::TX, nty = (N + S::TY - 1) / S::TY;
   const int i0 = (blockIdx.x % ntx) * S::TX, j0 = (blockIdx.x / ntx) % nty * S::TY, k0 = blockIdx.x / (ntx * nty) * S::KZ;
-  if constexpr (FIX)
+  if constexpr (FIX) {
     if (tid == 0) {
-      s_max = 1;
-      s_min = 0x7FF;
+      s_max = 0;
       s_bad = 0;
     }
+  }
   // the values of staged cell s: f(code, dof, whether it is interior)
   auto for_points = [&](int s, auto&& f) {
     const int ci = i0 - 1 + s % S::W, cj = j0 - 1 + (s / S::W) % S::H, ck = k0 - 1 + s / (S::W * S::H);
@@ -395,23 +515,21 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
       f(code, G.off[code] + ci + G.sy[code] * cj + G.sz[code] * ck,
         (code & 1 ? xo : xe) && (code & 2 ? yo : ye) && (code & 4 ? zo : ze));
   };
-  for (int s = tid; s < S::cells; s += S::threads)
-    for_points(s, [&](int code, int i, bool in) {
-      cp_async_or_zero<sizeof(T)>(raw + code * S::cells + s, R.x + (in ? i : 0), in);
-    });
-  cp_async_commit();
+  auto stage = [&] {
+    for (int s = tid; s < S::cells; s += S::threads)
+      for_points(s, [&](int code, int i, bool in) {
+        cp_async_or_zero<sizeof(T)>(raw + code * S::cells + s, R.x + (in ? i : 0), in);
+      });
+    cp_async_commit();
+  };
+  stage();
   for (int i = blockIdx.x * S::threads + tid; i < nb; i += gridDim.x * S::threads) {  // Dirichlet rows: identity
     identity_row<EPI>(R, bnd[i]);
   }
   cp_async_wait_all();
   __syncthreads();
-  int E = 0, passes = 1;
+  int E = 0;
   bool bad = false;
-  auto exponent = [&](int c) {  // of own cell c (the rows of a cell all couple to most of its eight points)
-    return (int)se[c % S::TX + 1 + S::W * ((c / S::TX) % S::TY + 1 + S::H * (c / (S::TX * S::TY) + 1))];
-  };
-  // windows that a cell of exponent e takes until what is left is below 2^(kRange - kTop) of its values
-  auto windows = [&](int e) { return E - e > kRange ? 1 + (E - e - kRange + kTop) / (kTop + 1) : 1; };
   if constexpr (FIX) {
     int emax = 0, nf = 0;
     for (int s = tid; s < S::cells; s += S::threads) {
@@ -436,105 +554,73 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
 #pragma unroll
       for (int code = 0; code < 8; ++code) {
         const double v = raw[code * S::cells + s];
-        xs[code * S::cells + s] = E >= 64 ? fixed_pair(v, E) : fixed_pair_window(v, E, 0);
+        xs[code * S::cells + s] = fixed_pair(v, max(E, 64));
       }
-    int emin = 0x7FF;
-    for (int c = tid; c < S::own; c += S::threads) {
-      const int e = exponent(c);
-      if (e > 0) emin = min(emin, e);
-    }
-    emin = __reduce_min_sync(0xffffffffu, emin);
-    if ((tid & 31) == 0) atomicMin(&s_min, emin);
     __syncthreads();
-    emin = s_min;
-    if (emin < 0x7FF) passes = windows(emin);
   }
-  for (int pass = 0; pass < passes; ++pass) {
-    double s1 = scale, s2 = 1.0, s64 = scale;
-    if constexpr (FIX) {
-      if (pass > 0) {  // the window of the next lower bits
-        __syncthreads();
-        for (int s = tid; s < S::cells; s += S::threads)
-          for_points(s, [&](int code, int i, bool in) {
-            xs[code * S::cells + s] = fixed_pair_window(in ? R.x[i] : 0.0, E, pass);
-          });
-        __syncthreads();
-      }
-      // rows are in units of scale 2^ex; applied in two factors where one would leave the FP64 range
-      const int ex = E - 1023 - kTop - pass * (kTop + 1);
-      const int ea = max(-900, min(900, ex));
-      s1 = scale * pow2(ea);
-      s64 = 64.0 * s1;
-      s2 = pow2(max(-1022, ex - ea));
-    }
-    const bool plain = !FIX || (passes == 1 && E > 300 && E < 1900);  // one window, one factor
-    for (int c = tid; c < S::own; c += S::threads) {
-      const int a = c % S::TX, b = (c / S::TX) % S::TY, e = c / (S::TX * S::TY);
-      const int vi = i0 + a, vj = j0 + b, vk = k0 + e;
-      if (vi >= N || vj >= N || vk >= N) continue;
-      int last = 0;  // the cell's last pass
-      if constexpr (FIX)
-        if (passes > 1) {
-          const int e = exponent(c);
-          last = e > 0 ? windows(e) - 1 : 0;
-          if (pass > last) continue;
-        }
-      const V* base = xs + (a + 1 + S::W * (b + 1 + S::H * (e + 1)));
-      auto at = [&](int x, int y, int z) -> V {
-        return base[((x & 1) | ((y & 1) << 1) | ((z & 1) << 2)) * S::cells + (x >> 1) +
-                    S::W * ((y >> 1) + S::H * (z >> 1))];
-      };
-      RowSum<V> rs[8];
-      RowIn<EPI, T> ins[8];  // FP32: every row's vectors in flight before the rows are formed
-      if constexpr (!FIX && EPI != EPI_APPLY) {
+  // rows in units of s1 (FIX: scale 2^(E - 1023 - kTop)), where that and every row lie well inside the FP64 range
+  const bool ranged = !FIX || (E > 300 && E < 1900);
+  const double s1 = FIX && ranged ? scale * pow2(E - 1023 - kTop) : scale, s64 = 64.0 * s1;
+  // |hi| of a row's own value below which it is tested: none in a tile of zeros
+  const int low_own = E == 0 ? 0 : ranged ? 1 << (29 - kOwnBits) : INT_MAX;
+  unsigned int low = 0u;  // this thread's rows that need a scale of their own: bit 8 (its cell) + code
+#pragma unroll 1
+  for (int c = tid, k = 0; c < S::own; c += S::threads, k += 8) {
+    const int a = c % S::TX, b = (c / S::TX) % S::TY, e = c / (S::TX * S::TY);
+    const int vi = i0 + a, vj = j0 + b, vk = k0 + e;
+    if (vi >= N || vj >= N || vk >= N) continue;
+    const V* base = xs + (a + 1 + S::W * (b + 1 + S::H * (e + 1)));
+    auto at = [&](int x, int y, int z) -> V {
+      return base[((x & 1) | ((y & 1) << 1) | ((z & 1) << 2)) * S::cells + (x >> 1) +
+                  S::W * ((y >> 1) + S::H * (z >> 1))];
+    };
+    RowSum<V> rs[8];
+    RowIn<EPI, T> ins[8];  // FP32: every row's vectors in flight before the rows are formed
+    if constexpr (!FIX && EPI != EPI_APPLY) {
 #pragma unroll
-        for (int code = 0; code < 8; ++code)
-          if (((code & 1) || vi > 0) && ((code & 2) || vj > 0) && ((code & 4) || vk > 0))
-            ins[code] = RowIn<EPI, T>(R, G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk);
-      }
-      if constexpr (!FIX) stencil_rows(rs, at, std::make_integer_sequence<int, 125>{});
-      auto row = [&](auto code_, auto plain_) {
-        constexpr int code = decltype(code_)::value;
-        if (!((code & 1) || vi > 0) || !((code & 2) || vj > 0) || !((code & 4) || vk > 0)) return;
-        const int i = G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk;
-        if constexpr (FIX) {
-          const RowIn<EPI, T> in(R, i);
-          const RowSum<V> r = stencil_row<code, V>(at);
-          // |hi|, |lo| < 216 * 2^30: as one int64 directly, or in units of 64 where hi is large
-          const bool small = (unsigned long long)(r.hi + (1ll << 32)) < (1ull << 33);
-          const long long v = small ? (long long)((unsigned long long)r.hi << 30) + r.lo
-                                    : (long long)((unsigned long long)r.hi << 24) + (r.lo >> 6);
-          const double sv = small ? s1 : s64;
-          if constexpr (decltype(plain_)::value) {
-            finish_row<EPI>(R, in, i, (double)v, sv, R.wd[code]);
-          } else {
-            const double y = (double)v * sv * s2 + (pass > 0 ? R.out[i] : 0.0);
-            if (pass < last)
-              R.out[i] = y;
-            else
-              finish_row<EPI>(R, in, i, y, 1.0, R.wd[code]);
-          }
-        } else {
-          finish_row<EPI>(R, ins[code], i, rs[code].s, (float)scale, R.wd[code]);
-        }
-      };
-      auto rows = [&](auto plain_) {
-        row(std::integral_constant<int, 0>{}, plain_);
-        row(std::integral_constant<int, 1>{}, plain_);
-        row(std::integral_constant<int, 2>{}, plain_);
-        row(std::integral_constant<int, 3>{}, plain_);
-        row(std::integral_constant<int, 4>{}, plain_);
-        row(std::integral_constant<int, 5>{}, plain_);
-        row(std::integral_constant<int, 6>{}, plain_);
-        row(std::integral_constant<int, 7>{}, plain_);
-      };
-      if (plain)
-        rows(std::true_type{});
-      else
-        rows(std::false_type{});
+      for (int code = 0; code < 8; ++code)
+        if (((code & 1) || vi > 0) && ((code & 2) || vj > 0) && ((code & 4) || vk > 0))
+          ins[code] = RowIn<EPI, T>(R, G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk);
     }
+    if constexpr (!FIX) stencil_rows(rs, at, std::make_integer_sequence<int, 125>{});
+    auto row = [&](auto code_) {
+      constexpr int code = decltype(code_)::value;
+      if (!((code & 1) || vi > 0) || !((code & 2) || vj > 0) || !((code & 4) || vk > 0)) return;
+      const int i = G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk;
+      if constexpr (FIX) {
+        const int own = abs(at(code & 1, code >> 1 & 1, code >> 2).hi);
+        if (own < low_own && !(ranged && row_kept<code>(at, own))) {
+          low |= 1u << (k + code);
+          return;
+        }
+        const RowIn<EPI, T> in(R, i);
+        const RowSum<V> r = stencil_row<code, V>(at);
+        const bool fits = r.fits();
+        finish_row<EPI>(R, in, i, r.value(fits), fits ? s1 : s64, R.wd[code]);
+      } else {
+        finish_row<EPI>(R, ins[code], i, rs[code].s, (float)scale, R.wd[code]);
+      }
+    };
+    for_codes(row);
   }
   if constexpr (FIX) {
+    if (__syncthreads_or((int)low)) {
+      stage();
+      for (int c = tid; c < S::own; c += S::threads, low >>= 8) marks[c] = (unsigned char)low;
+      for (int q = tid; q < 8 * kListStride; q += S::threads) lists[q] = d_lists<S>.p[q];
+      cp_async_wait_all();
+      __syncthreads();
+      for (int t = tid / 32; t < S::own / 4; t += S::threads / 32) {
+        const int code = t & 7, c = (t >> 3) * 32 + tid % 32;
+        if (!(marks[c] >> code & 1)) continue;
+        const int a = c % S::TX, b = (c / S::TX) % S::TY, e = c / (S::TX * S::TY);
+        const int i = G.off[code] + i0 + a + G.sy[code] * (j0 + b) + G.sz[code] * (k0 + e);
+        const RowIn<EPI, T> in(R, i);
+        double u;
+        const double v = listed_row(lists + code * kListStride, raw + (a + 1 + S::W * (b + 1 + S::H * (e + 1))), scale, u);
+        finish_row<EPI>(R, in, i, v, u, R.wd[code]);
+      }
+    }
     if (bad) {  // rows that couple to a value that is not finite (staged as 0) are NaN
       __syncthreads();
       for (int c = tid; c < S::own; c += S::threads) {
@@ -599,9 +685,9 @@ __global__ void __launch_bounds__(kDirectBlock)
   }
 }
 
-// FP64: 41 KB, five blocks per SM, on levels whose tiles are few, where the whole
+// FP64: 44 KB, five blocks per SM, on levels whose tiles are few, where the whole
 // grid is one or two rounds of blocks (two Chebyshev steps at 32^3 30.8 us against
-// 36.5 with the larger tile, 64^3 83 against 86); above, 71 KB and less of the
+// 36.5 with the larger tile, 64^3 83 against 86); above, 74 KB and less of the
 // values staged twice (128^3: 550 against 576 us).  FP32: rows of 32 cells, so that
 // a warp's shared-memory accesses fall into distinct banks (rows of 16: 58 against
 // 48 us at 128^3).

@@ -1,5 +1,7 @@
 """The operator by rows where a caller's use leaves the ordinary case: a change of the geometry form before a call on a
-stream of its own."""
+stream of its own; values of very different size side by side."""
+import functools
+
 import numpy as np
 import pytest
 
@@ -39,3 +41,122 @@ def test_geometry_form_is_complete_on_return(fe, N):
         h.apply_operator(xd, y, stream=stream)
         stream.synchronize()
         assert np.all(np.abs(y.cpu().numpy() - L.A @ x) <= 1e-14 * np.maximum(abs(L.A) @ np.abs(x), 1e-300))
+
+
+# ------------------------------------------------- P2 rows, value by value
+@functools.lru_cache(None)
+def p2_stencils():
+    """Per parity code of the lattice point: {offset: integer coefficient} of its row in units of 8 c, c = 1 / (120 N),
+    read from the oracle's assembled matrix around the centre of a 4^3 mesh."""
+    L = O.Level(4, 2)
+    X = np.rint(L.space.coords * 8).astype(int)
+    out = {}
+    for code in range(8):
+        p = np.array([4 + (code & 1), 4 + (code >> 1 & 1), 4 + (code >> 2)])
+        i = int(np.nonzero((X == p).all(1))[0][0])
+        row = L.A[i].tocoo()
+        k = row.data * (120 * 4) / 8
+        assert np.abs(k - np.rint(k)).max() < 1e-9
+        out[code] = {tuple(X[j] - p): int(v) for j, v in zip(row.col, np.rint(k)) if v}
+    return out
+
+
+def p2_rows(x, X, N):
+    """A x and |A| |x| of interior rows for kappa = 1 on N^3 cubes, x at the lattice points X: products with the integers
+    exact, sums by TwoSum."""
+    c = torch.zeros((2 * N + 5,) * 3, dtype=torch.float64, device=DEV)
+    X = torch.from_numpy(X).to(DEV)
+    inner = ((X > 0) & (X < 2 * N)).all(1)
+    at = tuple((X + 2).T)
+    c[at] = torch.where(inner, x, torch.zeros_like(x))
+    hi = c.view(torch.int64).bitwise_and(-(1 << 27)).view(torch.float64)  # 26 bits, the rest in c - hi
+    y, a = torch.zeros_like(x), torch.zeros_like(x)
+    for code, st in p2_stencils().items():
+        sel = inner & (X[:, 0] % 2 + 2 * (X[:, 1] % 2) + 4 * (X[:, 2] % 2) == code)
+        P = X[sel] + 2
+        s = e = m = torch.zeros(len(P), dtype=torch.float64, device=DEV)
+        for o, k in st.items():
+            q = tuple((P + torch.tensor(o, device=DEV)).T)
+            m = m + abs(k) * c[q].abs()
+            for t in (k * hi[q], k * (c[q] - hi[q])):
+                z = s + t
+                w = z - s
+                e = e + ((s - (z - w)) + (t - w))
+                s = z
+        y[sel], a[sel] = (s + e) * (8 / (120 * N)), m * (8 / (120 * N))
+    return y, a, inner
+
+
+def contrasts(kind, X, N):
+    """Vectors whose values differ by powers of two from one lattice point to the next."""
+    rng = np.random.default_rng(7)
+    x = np.zeros(len(X))
+    if kind.startswith("pair"):  # one large and one far smaller value in the same tile, zeros around
+        x[(X == [5, 5, 5]).all(1)] = 1.0
+        x[(X == [12, 4, 7]).all(1)] = 0.7 * 2.0 ** -int(kind[4:])
+    elif kind.startswith("step"):  # small values beside a region of large ones
+        x = rng.uniform(-1, 1, len(X))
+        x[X[:, 0] > 9] *= 2.0 ** -int(kind[4:])
+    elif kind == "any":  # every exponent from 2^-60 to 1, a fifth of the values zero
+        x = rng.uniform(0.5, 1, len(X)) * rng.choice([-1.0, 1.0], len(X)) * 2.0 ** -rng.integers(0, 61, len(X))
+        x[::5] = 0.0
+    elif kind == "class":  # only one parity class is of size 1: rows that do not couple to it stand alone
+        x = rng.uniform(-1, 1, len(X)) * 2.0 ** -45
+        x[(X % 2 == [1, 0, 0]).all(1)] *= 2.0 ** 45
+    else:  # far from 1
+        x = rng.uniform(-1, 1, len(X)) * 2.0 ** float(kind)
+    return x
+
+
+KINDS = ["pair20", "pair40", "pair70", "step12", "step13", "step16", "step40", "any", "class", "-900", "900"]
+
+
+# tiles of 16 x 4 x 4 cells with remainders (17, 33) and whole in y and z (20); the larger tile from 97 on
+@pytest.mark.parametrize("N", [17, 20, 33, 97])
+@pytest.mark.parametrize("kind", KINDS)
+def test_p2_rows_keep_their_own_bits(fe, N, kind):
+    """One coefficient, FP64: every row is within 1e-14 of its own |A| |x|, whatever the values around it are: less than
+    2^-47 (7.2e-15) of it is cut off the rows formed from the tile's scale and 216 2^-59 (3.8e-16) off those with a scale
+    of their own; both are then rounded three times (3.4e-16)."""
+    with fe.Hierarchy(N, 0, 2) as h:
+        X = np.rint(h.dof_coordinates() * 2 * N).astype(int)
+        x = dt(contrasts(kind, X, N))
+        y = torch.empty_like(x)
+        h.apply_operator(x, y)
+        ref, scale, inner = p2_rows(x, X, N)
+        assert ((y - ref).abs() <= 1e-14 * scale)[inner].all()
+        assert torch.equal(y[~inner], x[~inner])
+
+
+@pytest.mark.parametrize("kind", ["pair40", "step13", "any", "class"])
+def test_p2_chebyshev_rows_keep_their_own_bits(fe, kind):
+    """The same rows inside a Chebyshev step (two, from one vector to another and back): x + d is within 1e-14 of the sum of
+    the magnitudes it is formed of, applied to the step's own input.  N = 20."""
+    N = 20
+    with fe.Hierarchy(10, 1, 2) as h:
+        X = np.rint(h.dof_coordinates() * 2 * N).astype(int)
+        x = dt(contrasts(kind, X, N))
+        b = x * 0.5
+        lmax = h.lambda_max()
+        lo, hi = 0.1 * lmax, 1.1 * lmax
+        theta, delta = 0.5 * (hi + lo), 0.5 * (hi - lo)
+        sigma = theta / delta
+        diag = torch.empty_like(x)
+        h.diagonal(diag)
+        ref, bound, d, db = x.clone(), torch.zeros_like(x), None, None
+        rho = 1 / sigma
+        for k in range(2):
+            y, a, inner = p2_rows(ref, X, N)
+            _, spread, _ = p2_rows(bound, X, N)  # an error of x reaches the next step through |A|
+            y, a = torch.where(inner, y, ref), torch.where(inner, a, ref.abs())
+            if k == 0:
+                c1, c2 = 0.0, 1 / theta
+                d, db = c2 / diag * (b - y), c2 / diag * (b.abs() + a)
+            else:
+                rn = 1 / (2 * sigma - rho)
+                c1, c2 = rn * rho, 2 * rn / delta
+                d, db = c1 * d + c2 / diag * (b - y), c1 * db + c2 / diag * (b.abs() + a)
+            bound = bound + c2 / diag * spread + c1 * bound + 1e-14 * (ref.abs() + db)
+            ref = ref + d
+        h.smooth(b, x, steps=2)
+        assert ((x - ref).abs() <= bound).all()
