@@ -417,7 +417,7 @@ struct TileShape {  // BLOCKS: resident blocks per SM that the registers are lim
   static constexpr int W = TX + 2, H = TY + 2, D = KZ + 2, cells = W * H * D, own = TX * TY * KZ;
   template <typename T>
   static constexpr size_t smem() {
-    return (size_t)cells * (8 * sizeof(T) + (sizeof(T) == 8 ? 2 : 0)) + (sizeof(T) == 8 ? own + 4 * 8 * kListStride : 0);
+    return (size_t)cells * 8 * sizeof(T) + (sizeof(T) == 8 ? own + 4 * 8 * kListStride : 0);
   }
 };
 
@@ -464,17 +464,30 @@ __device__ __forceinline__ void for_list(const int* p, const double* cell, F&& f
   }
 }
 
-// The row of list p at the staged cell in units of u, from the scale of its own largest value; scale: of the matrix.
-__device__ __forceinline__ double listed_row(const int* p, const double* cell, double scale, double& u) {
+// The largest biased exponent of the values in the row of list p at the staged cell.
+__device__ __forceinline__ int list_exponent(const int* p, const double* cell) {
   int er = 0;
   for_list(p, cell, [&](int, double v) { er = max(er, (__double2hiint(v) >> 20) & 0x7FF); });
-  u = 1.0;
-  if (er == 0 || er == 0x7FF) return er ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;
+  return er;
+}
+// The row in units of u, from the scale er of its own largest value (subnormal values count as 0); scale: of the matrix.
+// With a value that is not finite, the FP64 sum.
+__device__ __forceinline__ double listed_row(const int* p, const double* cell, int er, double scale, double& u) {
+  u = scale;
+  if (er == 0x7FF) {
+    double s = 0.0;
+    for_list(p, cell, [&](int k, double v) { s += k != 0 ? (double)k * v : 0.0; });
+    return s;
+  }
+  if (er == 0) return 0.0;
   RowSum<Pair32> r;
   for_list(p, cell, [&](int k, double v) { r.add((__double2hiint(v) >> 20) & 0x7FF ? k : 0, fixed_pair(v, er)); });
   const bool fits = r.fits();
   const int ex = er - 1023 - kTop + (fits ? 0 : 6);  // the integers' unit
-  if (er <= 300 || er >= 1900) return r.value(fits) * scale * pow2(ex / 2) * pow2(ex - ex / 2);  // (2^ex out of range)
+  if (er <= 300 || er >= 1900) {                     // (2^ex can lie outside the FP64 range)
+    u = 1.0;
+    return r.value(fits) * scale * pow2(ex / 2) * pow2(ex - ex / 2);
+  }
   u = __hiloint2double(__double2hiint(scale) + ex * (1 << 20), __double2loint(scale));
   return r.value(fits);
 }
@@ -490,9 +503,7 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
   extern __shared__ __align__(16) unsigned char smem[];
   T* raw = reinterpret_cast<T*>(smem);  // [8][cells]
   V* xs = reinterpret_cast<V*>(smem);
-  unsigned short* se = reinterpret_cast<unsigned short*>(smem + (size_t)S::cells * 8 * sizeof(T));  // exponents
-  static_assert(S::cells % 8 == 0, "16-byte aligned lists");
-  int* lists = reinterpret_cast<int*>(se + S::cells);  // [8][kListStride]
+  int* lists = reinterpret_cast<int*>(smem + (size_t)S::cells * 8 * sizeof(T));  // [8][kListStride]
   unsigned char* marks = reinterpret_cast<unsigned char*>(lists + 8 * kListStride);  // [own]
   __shared__ int s_max, s_bad;
   const int tid = threadIdx.x, N = G.N;
@@ -537,9 +548,16 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
 #pragma unroll
       for (int code = 0; code < 8; ++code)
         e = max(e, (int)(((unsigned int)__double2hiint(raw[code * S::cells + s]) >> 20) & 0x7FFu));
-      nf |= e == 0x7FF;
-      se[s] = (unsigned short)e;
-      emax = max(emax, e == 0x7FF ? 0 : e);
+      if (e == 0x7FF) {  // values that are not finite are staged as 0
+        nf = 1;
+        e = 0;
+#pragma unroll 1
+        for (int code = 0; code < 8; ++code) {
+          const int ev = (int)(((unsigned int)__double2hiint(raw[code * S::cells + s]) >> 20) & 0x7FFu);
+          if (ev != 0x7FF) e = max(e, ev);
+        }
+      }
+      emax = max(emax, e);
     }
     emax = __reduce_max_sync(0xffffffffu, emax);
     nf = __any_sync(0xffffffffu, nf);
@@ -604,7 +622,8 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
     for_codes(row);
   }
   if constexpr (FIX) {
-    if (__syncthreads_or((int)low)) {
+    // in a tile with values that are not finite also the rows that couple to one
+    if (__syncthreads_or((int)low | (int)bad)) {
       stage();
       for (int c = tid; c < S::own; c += S::threads, low >>= 8) marks[c] = (unsigned char)low;
       for (int q = tid; q < 8 * kListStride; q += S::threads) lists[q] = d_lists<S>.p[q];
@@ -612,30 +631,21 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
       __syncthreads();
       for (int t = tid / 32; t < S::own / 4; t += S::threads / 32) {
         const int code = t & 7, c = (t >> 3) * 32 + tid % 32;
-        if (!(marks[c] >> code & 1)) continue;
-        const int a = c % S::TX, b = (c / S::TX) % S::TY, e = c / (S::TX * S::TY);
-        const int i = G.off[code] + i0 + a + G.sy[code] * (j0 + b) + G.sz[code] * (k0 + e);
-        const RowIn<EPI, T> in(R, i);
-        double u;
-        const double v = listed_row(lists + code * kListStride, raw + (a + 1 + S::W * (b + 1 + S::H * (e + 1))), scale, u);
-        finish_row<EPI>(R, in, i, v, u, R.wd[code]);
-      }
-    }
-    if (bad) {  // rows that couple to a value that is not finite (staged as 0) are NaN
-      __syncthreads();
-      for (int c = tid; c < S::own; c += S::threads) {
         const int a = c % S::TX, b = (c / S::TX) % S::TY, e = c / (S::TX * S::TY);
         const int vi = i0 + a, vj = j0 + b, vk = k0 + e;
-        if (vi >= N || vj >= N || vk >= N) continue;
-        bool hit = false;
-        for (int z = -1; z <= 1; ++z)
-          for (int y = -1; y <= 1; ++y)
-            for (int x = -1; x <= 1; ++x)
-              hit = hit || se[a + 1 + x + S::W * (b + 1 + y + S::H * (e + 1 + z))] == 0x7FF;
-        if (!hit) continue;
-        for (int code = 0; code < 8; ++code)
-          if (((code & 1) || vi > 0) && ((code & 2) || vj > 0) && ((code & 4) || vk > 0))
-            R.out[G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk] = __longlong_as_double(0x7ff8000000000000ll);
+        const bool mine = marks[c] >> code & 1;
+        if (!mine && !(bad && vi < N && vj < N && vk < N && ((code & 1) || vi > 0) && ((code & 2) || vj > 0) &&
+                       ((code & 4) || vk > 0)))
+          continue;
+        const int* list = lists + code * kListStride;
+        const T* cell = raw + (a + 1 + S::W * (b + 1 + S::H * (e + 1)));
+        const int er = list_exponent(list, cell);
+        if (!mine && er != 0x7FF) continue;
+        const int i = G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk;
+        const RowIn<EPI, T> in(R, i);
+        double u;
+        const double v = listed_row(list, cell, er, scale, u);
+        finish_row<EPI>(R, in, i, v, u, R.wd[code]);
       }
     }
   }
@@ -685,9 +695,9 @@ __global__ void __launch_bounds__(kDirectBlock)
   }
 }
 
-// FP64: 44 KB, five blocks per SM, on levels whose tiles are few, where the whole
+// FP64: 43 KB, five blocks per SM, on levels whose tiles are few, where the whole
 // grid is one or two rounds of blocks (two Chebyshev steps at 32^3 30.8 us against
-// 36.5 with the larger tile, 64^3 83 against 86); above, 74 KB and less of the
+// 36.5 with the larger tile, 64^3 83 against 86); above, 71 KB and less of the
 // values staged twice (128^3: 550 against 576 us).  FP32: rows of 32 cells, so that
 // a warp's shared-memory accesses fall into distinct banks (rows of 16: 58 against
 // 48 us at 128^3).

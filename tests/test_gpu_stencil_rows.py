@@ -160,3 +160,37 @@ def test_p2_chebyshev_rows_keep_their_own_bits(fe, kind):
             ref = ref + d
         h.smooth(b, x, steps=2)
         assert ((x - ref).abs() <= bound).all()
+
+
+# the direct kernel (12) and the tiled one, whose tiles stage such values as 0
+@pytest.mark.parametrize("N", [12, 20, 97])
+@pytest.mark.parametrize("bad", ["nan", "inf", "-inf", "both"])
+def test_p2_non_finite_values_reach_their_rows_only(fe, N, bad):
+    """A NaN or infinity in the cell of the vector's largest value makes exactly the rows that couple to it what IEEE
+    arithmetic makes of them (NaN; an infinity of the coefficient's sign; NaN where two of opposite sign meet), and every
+    other row keeps its bits."""
+    with fe.Hierarchy(N, 0, 2) as h:
+        X = np.rint(h.dof_coordinates() * 2 * N).astype(int)
+        x = dt(I.random_vector(len(X), 4))
+        at = lambda p: int(np.nonzero((X == p).all(1))[0][0])
+        p = np.array([9, 8, 8])
+        x[at(p + [1, 1, 0])] = 2.0 ** 13  # (the rows around keep their scale without the value beside it)
+        good, y = torch.empty_like(x), torch.empty_like(x)
+        h.apply_operator(x, good)
+        put = {"both": [(p, np.inf), (p + [2, 0, 0], -np.inf)]}.get(bad, [(p, float(bad if bad != "both" else 0))])
+        want = good.cpu().numpy().copy()
+        index = {tuple(X[i]): i for i in np.nonzero((np.abs(X - p) <= 6).all(1))[0]}
+        add = {}
+        for q, v in put:
+            x[at(q)] = v
+            for o in np.ndindex(5, 5, 5):
+                r = tuple(q - (np.array(o) - 2))  # row r couples to q = r + o
+                if not all(0 < c < 2 * N for c in r):
+                    continue
+                k = p2_stencils()[r[0] % 2 + 2 * (r[1] % 2) + 4 * (r[2] % 2)].get(tuple(np.array(o) - 2), 0)
+                if k:
+                    add[r] = add.get(r, 0.0) + k * v
+        for r, v in add.items():
+            want[index[r]] = v
+        h.apply_operator(x, y)
+        assert np.array_equal(y.cpu().numpy(), want, equal_nan=True)
