@@ -197,11 +197,11 @@ __global__ void k_edge_weights(int N, int n, const double* __restrict__ geo22, d
 // it is lost (row_kept).  The others, where values of very different size meet, and
 // the rows of tiles whose scale is near the ends of the FP64 range are formed
 // separately, each from a scale of its own: a thread marks them, the block stages the
-// tile once more, and its warps take 32 cells of one stencil in turn.  P2 64^3: 26.8
-// us without such rows (the test costs nothing there, 1 to 2 us of the 45 of a
-// Chebyshev step), 33 with a single value in a vector of zeros, 119 to 127 where
-// all rows of most tiles are such rows (values of 2^-60 .. 1 in every tile,
-// exp(-200 r^2)); 24^3: 10.4, 21 and 37 us.  In FP64 the same rows took 185 us
+// tile once more, and its warps take 32 cells of one stencil in turn.  P2 64^3: 26.7
+// us without such rows, as before they were looked for (128^3: 169 against 166, the
+// headline solve 4.19 ms both), 33 with a single value in a vector of zeros, 119 to
+// 132 where most rows of most tiles are such rows (values of 2^-60 .. 1 in every
+// tile, exp(-200 r^2)); 24^3: 10.4, 23 and 39 us.  In FP64 the same rows took 185 us
 // (64^3) and 48 (24^3), in windows of the next lower bits of the whole tile 120 and 74.
 template <typename V>
 struct RowSum;
@@ -425,8 +425,8 @@ struct Lattice2 {  // the P2 numbering per parity code px + 2 py + 4 pz: first d
   int N, off[8], sy[8], sz[8];
 };
 
-// The lists with the points' places in a staged tile, relative to the cell's: the number of points, then place * 256
-// + (k & 255), the last point again with k = 0 up to whole groups of four.
+// The lists with the points' places in a staged tile, relative to the cell's: the number of points, the sum of |k|,
+// then from entry 4 on place * 256 + (k & 255), the last point again with k = 0 up to whole groups of four.
 struct TileLists {
   int p[8 * kListStride];
 };
@@ -435,6 +435,7 @@ constexpr TileLists tile_lists(std::integer_sequence<int, CODE...>) {
   TileLists L{};
   auto list = [&L](int* p, const StencilList& a) {
     p[0] = (a.n + 3) / 4 * 4;
+    p[1] = a.sum;
     for (int i = 0; i < p[0]; ++i) {
       const int q = i < a.n ? i : a.n - 1;
       const int x = a.point[q] % 5 - 2, y = a.point[q] / 5 % 5 - 2, z = a.point[q] / 25 - 2;
@@ -449,14 +450,14 @@ template <typename S>
 __device__ const TileLists d_lists = tile_lists<S>(std::make_integer_sequence<int, 8>{});
 
 // f(k, x) for the points of list p (in shared memory) of the staged cell.
-template <typename F>
-__device__ __forceinline__ void for_list(const int* p, const double* cell, F&& f) {
+template <typename V, typename F>
+__device__ __forceinline__ void for_list(const int* p, const V* cell, F&& f) {
   const int4* a4 = reinterpret_cast<const int4*>(p + 4);
   const int n4 = p[0] / 4;
 #pragma unroll 2
   for (int q = 0; q < n4; ++q) {
     const int4 a = a4[q];
-    const double v0 = cell[a.x >> 8], v1 = cell[a.y >> 8], v2 = cell[a.z >> 8], v3 = cell[a.w >> 8];
+    const V v0 = cell[a.x >> 8], v1 = cell[a.y >> 8], v2 = cell[a.z >> 8], v3 = cell[a.w >> 8];
     f((int)(signed char)a.x, v0);
     f((int)(signed char)a.y, v1);
     f((int)(signed char)a.z, v2);
@@ -499,7 +500,7 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
   constexpr bool FIX = sizeof(T) == 8;
   using V = typename std::conditional<FIX, Pair32, float>::type;
   static_assert(sizeof(V) == sizeof(T), "staged in place");
-  static_assert(S::own % S::threads == 0 && S::own / S::threads <= 4, "marks of a thread's rows in one word");
+  static_assert(S::own % S::threads == 0 && S::own / S::threads <= 4, "a thread's rows in one word");
   extern __shared__ __align__(16) unsigned char smem[];
   T* raw = reinterpret_cast<T*>(smem);  // [8][cells]
   V* xs = reinterpret_cast<V*>(smem);
@@ -601,18 +602,26 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
           ins[code] = RowIn<EPI, T>(R, G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk);
     }
     if constexpr (!FIX) stencil_rows(rs, at, std::make_integer_sequence<int, 125>{});
+    const unsigned int edge = (vi == 0 ? 0x55u : 0u) | (vj == 0 ? 0x33u : 0u) | (vk == 0 ? 0x0Fu : 0u);  // boundary rows
     auto row = [&](auto code_) {
       constexpr int code = decltype(code_)::value;
-      if (!((code & 1) || vi > 0) || !((code & 2) || vj > 0) || !((code & 4) || vk > 0)) return;
+      if (edge >> code & 1) return;
       const int i = G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk;
       if constexpr (FIX) {
-        const int own = abs(at(code & 1, code >> 1 & 1, code >> 2).hi);
-        if (own < low_own && !(ranged && row_kept<code>(at, own))) {
+        auto left = [&] {
+          const int own = abs(at(code & 1, code >> 1 & 1, code >> 2).hi);
+          if (own >= low_own || (ranged && row_kept<code>(at, own))) return false;
           low |= 1u << (k + code);
-          return;
-        }
+          return true;
+        };
+        // a residual's row is tested first, the others once formed (64^3: 36.4 against 39.4 us; two Chebyshev steps 81.4
+        // against 84.4, an application 29.9 against 30.4)
+        if constexpr (EPI == EPI_RESIDUAL)
+          if (left()) return;
         const RowIn<EPI, T> in(R, i);
         const RowSum<V> r = stencil_row<code, V>(at);
+        if constexpr (EPI != EPI_RESIDUAL)
+          if (left()) return;
         const bool fits = r.fits();
         finish_row<EPI>(R, in, i, r.value(fits), fits ? s1 : s64, R.wd[code]);
       } else {
@@ -622,30 +631,68 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
     for_codes(row);
   }
   if constexpr (FIX) {
-    // in a tile with values that are not finite also the rows that couple to one
-    if (__syncthreads_or((int)low | (int)bad)) {
-      stage();
+    // The warps take 32 cells' rows of one stencil in turn: f(turn, code, cell, whether the row is marked).
+    auto for_rows = [&](auto&& f) {
+#pragma unroll 1
+      for (int t = tid / 32, turn = 0; t < S::own / 4; t += S::threads / 32, ++turn) {
+        const int code = t & 7, c = (t >> 3) * 32 + tid % 32;
+        f(turn, code, c, (marks[c] >> code & 1) != 0);
+      }
+    };
+    auto place = [&](int c) { return c % S::TX + 1 + S::W * ((c / S::TX) % S::TY + 1 + S::H * (c / (S::TX * S::TY) + 1)); };
+    auto put = [&](int code, int c, double v, double u) {
+      const int i = G.off[code] + i0 + c % S::TX + G.sy[code] * (j0 + (c / S::TX) % S::TY) +
+                    G.sz[code] * (k0 + c / (S::TX * S::TY));
+      finish_row<EPI>(R, RowIn<EPI, T>(R, i), i, v, u, R.wd[code]);
+    };
+    const int marking = __syncthreads_count(low != 0u);
+    if (marking > 0 || bad) {
       for (int c = tid; c < S::own; c += S::threads, low >>= 8) marks[c] = (unsigned char)low;
       for (int q = tid; q < 8 * kListStride; q += S::threads) lists[q] = d_lists<S>.p[q];
-      cp_async_wait_all();
       __syncthreads();
-      for (int t = tid / 32; t < S::own / 4; t += S::threads / 32) {
-        const int code = t & 7, c = (t >> 3) * 32 + tid % 32;
-        const int a = c % S::TX, b = (c / S::TX) % S::TY, e = c / (S::TX * S::TY);
-        const int vi = i0 + a, vj = j0 + b, vk = k0 + e;
-        const bool mine = marks[c] >> code & 1;
-        if (!mine && !(bad && vi < N && vj < N && vk < N && ((code & 1) || vi > 0) && ((code & 2) || vj > 0) &&
-                       ((code & 4) || vk > 0)))
-          continue;
+      // first, unless they are many, the exact test of what is cut off, on the values staged already: it keeps the rows
+      // where nodal planes of a smooth field meet (64^3: 31 us against 36)
+      const bool test = ranged && marking <= S::threads / 4;
+      unsigned int scaled = 0u, check = 0u;  // this thread's turns left: rows with a scale of their own; all others of a
+                                             // tile with values that are not finite, for the rows that couple to one
+      for_rows([&](int turn, int code, int c, bool marked) {
+        if (!marked) {
+          if (bad) check |= 1u << turn;
+          return;
+        }
         const int* list = lists + code * kListStride;
-        const T* cell = raw + (a + 1 + S::W * (b + 1 + S::H * (e + 1)));
-        const int er = list_exponent(list, cell);
-        if (!mine && er != 0x7FF) continue;
-        const int i = G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk;
-        const RowIn<EPI, T> in(R, i);
-        double u;
-        const double v = listed_row(list, cell, er, scale, u);
-        finish_row<EPI>(R, in, i, v, u, R.wd[code]);
+        RowSum<Pair32> r;
+        int w = 0;
+        if (test)
+          for_list(list, xs + place(c), [&](int k, Pair32 v) {
+            r.add(k, v);
+            w += abs(k) * (abs(v.hi) >> 9);
+          });
+        if (!test || w < list[1] << 8) {
+          scaled |= 1u << turn;
+          return;
+        }
+        if (bad) check |= 1u << turn;
+        const bool fits = r.fits();
+        put(code, c, r.value(fits), fits ? s1 : s64);
+      });
+      if (__syncthreads_or((int)(scaled | check))) {
+        stage();
+        cp_async_wait_all();
+        __syncthreads();
+        for_rows([&](int turn, int code, int c, bool) {
+          if (!((scaled | check) >> turn & 1)) return;
+          const int vi = i0 + c % S::TX, vj = j0 + (c / S::TX) % S::TY, vk = k0 + c / (S::TX * S::TY);
+          if (vi >= N || vj >= N || vk >= N || !((code & 1) || vi > 0) || !((code & 2) || vj > 0) ||
+              !((code & 4) || vk > 0))
+            return;
+          const int* list = lists + code * kListStride;
+          const int er = list_exponent(list, raw + place(c));
+          if (!(scaled >> turn & 1) && er != 0x7FF) return;
+          double u;
+          const double v = listed_row(list, raw + place(c), er, scale, u);
+          put(code, c, v, u);
+        });
       }
     }
   }
