@@ -6,8 +6,8 @@
 // reduces its grid-stride slice through shared memory, writes one partial, and
 // the last block to arrive (atomic ticket) sums the partials in a fixed order
 // and derives the CG scalars (alpha, beta, ...) in device memory, so the
-// recurrences never wait for the host.  Sums are accumulated in FP64 for
-// every vector type.
+// recurrences never wait for the host.  Sums are accumulated in FP64, those of
+// FP32 vectors with at least FP64's precision and range (SliceSum).
 #include "fe_df.cuh"
 #include "fe_internal.cuh"
 
@@ -85,6 +85,8 @@ constexpr int kUnroll = 4;
 // about 70 bits, and converted once per slice: FP64 accumulation takes two
 // conversions and an FMA per product, which bound these kernels by the FP64 pipe
 // (2 per clock and SM; 17 M elements: 99 us, the two vectors' bytes 20 us).
+// Products outside 2^-100 .. 2^100, whose error terms or sums can leave FP32's
+// range, are added in FP64 (a coefficient of 1e35 puts all of r.z there).
 template <typename T>
 struct SliceSum;
 template <>
@@ -96,14 +98,21 @@ struct SliceSum<double> {
 template <>
 struct SliceSum<float> {
   float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
+  double far = 0.0;
   __device__ __forceinline__ void add(float a, float b) {
-    const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
-    const fe_df::DF t = fe_df::two_sum(s0, p), u = fe_df::two_sum(s1, e), v = fe_df::two_sum(u.hi, t.lo);
-    s0 = t.hi;
-    s1 = v.hi;
-    s2 = __fadd_rn(s2, __fadd_rn(u.lo, v.lo));
+    const float p = __fmul_rn(a, b);
+    constexpr unsigned int lo = (127u - 100u) << 23, span = 200u << 23;
+    if ((__float_as_uint(p) & 0x7FFFFFFFu) - lo < span) {
+      const float e = __fmaf_rn(a, b, -p);
+      const fe_df::DF t = fe_df::two_sum(s0, p), u = fe_df::two_sum(s1, e), v = fe_df::two_sum(u.hi, t.lo);
+      s0 = t.hi;
+      s1 = v.hi;
+      s2 = __fadd_rn(s2, __fadd_rn(u.lo, v.lo));
+    } else if (p != 0.0f || (a != 0.0f && b != 0.0f)) {
+      far += (double)a * (double)b;
+    }
   }
-  __device__ __forceinline__ double value() const { return (double)s0 + ((double)s1 + (double)s2); }
+  __device__ __forceinline__ double value() const { return (double)s0 + ((double)s1 + (double)s2) + far; }
 };
 
 // Below this length k_cg_update sums FP32 products in FP64 too: its threads take one or two elements each, a chain of

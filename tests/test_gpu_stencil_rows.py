@@ -1,5 +1,5 @@
 """The operator by rows where a caller's use leaves the ordinary case: a change of the geometry form before a call on a
-stream of its own; values of very different size side by side."""
+stream of its own; values of very different size side by side; coefficients far from 1 in mixed precision."""
 import functools
 
 import numpy as np
@@ -194,3 +194,19 @@ def test_p2_non_finite_values_reach_their_rows_only(fe, N, bad):
             want[index[r]] = v
         h.apply_operator(x, y)
         assert np.array_equal(y.cpu().numpy(), want, equal_nan=True)
+
+
+# vectors below and above 2^19 entries, from where on the update's sums too are formed in floats
+@pytest.mark.parametrize("k,n0,levels", [(1, 4, 2), (2, 4, 2), (2, 11, 2)])
+@pytest.mark.parametrize("e", [-80, 100, 118, 122])
+def test_mixed_solve_scales_with_the_coefficient(fe, k, n0, levels, e):
+    """kappa = 2^e scales the whole solve by powers of two (2^122: entries of r . z down to 2^-170, outside FP32): the
+    iterations of kappa = 1, and its solution to the solve's tolerance (1e-9)."""
+    with fe.Hierarchy(n0, levels, k) as h:
+        f = dt(I.sin_product_rhs(h.dof_coordinates()))
+        u, v = torch.empty_like(f), torch.empty_like(f)
+        one = h.solve(f, u, precision=fe.FE_PREC_MIXED_F32, rtol=1e-10)
+        h.set_coefficient(torch.full((h.n_cells(),), 2.0 ** e, dtype=torch.float64, device=DEV))
+        st = h.solve(f, v, precision=fe.FE_PREC_MIXED_F32, rtol=1e-10)
+        assert (st.iterations, st.outer_iterations) == (one.iterations, one.outer_iterations)
+        assert float((v * 2.0 ** e - u).norm()) <= 1e-9 * float(u.norm())
