@@ -666,19 +666,19 @@ static void vcycle_level(fe_hierarchy* h, int l, int dtype, cudaStream_t s) {
 }
 
 // Enqueue one fine-level V-cycle (reads L.b of the finest level, writes
-// L.x); replays a captured CUDA graph when `use_graph` is set.
-static void run_vcycle(fe_hierarchy* h, int dtype, bool use_graph, cudaStream_t s) {
+// L.x); replays the captured CUDA graph of `cache` unless that is null.
+static void run_vcycle(fe_hierarchy* h, int dtype, GraphCache* cache, cudaStream_t s) {
   auto enqueue = [&](cudaStream_t st) {
     if (dtype == FE_F64)
       vcycle_level<double>(h, h->nlev - 1, dtype, st);
     else
       vcycle_level<float>(h, h->nlev - 1, dtype, st);
   };
-  if (!use_graph) {
+  if (!cache) {
     enqueue(s);
     return;
   }
-  GraphCache& gc = h->vgraph[dtype];
+  GraphCache& gc = *cache;
   if (gc.exec && (gc.steps != g_sp.steps || gc.lo != g_sp.lo || gc.hi != g_sp.hi)) {
     cudaGraphExecDestroy(gc.exec);
     gc.exec = nullptr;
@@ -721,13 +721,14 @@ static void run_vcycle(fe_hierarchy* h, int dtype, bool use_graph, cudaStream_t 
 }
 
 static void invalidate_graphs(fe_hierarchy* h) {
-  for (auto& g : h->vgraph) {
-    g.calls = 0;
-    if (g.exec) {
-      cudaGraphExecDestroy(g.exec);
-      g.exec = nullptr;
+  for (auto* graphs : {&h->vgraph, &h->vcall})
+    for (auto& g : *graphs) {
+      g.calls = 0;
+      if (g.exec) {
+        cudaGraphExecDestroy(g.exec);
+        g.exec = nullptr;
+      }
     }
-  }
   if (h->cgloop.exec) {
     cudaGraphExecDestroy(h->cgloop.exec);
     h->cgloop.exec = nullptr;
@@ -917,7 +918,7 @@ static void build_cg_loop(fe_hierarchy* h) {
   cudaGraph_t body = cp.conditional.phGraph_out[0];
   capture(body, [&] {
     float2* ps = presplit(h, h->nlev - 1) ? h->ps.p : nullptr;
-    run_vcycle(h, FE_F64, false, cs);
+    run_vcycle(h, FE_F64, nullptr, cs);
     launch_cg_beta<double>(R, n, r, z, cs);
     launch_cg_update_p<double>(R, n, p, z, cs, ps);
     apply_enqueue(h, h->nlev - 1, p, q, FE_F64, cs, ps);
@@ -984,7 +985,7 @@ static PcgResult pcg64(fe_hierarchy* h, const double* b, double* x, const fe_sol
     launch_dot<double>(R, n, b, b, S_BB, s);
   }
   if (gmg) {
-    run_vcycle(h, FE_F64, graphs, s);
+    run_vcycle(h, FE_F64, graphs ? &h->vgraph[FE_F64] : nullptr, s);
   } else {
     PhaseScope ps(FE_PHASE_SMOOTH, top, s);
     launch_cheb_step<double>(n, r, nullptr, F.dinv64, q, z, 0.0, 1.0, true, s);  // z = D^-1 r
@@ -1033,7 +1034,7 @@ static PcgResult pcg64(fe_hierarchy* h, const double* b, double* x, const fe_sol
       break;
     }
     if (res.rr <= tol2) break;
-    if (gmg) run_vcycle(h, FE_F64, graphs, s);
+    if (gmg) run_vcycle(h, FE_F64, graphs ? &h->vgraph[FE_F64] : nullptr, s);
     PhaseScope ps(FE_PHASE_BLAS1, top, s);
     if (gmg) launch_cg_beta<double>(R, n, r, z, s);
     launch_cg_update_p<double>(R, n, p, z, s, psplit);
@@ -1055,7 +1056,7 @@ static PcgResult pcg_low(fe_hierarchy* h, int dtype, const fe_solver_opts& o, cu
     CUDA_CHECK(cudaMemsetAsync(e, 0, sizeof(float) * n, s));
     launch_dot<float>(R, n, r, r, S_BB, s);
   }
-  run_vcycle(h, dtype, graphs, s);
+  run_vcycle(h, dtype, graphs ? &h->vgraph[dtype] : nullptr, s);
   {
     PhaseScope ps(FE_PHASE_BLAS1, top, s);
     launch_dot<float>(R, n, r, z, S_RZ, s);
@@ -1085,7 +1086,7 @@ static PcgResult pcg_low(fe_hierarchy* h, int dtype, const fe_solver_opts& o, cu
       break;
     }
     if (res.rr <= tol2) break;
-    run_vcycle(h, dtype, graphs, s);
+    run_vcycle(h, dtype, graphs ? &h->vgraph[dtype] : nullptr, s);
     PhaseScope ps(FE_PHASE_BLAS1, top, s);
     launch_cg_beta<float>(R, n, r, z, s);
     launch_cg_update_p<float>(R, n, p, z, s);
@@ -1406,8 +1407,9 @@ void fe_hierarchy_destroy(fe_hierarchy* h) {
   if (!h) return;
   cudaDeviceSynchronize();
   invalidate_graphs(h);
-  for (auto& g : h->vgraph)
-    if (g.stream) cudaStreamDestroy(g.stream);
+  for (auto* graphs : {&h->vgraph, &h->vcall})
+    for (auto& g : *graphs)
+      if (g.stream) cudaStreamDestroy(g.stream);
   for (auto& L : h->L) bf16_forget_level(&L);
   red_free(h->red);
   if (h->lmax_hist) cudaFreeHost(h->lmax_hist);
@@ -1717,14 +1719,17 @@ int fe_vcycle(const fe_hierarchy* hc, const void* b, void* x, int dtype, void* s
   const size_t es = dtype == FE_F64 ? sizeof(double) : sizeof(float);
   void* fb = dtype == FE_F64 ? (void*)F.b64.p : (void*)F.b32.p;
   void* fx = dtype == FE_F64 ? (void*)F.x64.p : (void*)F.x32.p;
-  // From the second call with the same coefficient and modes on, the cycle's launches are replayed from its graph (as in
-  // the solves): P2 40^3 is 45 launches and copies of 5 us, and enqueueing them one by one took longer than running
-  // them.  A stream that the caller is capturing takes the launches themselves.
+  // From the second call with the same coefficient and modes on, the cycle's launches are replayed from a graph of their
+  // own (the solves' is rebuilt when the smoother's parameters change): enqueueing them one by one takes longer than
+  // running them.  P2 40^3, us per cycle for 1, 2, 3 and 20 cycles of one coefficient: 287, 243, 226 and 198, without a
+  // graph 287, 276, 272 and 264; P1 8^3 55, 53, 44 and 30 against 57, 48, 45 and 41, so the capture is paid for by the
+  // third call at the latest.  A stream that the caller is capturing takes the launches themselves.
   cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
   CUDA_CHECK(cudaStreamIsCapturing(s, &capturing));
-  const bool replay = capturing == cudaStreamCaptureStatusNone && h->vgraph[dtype].calls++ > 0;
+  GraphCache& own = h->vcall[dtype];
+  const bool replay = capturing == cudaStreamCaptureStatusNone && own.calls++ > 0;
   CUDA_CHECK(cudaMemcpyAsync(fb, b, es * F.n, cudaMemcpyDefault, s));
-  run_vcycle(h, dtype, replay, s);
+  run_vcycle(h, dtype, replay ? &own : nullptr, s);
   CUDA_CHECK(cudaMemcpyAsync(x, fx, es * F.n, cudaMemcpyDefault, s));
   if (!is_device_ptr(x)) CUDA_CHECK(cudaStreamSynchronize(s));
   if (dtype == FE_BF16) FE_REQUIRE(bf16_take_error(s) == 0, FE_ERR_TIMEOUT, "tensor-core apply gave up a bounded wait");

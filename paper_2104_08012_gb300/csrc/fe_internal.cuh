@@ -413,7 +413,8 @@ struct fe_hierarchy {
   DBuf<float> r32, z32, p32, q32, e32;
   // staging for host pointers
   DBuf<unsigned char> stage[4];
-  GraphCache vgraph[3];  // per dtype
+  GraphCache vgraph[3];  // the solves' V-cycle, per dtype
+  GraphCache vcall[3];   // fe_vcycle's
   GraphCache fmggraph;   // the full-multigrid sequence (steps = V-cycles per level in `lo`)
   // device-side FP64 GMG-PCG loop: a graph whose while node repeats
   // (V-cycle, beta, p update, apply, alpha, x/r update, loop test)

@@ -1,5 +1,6 @@
 """The operator by rows where a caller's use leaves the ordinary case: a change of the geometry form before a call on a
-stream of its own; values of very different size side by side; coefficients far from 1 in mixed precision."""
+stream of its own; values of very different size side by side; coefficients far from 1 in mixed precision; V-cycles
+between solves with other smoothing."""
 import functools
 
 import numpy as np
@@ -210,3 +211,35 @@ def test_mixed_solve_scales_with_the_coefficient(fe, k, n0, levels, e):
         st = h.solve(f, v, precision=fe.FE_PREC_MIXED_F32, rtol=1e-10)
         assert (st.iterations, st.outer_iterations) == (one.iterations, one.outer_iterations)
         assert float((v * 2.0 ** e - u).norm()) <= 1e-9 * float(u.norm())
+
+
+def graphs_built(run):
+    """Graph instantiations during run(), by the CUDA runtime calls that the profiler records."""
+    from torch.profiler import ProfilerActivity, profile
+    with profile(activities=[ProfilerActivity.CPU, ProfilerActivity.CUDA]) as prof:
+        run()
+        torch.cuda.synchronize()
+    return sum(e.count for e in prof.key_averages() if "GraphInstantiate" in e.key)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_vcycles_and_solves_keep_their_graphs(fe, dtype):
+    """A caller that alternates V-cycles (two smoothing steps) with solves of three steps builds each graph once."""
+    code, d = (fe.FE_F64, torch.float64) if dtype == "f64" else (fe.FE_F32, torch.float32)
+    prec = fe.FE_PREC_F64 if dtype == "f64" else fe.FE_PREC_MIXED_F32
+    with fe.Hierarchy(4, 2, 2) as h:
+        f = dt(I.sin_product_rhs(h.dof_coordinates()))
+        u, b = torch.empty_like(f), f.to(d)
+        x = torch.empty_like(b)
+
+        def both():
+            h.solve(f, u, precision=prec, cheb_steps=3)
+            for _ in range(3):
+                h.vcycle(b, x, dtype=code)
+
+        graphs_built(torch.cuda.synchronize)  # (a process's first recording can miss calls)
+        if graphs_built(both) == 0:
+            pytest.skip("the profiler records no runtime calls here")
+        ref = x.clone()
+        assert graphs_built(both) == 0
+        assert (x - ref).abs().max() <= (1e-13 if dtype == "f64" else 1e-5) * ref.abs().max()
