@@ -621,7 +621,8 @@ static void coarse_setup_dense(fe_hierarchy* h, cudaStream_t s) {
   } else {
     launch_coarse_assemble_p3(L0, cs.dof2int, nci, cs.A, -1, s);
   }
-  // L in the storage of the float-pair inverse, which is formed from Linv below (8-byte entries, rows of ld)
+  // L in the storage of the float-pair inverse (8-byte entries, rows of ld), where it has to stay until k_tri_backward has
+  // formed A^-1 in cs.A from it; k_split_rows overwrites it afterwards.  L^T in the upper triangle of cs.A, until then.
   double* Lf = reinterpret_cast<double*>(cs.AinvDF.p);
   CUDA_CHECK(cudaMemsetAsync(cs.flag, 0, sizeof(int), s));
   for (int j = 0; j < nci; j += kPanel) {

@@ -339,7 +339,7 @@ struct CoarseSolver {
   DBuf<double> yb;      // [npad] forward-substitution result
   DBuf<int> ci;        // interior unknown j -> coarse dof
   DBuf<int> dof2int;   // coarse dof -> interior index or -1
-  DBuf<double> A;      // nci*nci dense, then L (lower)
+  DBuf<double> A;      // nci*nci dense, then L^T (upper triangle), then A^-1
   DBuf<double> Linv, LinvT;
   // A^-1 = L^-T L^-1 times 2^(1023 - ainv_exp) (ainv_exp: the largest biased exponent of its diagonal) as float
   // pairs, rows padded to the even length ld: the dense coarse solve of the float-pair modes is one product with
