@@ -1,6 +1,6 @@
 """The operator by rows where a caller's use leaves the ordinary case: a change of the geometry form before a call on a
 stream of its own; values of very different size side by side; coefficients far from 1 in mixed precision; V-cycles
-between solves with other smoothing."""
+between solves with other smoothing; the pair-of-tets operator on the levels of a cycle."""
 import functools
 
 import numpy as np
@@ -213,13 +213,17 @@ def test_mixed_solve_scales_with_the_coefficient(fe, k, n0, levels, e):
         assert float((v * 2.0 ** e - u).norm()) <= 1e-9 * float(u.norm())
 
 
-def graphs_built(run):
-    """Graph instantiations during run(), by the CUDA runtime calls that the profiler records."""
+def recorded(run, name):
+    """How many CUDA runtime calls or kernels whose name holds `name` the profiler records during run()."""
     from torch.profiler import ProfilerActivity, profile
     with profile(activities=[ProfilerActivity.CPU, ProfilerActivity.CUDA]) as prof:
         run()
         torch.cuda.synchronize()
-    return sum(e.count for e in prof.key_averages() if "GraphInstantiate" in e.key)
+    return sum(e.count for e in prof.key_averages() if name in e.key)
+
+
+def graphs_built(run):
+    return recorded(run, "GraphInstantiate")
 
 
 @pytest.mark.parametrize("dtype", ["f64", "f32"])
@@ -243,3 +247,28 @@ def test_vcycles_and_solves_keep_their_graphs(fe, dtype):
         ref = x.clone()
         assert graphs_built(both) == 0
         assert (x - ref).abs().max() <= (1e-13 if dtype == "f64" else 1e-5) * ref.abs().max()
+
+
+def test_vcycle_with_pairs_of_tets_on_every_level(fe):
+    """A coefficient per coarsest cube varies over the mesh and agrees on the two tets of every pair on all levels: the
+    cycle's FP64 operator takes pairs of tets (not one coefficient's stencils, nor single tets) below the finest level
+    too, and equals the oracle's cycle (1e-11 of its norm, as for the other coefficients)."""
+    with fe.Hierarchy(2, 2, 2) as h:
+        cube = np.floor(h.cell_centroids() * 2).astype(int) @ [1, 2, 4]
+        kappa = np.exp(I.random_vector(8, 5))[cube]
+        h.set_coefficient(dt(kappa))
+        oh = O.Hierarchy(2, 2, 2, kappa)
+        oh.lmax = [h.lambda_max(l) for l in range(3)]
+        b = I.random_vector(oh.fine.n, 5)
+        b[oh.fine.space.boundary] = 0
+        bd, x = dt(b), torch.empty(oh.fine.n, dtype=torch.float64, device=DEV)
+        names = []
+        recorded(torch.cuda.synchronize, "")
+        for name in ("KuhnPair", "KuhnTet", "k_stencil2"):
+            h.set_coefficient(dt(kappa))  # (the next cycle's kernels are launched, not replayed)
+            names.append(recorded(lambda: h.vcycle(bd, x), name))
+        ref = oh.vcycle(b)
+        assert np.linalg.norm(x.cpu().numpy() - ref) <= 1e-11 * np.linalg.norm(ref)
+        if not any(names):
+            pytest.skip("the profiler records no kernels here")
+        assert names[0] == 8 and names[1:] == [0, 0]  # 1 + 1 + 2 applications on each of two levels
