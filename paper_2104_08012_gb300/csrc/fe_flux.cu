@@ -65,6 +65,10 @@ struct RowIn {
 __device__ __forceinline__ double fma_t(double a, double b, double c) { return __fma_rn(a, b, c); }
 __device__ __forceinline__ float fma_t(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 
+// By the exponent field (a comparison would go to the FP64 pipe).
+__device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v) & 0x7FF00000) == 0x7FF00000; }
+__device__ __forceinline__ bool not_finite(float v) { return (__float_as_int(v) & 0x7F800000) == 0x7F800000; }
+
 // Row y_i = s v; residual: b - y; Chebyshev: d = c1 d + w (b - y), x += d with w = c2 / A_ii.
 // FP64 operations are scarce (2 per clock and SM), so the scaling of y and the
 // diagonal are folded: 4 of them per row with a previous direction.
@@ -114,7 +118,13 @@ __global__ void __launch_bounds__(kP1Block) k_flux1(int N, int n, const T* __res
   const T yl = Y > 1 ? x[i - n1] : T(0), yr = Y < N - 1 ? x[i + n1] : T(0);
   const T zl = Z > 1 ? x[i - sz] : T(0), zr = Z < N - 1 ? x[i + sz] : T(0);
   if constexpr (CONST) {
-    finish_row<EPI>(R, in, i, fma_t(T(6), xi, -(((xl + xr) + (yl + yr)) + (zl + zr))), c, R.wd[0]);
+    T v = fma_t(T(6), xi, -(((xl + xr) + (yl + yr)) + (zl + zr))), unit = c;
+    if (not_finite(v)) {  // values close to the end of the range
+      const T q = T(0.0625);
+      v = fma_t(6 * q, xi, -(((q * xl + q * xr) + (q * yl + q * yr)) + (q * zl + q * zr)));
+      unit *= T(16);
+    }
+    finish_row<EPI>(R, in, i, v, unit, R.wd[0]);
   } else {
     const T* wx = w;
     const T* wy = w + n;
@@ -207,14 +217,16 @@ template <typename V>
 struct RowSum;
 template <>
 struct RowSum<float> {
+  static constexpr double unit = 8.0;  // sums of |k| / 8 leave FP32's range no sooner than the sums of an element
   float s = 0.0f;
   template <typename... A>
   __device__ __forceinline__ void add(int k, A... v) {
-    s = __fmaf_rn((float)k, (v + ...), s);
+    s = __fmaf_rn((float)k * 0.125f, (v + ...), s);
   }
 };
 template <>
 struct RowSum<double> {
+  static constexpr double unit = 1.0;
   double s = 0.0;
   template <typename... A>
   __device__ __forceinline__ void add(int k, A... v) {
@@ -625,7 +637,7 @@ __global__ void __launch_bounds__(S::threads, S::blocks)
         const bool fits = r.fits();
         finish_row<EPI>(R, in, i, r.value(fits), fits ? s1 : s64, R.wd[code]);
       } else {
-        finish_row<EPI>(R, ins[code], i, rs[code].s, (float)scale, R.wd[code]);
+        finish_row<EPI>(R, ins[code], i, rs[code].s, (float)(scale * RowSum<V>::unit), R.wd[code]);
       }
     };
     for_codes(row);
@@ -727,8 +739,13 @@ __global__ void __launch_bounds__(kDirectBlock)
     };
     const int i = G.off[code] + vi + G.sy[code] * vj + G.sz[code] * vk;
     const RowIn<EPI, T> in(R, i);
-    const RowSum<T> r = stencil_row<code, T>(at);
-    finish_row<EPI>(R, in, i, r.s, (T)scale, R.wd[code]);
+    RowSum<T> r = stencil_row<code, T>(at);
+    T unit = (T)(scale * RowSum<T>::unit);
+    if (not_finite(r.s)) {  // values close to the end of the range
+      r = stencil_row<code, T>([&](int x, int y, int z) { return at(x, y, z) * T(0.00390625); });
+      unit *= T(256);
+    }
+    finish_row<EPI>(R, in, i, r.s, unit, R.wd[code]);
   };
   switch (blockIdx.y) {
     case 0: row(std::integral_constant<int, 0>{}); break;

@@ -272,3 +272,26 @@ def test_vcycle_with_pairs_of_tets_on_every_level(fe):
         if not any(names):
             pytest.skip("the profiler records no kernels here")
         assert names[0] == 8 and names[1:] == [0, 0]  # 1 + 1 + 2 applications on each of two levels
+
+
+# (FP32: up to where the sums of a P2 element stay in its range)
+@pytest.mark.parametrize("k,N,e32", [(1, 3, 126), (1, 40, 126), (2, 3, 123), (2, 12, 123), (2, 20, 123), (3, 3, None)])
+@pytest.mark.parametrize("coef", ["one", "field"])
+def test_rows_up_to_the_end_of_the_range(fe, k, N, e32, coef):
+    """Values up to 2^1022 (FP32 2^126 and 2^123), whose rows lie in the range although 54 times a value does not: 2^1022
+    times the rows of the same values below 1, up to 1e-13 of |A| |x| (the element kernels' tolerance; FP32 1e-5)."""
+    with fe.Hierarchy(N, 0, k) as h:
+        kappa = np.exp(I.random_vector(h.n_cells(), 5)) if coef == "field" else np.ones(h.n_cells())
+        h.set_coefficient(dt(kappa))
+        L = O.Level(N, k, kappa)
+        x = I.random_vector(L.n, 3)
+        x *= min(1.0, 2 / (abs(L.A) @ np.abs(x)).max())  # (rows in range)
+        for d, code, e, tol in ((torch.float64, fe.FE_F64, 1022, 1e-13), (torch.float32, fe.FE_F32, e32, 1e-5)):
+            if e is None:
+                continue
+            xd = dt(x, d)
+            y = torch.empty_like(xd)
+            h.apply_operator(xd * 2.0 ** e, y, dtype=code)
+            v = xd.double().cpu().numpy()
+            ref, scale = L.A @ v, abs(L.A) @ np.abs(v)
+            assert np.all(np.abs(y.double().cpu().numpy() * 2.0 ** -e - ref) <= tol * scale), d
