@@ -34,6 +34,7 @@
 #include <cudaTypedefs.h>
 
 #include <cstring>
+#include <list>
 #include <mutex>
 
 #include "fe_internal.cuh"
@@ -511,7 +512,7 @@ DBuf<uint16_t> g_btile[3][2];
 int g_has_lo[3][2] = {};
 float g_escale[3] = {1.0f, 1.0f, 1.0f};
 DBuf<int> g_err;
-std::vector<TcLevelData> g_levels;
+std::list<TcLevelData> g_levels;  // (references to entries stay valid while other levels come and go)
 
 // cuTensorMapEncodeTiled is fetched from the driver at run time, so the
 // library loads (and reports FE_ERR_CUDA) on hosts without a CUDA driver.
@@ -643,9 +644,5 @@ int bf16_take_error(cudaStream_t s) {
 
 void bf16_forget_level(const Level* L) {
   std::lock_guard<std::mutex> lock(g_tc_mu);
-  for (size_t i = 0; i < g_levels.size(); ++i)
-    if (g_levels[i].L == L) {
-      g_levels.erase(g_levels.begin() + i);
-      return;
-    }
+  g_levels.remove_if([L](const TcLevelData& d) { return d.L == L; });  // both forms: a later level can have its address
 }

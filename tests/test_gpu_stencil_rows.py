@@ -1,6 +1,7 @@
 """The operator by rows where a caller's use leaves the ordinary case: a change of the geometry form before a call on a
 stream of its own; values of very different size side by side; coefficients far from 1 in mixed precision; V-cycles
-between solves with other smoothing; the pair-of-tets operator on the levels of a cycle."""
+between solves with other smoothing; the pair-of-tets operator on the levels of a cycle;
+bf16 applications after hierarchies that used both geometry forms."""
 import functools
 
 import numpy as np
@@ -295,3 +296,21 @@ def test_rows_up_to_the_end_of_the_range(fe, k, N, e32, coef):
             v = xd.double().cpu().numpy()
             ref, scale = L.A @ v, abs(L.A) @ np.abs(v)
             assert np.all(np.abs(y.double().cpu().numpy() * 2.0 ** -e - ref) <= tol * scale), d
+
+
+@pytest.mark.parametrize("k", [1, 2])
+def test_bf16_after_hierarchies_with_both_geometry_forms(fe, k):
+    """A level's tensor maps of both geometry forms go with it: hierarchies that come to lie at its address afterwards,
+    with other sizes and buffers, apply their own operator (two bf16 terms per value, 16 bits: 1e-4 of |A| |x|)."""
+    for N in (6, 9, 7, 6, 10, 8):
+        with fe.Hierarchy(N, 0, k) as h:
+            kappa = np.exp(I.random_vector(h.n_cells(), 5))
+            h.set_coefficient(dt(kappa))
+            L = O.Level(N, k, kappa)
+            x = I.random_vector(L.n, N).astype(np.float32).astype(float)
+            ref, scale = L.A @ x, abs(L.A) @ np.abs(x)
+            xd, y = dt(x, torch.float32), torch.empty(L.n, device=DEV)
+            for form in (fe.FE_GEOMETRY_AUTO, fe.FE_GEOMETRY_PER_CELL):
+                h.set_geometry_form(form)
+                h.apply_operator(xd, y, dtype=fe.FE_BF16)
+                assert np.all(np.abs(y.double().cpu().numpy() - ref) <= 1e-4 * scale)
