@@ -100,6 +100,14 @@ __device__ __forceinline__ void identity_row(const Rows<T>& R, int i) {
 // the FP64 pipe with a coefficient per edge, else by memory.
 constexpr int kP1Block = 256;
 
+// The row from sixteenths of the values (a call, so that its operations are not issued with every row: 112^3 V-cycle 374
+// against 253 us).
+template <typename T>
+__device__ __noinline__ T p1_sixteenth(T xi, T xl, T xr, T yl, T yr, T zl, T zr) {
+  const T q = T(0.0625);
+  return fma_t(6 * q, xi, -(((q * xl + q * xr) + (q * yl + q * yr)) + (q * zl + q * zr)));
+}
+
 template <typename T, bool CONST, int EPI>
 __global__ void __launch_bounds__(kP1Block) k_flux1(int N, int n, const T* __restrict__ w, T c, Rows<T> R) {
   const int i = blockIdx.x * kP1Block + threadIdx.x;
@@ -120,8 +128,7 @@ __global__ void __launch_bounds__(kP1Block) k_flux1(int N, int n, const T* __res
   if constexpr (CONST) {
     T v = fma_t(T(6), xi, -(((xl + xr) + (yl + yr)) + (zl + zr))), unit = c;
     if (not_finite(v)) {  // values close to the end of the range
-      const T q = T(0.0625);
-      v = fma_t(6 * q, xi, -(((q * xl + q * xr) + (q * yl + q * yr)) + (q * zl + q * zr)));
+      v = p1_sixteenth(xi, xl, xr, yl, yr, zl, zr);
       unit *= T(16);
     }
     finish_row<EPI>(R, in, i, v, unit, R.wd[0]);
