@@ -8,6 +8,8 @@
 // and derives the CG scalars (alpha, beta, ...) in device memory, so the
 // recurrences never wait for the host.  Sums are accumulated in FP64, those of
 // FP32 vectors with at least FP64's precision and range (SliceSum).
+#include <type_traits>
+
 #include "fe_df.cuh"
 #include "fe_internal.cuh"
 
@@ -85,35 +87,52 @@ constexpr int kUnroll = 4;
 // about 70 bits, and converted once per slice: FP64 accumulation takes two
 // conversions and an FMA per product, which bound these kernels by the FP64 pipe
 // (2 per clock and SM; 17 M elements: 99 us, the two vectors' bytes 20 us).
-// Products outside 2^-100 .. 2^100, whose error terms or sums can leave FP32's
-// range, are added in FP64 (a coefficient of 1e35 puts all of r.z there).
+// A slice that leaves FP32's range is summed again in FP64 (a coefficient of 1e35
+// takes all of r.z below it): one with a sum that is not in 2^-80 .. 2^120 after
+// its unrolled part (a product's lost parts are below 2^-149), or with a product
+// outside 2^-100 .. 2^100 in the rest.  Testing every product took 2 to 5 us of the
+// 34 at 17 M elements; adding just those products in FP64, inlined, 1 us of every
+// short launch.
 template <typename T>
 struct SliceSum;
 template <>
 struct SliceSum<double> {
   double s = 0.0;
   __device__ __forceinline__ void add(double a, double b) { s += a * b; }
+  __device__ __forceinline__ void add_tested(double a, double b) { add(a, b); }
+  __device__ __forceinline__ void test() {}
   __device__ __forceinline__ double value() const { return s; }
+  __device__ __forceinline__ bool far() const { return false; }
 };
 template <>
 struct SliceSum<float> {
   float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
-  double far = 0.0;
+  bool out = false;
   __device__ __forceinline__ void add(float a, float b) {
-    const float p = __fmul_rn(a, b);
-    constexpr unsigned int lo = (127u - 100u) << 23, span = 200u << 23;
-    if ((__float_as_uint(p) & 0x7FFFFFFFu) - lo < span) {
-      const float e = __fmaf_rn(a, b, -p);
-      const fe_df::DF t = fe_df::two_sum(s0, p), u = fe_df::two_sum(s1, e), v = fe_df::two_sum(u.hi, t.lo);
-      s0 = t.hi;
-      s1 = v.hi;
-      s2 = __fadd_rn(s2, __fadd_rn(u.lo, v.lo));
-    } else if (p != 0.0f || (a != 0.0f && b != 0.0f)) {
-      far += (double)a * (double)b;
-    }
+    const float p = __fmul_rn(a, b), e = __fmaf_rn(a, b, -p);
+    const fe_df::DF t = fe_df::two_sum(s0, p), u = fe_df::two_sum(s1, e), v = fe_df::two_sum(u.hi, t.lo);
+    s0 = t.hi;
+    s1 = v.hi;
+    s2 = __fadd_rn(s2, __fadd_rn(u.lo, v.lo));
   }
-  __device__ __forceinline__ double value() const { return (double)s0 + ((double)s1 + (double)s2) + far; }
+  static __device__ __forceinline__ bool outside(float v, unsigned int below, unsigned int above) {
+    return (__float_as_uint(v) & 0x7FFFFFFFu) - ((127u - below) << 23) >= (below + above) << 23;
+  }
+  __device__ __forceinline__ void add_tested(float a, float b) {
+    add(a, b);
+    out = out || (outside(__fmul_rn(a, b), 100, 100) && a != 0.0f && b != 0.0f);
+  }
+  __device__ __forceinline__ void test() { out = out || outside(s0, 80, 120); }
+  __device__ __forceinline__ double value() const { return (double)s0 + ((double)s1 + (double)s2); }
+  __device__ __forceinline__ bool far() const { return out; }
 };
+// this thread's slice in FP64
+template <typename T>
+__device__ __noinline__ double slice_dot_far(int n, const T* a, const T* b) {
+  double s = 0.0;
+  for (int i = blockIdx.x * kRedBlock + threadIdx.x; i < n; i += gridDim.x * kRedBlock) s += (double)a[i] * (double)b[i];
+  return s;
+}
 
 // Below this length k_cg_update sums FP32 products in FP64 too: its threads take one or two elements each, a chain of
 // latencies that the floats' longer code extends (275 k elements: 10.7 against 12.8 us; the plain dots are the same).
@@ -135,8 +154,9 @@ __device__ __forceinline__ double slice_dot(int n, const T* __restrict__ a, cons
 #pragma unroll
     for (int u = 0; u < kUnroll; ++u) s.add(av[u], bv[u]);
   }
-  for (; i < n; i += G) s.add(a[i], b[i]);
-  return s.value();
+  if (i >= kUnroll * G) s.test();  // (i counts from the thread's first element, below G)
+  for (; i < n; i += G) s.add_tested(a[i], b[i]);
+  return s.far() ? slice_dot_far(n, a, b) : s.value();
 }
 
 template <typename T>
@@ -162,15 +182,21 @@ __global__ void __launch_bounds__(kRedBlock)
                 const T* __restrict__ dinv, T* __restrict__ z, double* partials, unsigned int* counter, double* scal) {
   const T alpha = (T)scal[S_ALPHA];
   Sum rr, rz;
-  auto one = [&](int i, T xi, T pi, T ri0, T qi) {
+  auto one = [&](int i, T xi, T pi, T ri0, T qi, auto tested) {
     x[i] = xi + alpha * pi;
     const T ri = ri0 - alpha * qi;
     r[i] = ri;
-    rr.add(ri, ri);
+    if constexpr (decltype(tested)::value)
+      rr.add_tested(ri, ri);
+    else
+      rr.add(ri, ri);
     if (dinv) {
       const T zi = dinv[i] * ri;
       z[i] = zi;
-      rz.add(ri, zi);
+      if constexpr (decltype(tested)::value)
+        rz.add_tested(ri, zi);
+      else
+        rz.add(ri, zi);
     }
   };
   const int G = gridDim.x * kRedBlock;
@@ -185,15 +211,19 @@ __global__ void __launch_bounds__(kRedBlock)
       qv[u] = q[i + u * G];
     }
 #pragma unroll
-    for (int u = 0; u < kUnroll; ++u) one(i + u * G, xv[u], pv[u], rv[u], qv[u]);
+    for (int u = 0; u < kUnroll; ++u) one(i + u * G, xv[u], pv[u], rv[u], qv[u], std::false_type{});
   }
-  for (; i < n; i += G) one(i, x[i], p[i], r[i], q[i]);
+  if (i >= kUnroll * G) {
+    rr.test();
+    if (dinv) rz.test();
+  }
+  for (; i < n; i += G) one(i, x[i], p[i], r[i], q[i], std::true_type{});
   if (!dinv) {
-    double v[1] = {rr.value()};
+    double v[1] = {rr.far() ? slice_dot_far(n, r, r) : rr.value()};
     if (grid_reduce<1>(v, partials, counter)) scal[S_RR] = v[0];
     return;
   }
-  double v[2] = {rr.value(), rz.value()};
+  double v[2] = {rr.far() ? slice_dot_far(n, r, r) : rr.value(), rz.far() ? slice_dot_far(n, r, z) : rz.value()};
   if (grid_reduce<2>(v, partials, counter)) {
     scal[S_RR] = v[0];
     scal[S_RZNEW] = v[1];
