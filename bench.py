@@ -46,11 +46,11 @@ BYTES_PER_DOF_P2 = {"f64": 16.0, "f32": 8.0, "bf16": 41.0}
 # x read once, y and the halo re-reads stay in L2); None where there is no capture.
 TRAFFIC = {0: None, 1: 17.6e6, 2: None}
 # Native FP64 P2 element application (c, d, S, four G-products, transpose), per tet:
-# 151 flops (an FMA counts 2).  By rows (k_stencil2): 177 instructions per dof
+# 151 flops (an FMA counts 2).  By rows (k_stencil2): 233 instructions per dof
 # counted by ncu (smsp__inst_executed x 32 / dofs), staging and conversion of the
 # tile's halo included.
 FLOPS_PER_CELL_P2_F64 = 151
-OPS_PER_DOF_P2_ROWS = 177
+OPS_PER_DOF_P2_ROWS = 233
 # Operations of one P3 element application through the gradient at the P2 nodes (fe_p3.cuh; an FMA counts 1):
 # 206 additions, 165 multiplications, 284 FMAs, 22 negations (counted by tests/test_p3_element_host.py)
 OPS_PER_CELL_P3 = 677
@@ -757,7 +757,7 @@ def run_ours(args, rank, world, local_rank, oracle=None):
                  "tile's values, staged once in shared memory as pairs of 30-bit integers; exact 64-bit sums, one "
                  "rounding per row)")
         ops, opeak, ounit = OPS_PER_DOF_P2_ROWS * n, FP32_PEAK_TOPS, "T op/s"
-        oderiv = ("177 instructions per dof (ncu: 11.9 M warp instructions for 2.15 M dofs) / launch duration, against "
+        oderiv = ("233 instructions per dof (ncu: 15.6 M warp instructions for 2.15 M dofs) / launch duration, against "
                   "the nominal issue rate 152 SMs x 128 lanes x 1 op/clk x 2.07 GHz = 40.3 T op/s")
     else:
         kname = "k_apply<2,double> (native FP64 operator)"

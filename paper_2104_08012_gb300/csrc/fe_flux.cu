@@ -209,7 +209,7 @@ __global__ void k_edge_weights(int N, int n, const double* __restrict__ geo22, d
 // row is rounded once, by one int64 -> FP64 conversion and one multiplication.
 // The FP64 pipe (2 operations per clock and SM) would need 23 operations per row,
 // the element-by-element form on the FP32 pipes 453 instructions per dof, this
-// form 180.  What the integers cut off a value is below 2^-59 of the tile's scale
+// form 233.  What the integers cut off a value is below 2^-59 of the tile's scale
 // 2^E.  They form the rows whose |A| |x| is large enough that less than 2^-47 of
 // it is lost (row_kept).  The others, where values of very different size meet, and
 // the rows of tiles whose scale is near the ends of the FP64 range are formed
