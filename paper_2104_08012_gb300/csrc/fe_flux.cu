@@ -772,15 +772,18 @@ __global__ void __launch_bounds__(kDirectBlock)
 
 // FP64: 43 KB, five blocks per SM, on levels whose tiles are few, where the whole
 // grid is one or two rounds of blocks (two Chebyshev steps at 32^3 30.8 us against
-// 36.5 with the larger tile, 64^3 83 against 86); above, 71 KB and less of the
-// values staged twice (128^3: 550 against 576 us).  FP32: rows of 32 cells, so that
+// 35.0 with the larger tile, 64^3 80.6 against 84.6, 80^3 166.9 against 167.5); above,
+// 71 KB and less of the values staged twice (96^3 267 against 254, 128^3 568 against
+// 547; applications are within 2% of each other).  FP32: rows of 32 cells, so that
 // a warp's shared-memory accesses fall into distinct banks (rows of 16: 58 against
 // 48 us at 128^3).
 using Tile64Few = TileShape<16, 4, 4, 128, 5>;
 using Tile64Many = TileShape<16, 8, 4, 256, 3>;
 using Tile32 = TileShape<32, 4, 8, 256, 3>;
 constexpr int kTileFewMax = 96;  // cubes per axis
-// The direct kernel: 16^3 8.7 us against 12 us tiled; its operations grow with the level, the tiles' latency does not.
+// The direct kernel: an application at 16^3 6.2 us against 12.3 tiled, two Chebyshev steps 14.4 against 34.8; its
+// operations grow with the level, the tiles' latency does not (24^3 10.6 against 10.3, steps 24.8 against 30.7, with the
+// smaller tile).
 constexpr int kDirectMax = 16;
 
 Lattice2 lattice_of(const Level& L) {
