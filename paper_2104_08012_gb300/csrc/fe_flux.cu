@@ -781,7 +781,7 @@ using Tile64Few = TileShape<16, 4, 4, 128, 5>;
 using Tile64Many = TileShape<16, 8, 4, 256, 3>;
 using Tile32 = TileShape<32, 4, 8, 256, 3>;
 constexpr int kTileFewMax = 96;  // cubes per axis
-// The direct kernel: an application at 16^3 6.2 us against 12.3 tiled, two Chebyshev steps 14.4 against 34.8; its
+// The direct kernel: an application at 16^3 6.2 us against 12.3 with the larger tile, two steps 14.4 against 34.8; its
 // operations grow with the level, the tiles' latency does not (24^3 10.6 against 10.3, steps 24.8 against 30.7, with the
 // smaller tile).
 constexpr int kDirectMax = 16;
